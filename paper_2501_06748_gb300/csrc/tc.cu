@@ -30,6 +30,7 @@
 // k-tiles into each level: at most 12 digit products of <= 257^2 times 16 terms,
 // 1.3e7 < 2^24, still exact in FP32.
 #include <cstdint>
+#include <type_traits>
 #include <cuda_fp16.h>
 
 #include "internal.h"
@@ -42,8 +43,8 @@ namespace sbfwi {
 // set-up: slices of the per-step operators in mma fragment layout
 // ---------------------------------------------------------------------------
 // Operators per element and radial point i: P_i, Q_i, H_i (16 x 16 each after
-// padding); per element R and T.  Each is stored as kSlices fragments of 32 lanes x
-// uint4 with 16 row exponents.
+// padding); per element R and T.  Each is stored as two n-tiles of kSlices B fragments (32
+// lanes x uint2, see the shot-major product in tc_digits.cuh) with 16 row exponents.
 //
 // P_i v_i + Q_i q_{i-1} is formed as ONE product [P_i | Q_i 2^-a][v_i ; q_{i-1} 2^a]
 // with shared row exponents (over both halves) and a shared column exponent, where the
@@ -63,16 +64,16 @@ __global__ void slice_operators_kernel(SliceArgs a) {
   const int64_t nmat = a.E * n * 3;
   if (w >= nmat + a.E * 2) return;
   const double* h;
-  uint4* out;
+  uint2* out;
   int* eout;
   if (w < nmat) {
     h = a.mats + w * nn;
-    out = a.frag + w * kSlices * 32;
+    out = reinterpret_cast<uint2*>(a.frag + w * kSlices * 32);
     eout = a.exps + w * 16;
   } else {
     const int64_t k = w - nmat;
     h = a.rt + k * nn;
-    out = a.frag_rt + k * kSlices * 32;
+    out = reinterpret_cast<uint2*>(a.frag_rt + k * kSlices * 32);
     eout = a.exps_rt + k * 16;
   }
   auto val = [&](int r, int c) { return (r < nb && c < nb) ? h[(int64_t)r * nb + c] : 0.0; };
@@ -110,14 +111,11 @@ __global__ void slice_operators_kernel(SliceArgs a) {
     const int r = g + ((j >> 1) & 1) * 8, c = 2 * t + (j & 1) + (j >> 2) * 8;
     digits(to_fixed(val(r, c), r < 8 ? e_lo : e_hi), dg[j]);
   }
+  // B fragments of the shot-major product: n-tile 0 holds rows 0..7, n-tile 1 rows 8..15
 #pragma unroll
   for (int k = 0; k < kSlices; ++k) {
-    uint4 v;
-    v.x = pack_digits(dg[0][k], dg[1][k]);
-    v.y = pack_digits(dg[2][k], dg[3][k]);
-    v.z = pack_digits(dg[4][k], dg[5][k]);
-    v.w = pack_digits(dg[6][k], dg[7][k]);
-    out[k * 32 + lane] = v;
+    out[k * 32 + lane] = make_uint2(pack_digits(dg[0][k], dg[1][k]), pack_digits(dg[4][k], dg[5][k]));
+    out[(kSlices + k) * 32 + lane] = make_uint2(pack_digits(dg[2][k], dg[3][k]), pack_digits(dg[6][k], dg[7][k]));
   }
 }
 
@@ -134,7 +132,6 @@ constexpr int kStageFrags = 2 * kSlices * 32;     // uint4
 struct WarpSmem {
   uint4 frag[2][kStageFrags];
   int exps[2][32];
-  double xch[kTile * kCols];
   uint64_t bar[2];
 };
 constexpr int kWarpsPerBlock = 4;
@@ -178,105 +175,75 @@ __global__ void __launch_bounds__(128, 4) element_step_tc_kernel(ElemTcArgs a) {
   };
   const int nb = a.nb, n = a.n, B = a.B;
   const int per = nb * B;
-  double* X = W.xch;
+  // this lane's vector entries: shot g, rows 2t, 2t+1, 2t+8, 2t+9
+  const int row[4] = {2 * t, 2 * t + 1, 2 * t + 8, 2 * t + 9};
+  bool ok[4];
+  int off[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    ok[j] = row[j] < nb && g < B;
+    off[j] = row[j] * B + g;
+  }
   const int64_t base = e * (int64_t)n * per;
-  // C-fragment positions of this lane: (row, col) = (g, 2t), (g, 2t+1), (g+8, 2t), (g+8, 2t+1)
-  const int cr[4] = {g, g, g + 8, g + 8};
-  const int cc[4] = {2 * t, 2 * t + 1, 2 * t, 2 * t + 1};
-  bool cok[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) cok[j] = cr[j] < nb && cc[j] < B;
-  // B-fragment positions: (row, col) = (2t, g), (2t+1, g), (2t+8, g), (2t+9, g)
-  const int br[4] = {2 * t, 2 * t + 1, 2 * t + 8, 2 * t + 9};
-  bool bok[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) bok[j] = br[j] < nb && g < B;
+  const float start[4] = {kMagicF, kMagicF, kMagicF, kMagicF};
 
-  // C layout -> B layout through the warp's shared tile
-  auto c_to_b = [&](const double (&c)[4], double (&b)[4]) {
+  // y = A x over kOps operands (operator digits A[o] in shared memory, row exponents rexp, the
+  // operands' digits x[o] at one common column exponent f); kNeg: -y
+  auto apply = [&](auto ops, auto neg, const uint4* A, const XDigits* x, const int* rexp, int f, double (&y)[4]) {
+    constexpr int kOps = decltype(ops)::value;
+    constexpr bool kNeg = decltype(neg)::value;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) X[cr[j] * kCols + cc[j]] = c[j];
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = X[br[j] * kCols + g];
-    __syncwarp();
+    for (int nt = 0; nt < 2; ++nt) {
+      const uint2* b = reinterpret_cast<const uint2*>(A) + nt * kSlices * 32 + lane;
+      LevelSums<kOps> s;
+      s.template add<0>(x[0], b, start);
+      if constexpr (kOps > 1) s.template add<1>(x[1], b + 2 * kSlices * 32, start);
+      const int2 er = *reinterpret_cast<const int2*>(rexp + nt * 8 + 2 * t);
+      y[2 * nt] = scaled_double<kNeg>(s.total(0), er.x + f - 52);
+      y[2 * nt + 1] = scaled_double<kNeg>(s.total(1), er.y + f - 52);
+    }
   };
-  auto col_exp_b = [&](const double (&b)[4]) {
-    int f = -1100;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) f = max(f, exp_bound(b[j]));
-    return column_exponent(f);
-  };
-  // one product y = A x with A's row exponents (rows g, g+8) and x's column exponent,
-  // A's digits in shared memory; returned in C layout
-  auto apply = [&](const uint4* A, const int* rexp, const double (&xbv)[4], double (&y)[4]) {
-    const int f = col_exp_b(xbv);
-    BDigits d;
-    split_b(xbv, f, d);
-    float acc[kLevels][4];
-    zero(acc);
-    product(acc, A + lane, d);
-    const int er0 = rexp[g], er1 = rexp[g + 8];
-    const int fc0 = __shfl_sync(0xffffffffu, f, 4 * cc[0]), fc1 = __shfl_sync(0xffffffffu, f, 4 * cc[1]);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) y[j] = recombine(acc, j, (j < 2 ? er0 : er1) + ((j & 1) ? fc1 : fc0));
+  // one product y = A x, x split here
+  auto apply_one = [&](const uint4* A, const int* rexp, double (&x)[4], double (&y)[4]) {
+    int adj;
+    const int E = column_scale(x, adj);
+    XDigits d[1];
+    split_rows(x, E, d[0]);
+    apply(std::integral_constant<int, 1>{}, std::false_type{}, A, d, rexp, E - 1022 - adj, y);
   };
 
-  // -y = -[P | Q 2^-a][v ; q 2^a] for one radial point (the sweep's q_i directly): P's
-  // and Q's digits in shared memory, joint row exponents in rexp, a in aexp[0]; returned
-  // in C layout
-  auto apply_pq = [&](const uint4* Pf, const uint4* Qf, const int* rexp, const int* aexp, const double (&vbv)[4],
-                      const double (&qbv)[4], double (&y)[4]) {
-    const int bal = aexp[0];
-    int fl = -1100;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) fl = max(fl, max(exp_bound(vbv[j]), exp_bound(qbv[j]) + bal));
-    const int f = column_exponent(fl);
-    BDigits dv, dq;
-    split_b(vbv, f, dv);
-    split_b(qbv, f - bal, dq);
-    float acc[kLevels][4];
-    zero(acc);
-    product(acc, Pf + lane, dv);
-    product(acc, Qf + lane, dq);
-    const int er0 = rexp[g], er1 = rexp[g + 8];
-    const int fc0 = __shfl_sync(0xffffffffu, f, 4 * cc[0]), fc1 = __shfl_sync(0xffffffffu, f, 4 * cc[1]);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) y[j] = recombine<true>(acc, j, (j < 2 ? er0 : er1) + ((j & 1) ? fc1 : fc0));
-  };
-
-  double xb[4];       // the operand of the next product, B layout
+  double x[4];        // the operand of the next product
   if (a.do_down) {
     const int64_t hop = (int64_t)3 * kSlices * 32;       // uint4 between radial points
     const uint4* Hsrc = a.frag + ((e * n + (n - 1)) * 3 + 2) * kSlices * 32;
     const int* Hexp = a.exps + ((e * n + (n - 1)) * 3 + 2) * 16;
     stage_ops(W, (n - 1) & 1, Hsrc, Hexp, 1, lane);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) xb[j] = bok[j] ? a.ub[(int64_t)a.dofs[e * nb + br[j]] * B + g] : 0.0;
+    for (int j = 0; j < 4; ++j) x[j] = ok[j] ? a.ub[(int64_t)a.dofs[e * nb + row[j]] * B + g] : 0.0;
     for (int i = n - 1; i >= 0; --i) {
       const int buf = i & 1;
       if (i > 0) stage_ops(W, buf ^ 1, Hsrc - (int64_t)(n - i) * hop, Hexp - (int64_t)(n - i) * 48, 1, lane);
       // the state of this radial point, loaded ahead of the product
       double zo[4], vo[4], qo[4], fw[4], gr[4];
+      const int64_t oi = base + (int64_t)i * per;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int64_t o = base + (int64_t)i * per + cr[j] * B + cc[j];
-        zo[j] = cok[j] ? a.ud[o] : 0.0;
-        vo[j] = cok[j] ? a.v[o] : 0.0;
-        qo[j] = cok[j] ? a.q[o] : 0.0;
-        fw[j] = (cok[j] && a.grad_int) ? a.fwd_int[o] : 0.0;
-        gr[j] = (cok[j] && a.grad_int) ? a.grad_int[o] : 0.0;
+        zo[j] = ok[j] ? a.ud[oi + off[j]] : 0.0;
+        vo[j] = ok[j] ? a.v[oi + off[j]] : 0.0;
+        qo[j] = ok[j] ? a.q[oi + off[j]] : 0.0;
+        fw[j] = (ok[j] && a.grad_int) ? a.fwd_int[oi + off[j]] : 0.0;
+        gr[j] = (ok[j] && a.grad_int) ? a.grad_int[oi + off[j]] : 0.0;
       }
       wait_stage(buf);
       double hu[4];
-      apply(W.frag[buf], W.exps[buf], xb, hu);
-      double un[4];
+      apply_one(W.frag[buf], W.exps[buf], x, hu);
+      __syncwarp();       // the stage just read may be refilled
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        un[j] = 0.0;
-        if (cok[j]) {
-          const int64_t o = base + (int64_t)i * per + cr[j] * B + cc[j];
-          const double u_new = qo[j] - hu[j];
+        const double u_new = qo[j] - hu[j];
+        x[j] = ok[j] ? u_new : 0.0;
+        if (ok[j]) {
+          const int64_t o = oi + off[j];
           const double uddn = fma(a.a0, u_new, -vo[j]);
           const double udn = fma(a.c2, uddn, zo[j]);
           // the interior displacement is not kept: the predictor v carries it
@@ -296,10 +263,8 @@ __global__ void __launch_bounds__(128, 4) element_step_tc_kernel(ElemTcArgs a) {
           if (a.store_int) a.store_int[o] = udn;
           if (a.grad_int) a.grad_int[o] = fma(fw[j], udn, gr[j]);    // dt applied at the end
           if (a.u_out) a.u_out[o] = u_new;
-          un[j] = u_new;
         }
       }
-      c_to_b(un, xb);     // ends with __syncwarp: the stage just read may be refilled
     }
   }
   if (!a.do_up) return;
@@ -312,45 +277,55 @@ __global__ void __launch_bounds__(128, 4) element_step_tc_kernel(ElemTcArgs a) {
   stage_up(0, 0);
   double vnext[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) vnext[j] = bok[j] ? a.v[base + br[j] * B + g] : 0.0;
-  double qb[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int j = 0; j < 4; ++j) vnext[j] = ok[j] ? a.v[base + off[j]] : 0.0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) x[j] = 0.0;     // q of the previous radial point
   for (int i = 0; i < n; ++i) {
     const int buf = i & 1;
     stage_up(i + 1, buf ^ 1);
-    double vb[4];
+    const int64_t oi = base + (int64_t)i * per;
+    double v[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      vb[j] = vnext[j];
-      vnext[j] = (i + 1 < n && bok[j]) ? a.v[base + (int64_t)(i + 1) * per + br[j] * B + g] : 0.0;
+      v[j] = vnext[j];
+      vnext[j] = (i + 1 < n && ok[j]) ? a.v[oi + per + off[j]] : 0.0;
     }
     wait_stage(buf);
+    // -[P | Q 2^-a][v ; q 2^a] as one product: P's and Q's digits, joint row exponents in P's
+    // exponent slot, a in Q's
+    const int bal = W.exps[buf][16];
+    int adj;
+    const int E = column_scale2(v, x, bal, adj);
+    XDigits d[2];
+    split_rows(v, E, d[0]);
+    split_rows(x, max(E - bal, kMinExp), d[1]);
     double qc[4];
-    apply_pq(W.frag[buf], W.frag[buf] + kSlices * 32, W.exps[buf], W.exps[buf] + 16, vb, qb, qc);
+    apply(std::integral_constant<int, 2>{}, std::true_type{}, W.frag[buf], d, W.exps[buf], E - 1022 - adj, qc);
+    __syncwarp();         // the stage just read may be refilled
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      if (cok[j]) a.q[base + (int64_t)i * per + cr[j] * B + cc[j]] = qc[j];
-      else qc[j] = 0.0;
+      if (ok[j]) a.q[oi + off[j]] = qc[j];
+      x[j] = ok[j] ? qc[j] : 0.0;
     }
-    c_to_b(qc, qb);
   }
   // effective source: f_hat = R q_{n-1} + T v_n, v_n the predictor of the boundary state
   double vb[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     vb[j] = 0.0;
-    if (bok[j]) {
-      const int64_t gi = (int64_t)a.dofs[e * nb + br[j]] * B + g;
+    if (ok[j]) {
+      const int64_t gi = (int64_t)a.dofs[e * nb + row[j]] * B + g;
       vb[j] = fma(a.a0, a.ub[gi], fma(a.a1, a.udb[gi], a.a2 * a.uddb[gi]));
     }
   }
   const int bn = n & 1;
   wait_stage(bn);
   double rq[4], tv[4];
-  apply(W.frag[bn], W.exps[bn], qb, rq);
-  apply(W.frag[bn] + kSlices * 32, W.exps[bn] + 16, vb, tv);
+  apply_one(W.frag[bn], W.exps[bn], x, rq);
+  apply_one(W.frag[bn] + kSlices * 32, W.exps[bn] + 16, vb, tv);
 #pragma unroll
   for (int j = 0; j < 4; ++j)
-    if (cok[j]) a.fhat[(e * nb + cr[j]) * B + cc[j]] = rq[j] + tv[j];
+    if (ok[j]) a.fhat[(e * nb + row[j]) * B + g] = rq[j] + tv[j];
 }
 
 // ---------------------------------------------------------------------------

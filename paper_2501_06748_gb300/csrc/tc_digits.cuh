@@ -165,6 +165,236 @@ __device__ __forceinline__ void zero(float (&acc)[kLevels][4]) {
 }
 
 
+// ---------------------------------------------------------------------------
+// The shot-major product of the element step: y^T = x^T A^T, shots in the rows of the
+// mma.  The 16 rows of m16n8k16 hold 8 shots times two consecutive digits of x (row g:
+// digit 2p of shot g, row g + 8: digit 2p + 1), its 8 columns 8 rows of the operator, so
+// lane (g, t) = (lane / 4, lane % 4) has shot g and vector rows 2t, 2t+1, 2t+8, 2t+9 both
+// as the product's operand and as its result: the sweep's next product starts from the
+// registers of the last one, without an exchange between lanes, and 28 mma cover the 26
+// digit pairs of a 16 x 16 product.
+// What bounds it: the number of instructions around the mma (a warp issues them one
+// dependent chain at a time, 4 warps per scheduler), so both conversions are cut to
+// shifts, byte permutes and 32-bit adds:
+//  - the significand is shifted once, with eight fraction bits kept for the rounding; its
+//    balanced digits are the 9-bit fields of the integer plus a constant (each field less
+//    256), taken for two values at once by byte permutes of 16-bit windows;
+//  - accumulators start at 1.5 * 2^23, so the bits of a sum are the constant plus the sum
+//    (exact while |sum| <= 2^22: at most four mma of 16 products of |digit| <= 256 per
+//    accumulator) and the levels are added as 32-bit integers.
+// The digits, the kept levels and the rounding are those of split_b and recombine.
+// Measured (64 x 64 elements, n_b 16, N_r 32, 8 shots): fused launch 0.555 -> 0.463 ms,
+// 2124 -> 1665 instructions per warp and radial point of both sweeps, DRAM 5.5 TB/s.
+// ---------------------------------------------------------------------------
+constexpr int kPairs = kSlices / 2;
+constexpr float kMagicF = 12582912.0f;            // 1.5 * 2^23: bits 0x4B400000
+constexpr unsigned kMagicBits = 0x4B400000u;
+constexpr int kMinExp = 64;                       // least biased exponent of a column's scale
+constexpr int kScaledExp = 128;                   // columns below 2^(128 - 1023) are scaled up first
+constexpr int kScaleBits = 256;
+
+struct XDigits {          // A fragments of m16n8k16: digit pairs (0,1), (2,3), (4,5) of one 16-row operand
+  uint4 f[kPairs];
+};
+
+// |x| as an ordered key: its high word without the sign (0 for |x| < 2^-1042)
+__device__ __forceinline__ int mag_key(double x) { return __double2hiint(x) & 0x7FFFFFFF; }
+__device__ __forceinline__ int max4(int a, int b, int c, int d) { return max(max(a, b), max(c, d)); }
+
+// 256 * round-half-away(x 2^(53 - f)) in [0.., 8 fraction bits], two's complement, plus the digit
+// constants, for E = f + 1022 (f the column's exponent): bits 8 + 9 j .. 16 + 9 j hold digit 5 - j plus
+// 256 (j < 5), bits 53..62 digit 0 plus 512
+__device__ __forceinline__ uint2 biased_fixed(double x, int E) {
+  const unsigned lo = (unsigned)__double2loint(x);
+  const int hi = __double2hiint(x);
+  const int sgn = hi >> 31;
+  const int ex = (hi >> 20) & 0x7FF;
+  // the significand with its leading bit at position 60, its bits inverted for x < 0; an arithmetic shift
+  // then gives floor(|x| ..) or its complement, and adding half a unit rounds half away from zero
+  const int mh = (int)(__funnelshift_l(lo, (unsigned)hi, 8) & 0x0FFFFFFFu) ^ (sgn ^ 0x10000000);
+  const unsigned ml = (lo << 8) ^ (unsigned)sgn;
+  const int sh = min(max(E - ex, 0), 62);          // 62: the value vanishes (also zeros and subnormals)
+  const long long d = (long long)(((unsigned long long)(unsigned)mh << 32) | ml) >> sh;
+  constexpr unsigned long long kC =
+      256ULL * (1ULL + (1ULL << 9) + (1ULL << 18) + (1ULL << 27) + (1ULL << 36)) + (512ULL << 45);
+  const unsigned long long y = (unsigned long long)d + ((kC << 8) + 128ULL);
+  return make_uint2((unsigned)y, (unsigned)(y >> 32));
+}
+
+__device__ __forceinline__ unsigned unbias(unsigned fields, unsigned bias2) {
+  const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&fields), *reinterpret_cast<const __half2*>(&bias2));
+  return *reinterpret_cast<const unsigned*>(&h);
+}
+
+// the six digits of two values as half2 (first value in the low half)
+__device__ __forceinline__ void digit_pairs(uint2 a, uint2 b, unsigned (&d)[kSlices]) {
+  // 16-bit windows of both values: fields at bit offset 0, 1, 0, 3, 4, 5 of each half
+  const unsigned w5 = __byte_perm(a.x, b.x, 0x6521), w4 = __byte_perm(a.x, b.x, 0x7632);
+  const unsigned w3 = __byte_perm(__funnelshift_r(a.x, a.y, 26), __funnelshift_r(b.x, b.y, 26), 0x5410);
+  const unsigned w2 = __byte_perm(a.y, b.y, 0x5410), w1 = __byte_perm(a.y, b.y, 0x6521), w0 = __byte_perm(a.y, b.y, 0x7632);
+  constexpr unsigned m9 = 0x01FF01FFu, one = 0x64006400u, b9 = 0x65006500u;   // 1024 + field; 1280
+  d[5] = unbias((w5 & m9) | one, b9);
+  d[4] = unbias((w4 & 0x03FE03FEu) | 0x60006000u, 0x62006200u);               // 512 + field; 768
+  d[3] = unbias((w3 & m9) | one, b9);
+  d[2] = unbias(((w2 >> 3) & m9) | one, b9);
+  d[1] = unbias(((w1 >> 4) & m9) | one, b9);
+  d[0] = unbias(((w0 >> 5) & 0x03FF03FFu) | one, 0x66006600u);                // 1024 + field; 1536
+}
+
+__device__ __forceinline__ void split_rows(const double (&x)[4], int E, XDigits& d) {
+  unsigned lo[kSlices], hi[kSlices];
+  digit_pairs(biased_fixed(x[0], E), biased_fixed(x[1], E), lo);
+  digit_pairs(biased_fixed(x[2], E), biased_fixed(x[3], E), hi);
+#pragma unroll
+  for (int p = 0; p < kPairs; ++p) d.f[p] = make_uint4(lo[2 * p], lo[2 * p + 1], hi[2 * p], hi[2 * p + 1]);
+}
+
+// Biased exponent E of the scale of a column (shot) of 16 rows: |x| < 2^(E - 1022) for its entries, shared
+// by the four lanes of the shot.  Columns near the bottom of the range are scaled up by 2^256 first
+// (adj = 256, a whole warp's branch that the path's fields rarely take), so that subnormal entries keep
+// their bits; E is at least kMinExp, which makes the shift of zero entries clear them.
+__device__ __forceinline__ int quad_max(int v) {
+  v = max(v, __shfl_xor_sync(0xffffffffu, v, 1));
+  return max(v, __shfl_xor_sync(0xffffffffu, v, 2));
+}
+constexpr int kZeroExp = -8192;                   // a column of zeros (or below 2^-1042)
+__device__ __forceinline__ int exp_of_key(int key) { return key > 0 ? max(key >> 20, 1) : kZeroExp; }
+__device__ __forceinline__ bool scale_small(int ex) { return ex > kZeroExp / 2 && ex < kScaledExp; }
+
+__device__ __forceinline__ int column_scale(double (&x)[4], int& adj) {
+  auto ex_of = [&] { return exp_of_key(quad_max(max4(mag_key(x[0]), mag_key(x[1]), mag_key(x[2]), mag_key(x[3])))); };
+  int ex = ex_of();
+  adj = 0;
+  if (__any_sync(0xffffffffu, scale_small(ex))) {
+    if (scale_small(ex)) {
+      adj = kScaleBits;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[j] *= 0x1p256;
+    }
+    ex = ex_of();
+  }
+  return max(ex, kMinExp);
+}
+
+// the same for the joint operand [v ; q 2^bal]
+__device__ __forceinline__ int column_scale2(double (&v)[4], double (&q)[4], int bal, int& adj) {
+  auto ex_of = [&] {
+    const int ev = exp_of_key(max4(mag_key(v[0]), mag_key(v[1]), mag_key(v[2]), mag_key(v[3])));
+    const int eq = exp_of_key(max4(mag_key(q[0]), mag_key(q[1]), mag_key(q[2]), mag_key(q[3])));
+    return quad_max(max(ev, eq + bal));
+  };
+  int ex = ex_of();
+  adj = 0;
+  if (__any_sync(0xffffffffu, scale_small(ex))) {
+    if (scale_small(ex)) {
+      adj = kScaleBits;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) { v[j] *= 0x1p256; q[j] *= 0x1p256; }
+    }
+    ex = ex_of();
+  }
+  return max(ex, kMinExp);
+}
+
+// mma of a digit pair fragment and an operator digit, on top of c (kFirst: of the start value)
+template <bool kFirst>
+__device__ __forceinline__ void mma_pair(float (&c)[4], const uint4& a, const uint2& b, const float (&start)[4]) {
+  if (kFirst) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};\n"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "f"(start[0]), "f"(start[1]), "f"(start[2]),
+          "f"(start[3]));
+  } else {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y));
+  }
+}
+
+// Digit products of one accumulator row m = k + 2p (k: operator digit, p: pair of x digits) of one
+// operand, and their number before operator digit k; m holds level m (even digit of the pair) in the
+// results of row g and level m + 1 (odd digit) in those of row g + 8
+__host__ __device__ constexpr bool pair_kept(int k, int p) { return k + 2 * p < kLevels; }
+__host__ __device__ constexpr int pairs_before(int m, int k) {   // of row m, with an operator digit below k
+  int c = 0;
+  for (int p = 0; p < kPairs; ++p) c += (m - 2 * p >= 0 && m - 2 * p < k) ? 1 : 0;
+  return c;
+}
+__host__ __device__ constexpr int pairs_of(int m) { return pairs_before(m, kSlices); }
+// accumulators of row m for `ops` summed operands: four mma each (exact, see above)
+__host__ __device__ constexpr int parts_of(int m, int ops) { return (ops * pairs_of(m) + 3) / 4; }
+
+// The level sums of 8 operator rows (one n-tile), ops operands (16 columns each) summed: add(op, b) gives
+// operand op's digits, b[k] the operator's B fragments.  Every (m, part) is a separate accumulator.
+template <int kOps>
+struct LevelSums {
+  static constexpr int kMaxParts = parts_of(4, kOps);
+  float acc[kLevels][kMaxParts][4];
+
+  template <int kOp>
+  __device__ __forceinline__ void add(const XDigits& x, const uint2* B, const float (&start)[4]) {
+#pragma unroll
+    for (int k = 0; k < kSlices; ++k) {
+      const uint2 b = B[k * 32];
+#pragma unroll
+      for (int p = 0; p < kPairs; ++p) {
+        if (!pair_kept(k, p)) continue;
+        const int m = k + 2 * p;
+        const int pos = kOp * pairs_of(m) + pairs_before(m, k);
+        if (pos % 4 == 0) mma_pair<true>(acc[m][pos / 4], x.f[p], b, start);
+        else mma_pair<false>(acc[m][pos / 4], x.f[p], b, start);
+      }
+    }
+  }
+
+  // column c (0, 1) of this lane's row pair: the sum over the levels as an int64 (see recombine)
+  __device__ __forceinline__ long long total(int c) const {
+    int L[kLevels];
+#pragma unroll
+    for (int l = 0; l < kLevels; ++l) {
+      unsigned v = 0, parts = 0;
+#pragma unroll
+      for (int q = 0; q < parts_of(l, kOps); ++q) { v += __float_as_uint(acc[l][q][c]); ++parts; }
+      if (l > 0) {
+#pragma unroll
+        for (int q = 0; q < parts_of(l - 1, kOps); ++q) { v += __float_as_uint(acc[l - 1][q][c + 2]); ++parts; }
+      }
+      L[l] = (int)(v - parts * kMagicBits);
+    }
+    return combine(L);
+  }
+  static __device__ __forceinline__ long long combine(const int (&L)[kLevels]) {
+    // levels 0, 1 of a product stay below 2^22 (kOps <= 2), so their sum fits 32 bits; the two lowest are
+    // rounded once to the nearest unit (floor(floor(x / 2^9) + 2^8) / 2^9 = floor((x + 2^17) / 2^18))
+    const int low = (L[5] + (L[6] >> 9) + 256) >> 9;
+    const int top = L[0] * 512 + L[1];
+    long long t = (long long)(L[4] + low);
+    t += (long long)L[3] * 512;
+    t += (long long)L[2] * (1 << 18);
+    t += (long long)top * (1 << 27);
+    return t;
+  }
+};
+
+// t * 2^(s) as a binary64, rounded to nearest-even (int_to_double_scaled with fewer operations: the
+// significand is normalised to bit 62 and a carry of the rounding moves into the exponent by itself)
+template <bool kNeg>
+__device__ __forceinline__ double scaled_double(long long t, int s) {
+  const unsigned neg = kNeg ? ~0u : 0u;
+  const unsigned long long mag = (unsigned long long)(t < 0 ? -t : t);
+  const unsigned sign = (((unsigned)(t >> 32)) ^ neg) & 0x80000000u;
+  const int lz = __clzll((long long)mag);
+  unsigned long long m = mag << ((lz - 1) & 63);
+  m += 0x1FFULL + ((m >> 10) & 1ULL);
+  const int be = s - lz + (1023 + 62);            // biased exponent - 1 (t != 0)
+  unsigned long long bits = (m >> 10) + ((unsigned long long)(unsigned)be << 52);
+  if (t == 0) return 0.0;
+  if ((unsigned)be > 2044u) return int_to_double_scaled_slow(kNeg ? -t : t, s);
+  return __longlong_as_double((long long)(bits | ((unsigned long long)sign << 32)));
+}
+
 // Bulk global -> shared copies by the TMA engine (cp.async.bulk), completing on an mbarrier
 // in shared memory: one thread arms the barrier with the byte count and issues the copies;
 // every consumer waits on the barrier's phase.  Addresses and sizes are multiples of 16 bytes.
