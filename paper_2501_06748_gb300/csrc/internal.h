@@ -236,10 +236,11 @@ struct Model {
   const int32_t* solve_bnd = nullptr;
   size_t solve_bytes = 0;
   DevBuf pts_hi, pts_lo; // [n_nodal][dim] dd location of every nodal point
-  // the same operators split into FP16 digits for the tensor-core element kernel
-  DevBuf tc_frag, tc_frag_rt, tc_exps, tc_exps_rt;
+  // the same operators split into FP16 digits for the tensor-core element kernels: one block
+  // (digits, row exponents; tc::OpBlock) per operator, [E][P_0 Q_0 H_0 .. H_{n-1} R T]
+  DevBuf tc_ops;
   bool tc_ready = false;
-  bool tc_one_tile = false;   // tc_frag holds one-tile digits although nb > 16 (mixed element kernels)
+  bool tc_one_tile = false;   // tc_ops holds one-tile digits although nb > 16 (mixed element kernels)
   DevBuf rho_lo;           // [n_nodal] low part of the set-up's double-double density (re-runs of the set-up)
   // exact discrete adjoint (sbfwi_set_gradient_mode(EXACT)): operators the set-up emits on request
   int grad_mode = SBFWI_GRAD_KERNEL;
@@ -342,9 +343,10 @@ bool tc_supported(int nb, int B);   // the tensor-core kernel is the default for
 bool tc_available(int nb, int B);   // a tensor-core kernel exists for these shapes
 int tc_prepare(Model& md, cudaStream_t st);
 int tc_prepare_one_tile(Model& md, cudaStream_t st);   // one-tile digits even when n_b is padded beyond 16
-int tc_element_launch(const Model& md, int B, int down, int up, double* u, double* ud, double* udd, double* v,
-                      const double* ub, const double* udb, const double* uddb, double* q, double* fhat,
-                      double* store_int, const double* fwd_int, double* grad_int, double* u_out, cudaStream_t st,
+// pair: v, z (ud), q and grad_int are in pairs of rows [row / 2][shot][row % 2] per radial point (tc_step.cuh)
+int tc_element_launch(const Model& md, int B, int down, int up, double* ud, double* v, const double* ub,
+                      const double* udb, const double* uddb, double* q, double* fhat, double* store_int,
+                      const double* fwd_int, double* grad_int, double* u_out, bool pair, cudaStream_t st,
                       const int32_t* elems = nullptr, int64_t n_elems = 0, int* status = nullptr);
 
 struct FwdState {

@@ -943,11 +943,18 @@ __global__ void sources_kernel(double* ext, int B, int nsrc, const int64_t* node
 // ---------------------------------------------------------------------------
 // gradient: shots summed, then optionally the transpose of the bilinear map
 // ---------------------------------------------------------------------------
+// Per-shot value of row q, shot s in a [row][shot] array whose first `pair_rows` rows are in pairs
+// [row / 2][shot][row % 2] (the interior state and gradient of the tensor-core element kernels)
+__device__ __forceinline__ int64_t shot_index(int64_t q, int s, int B, int64_t pair_rows) {
+  return q < pair_rows ? ((q >> 1) * B + s) * 2 + (q & 1) : q * B + s;
+}
+
 // g(node) = dt * sum over shots of the accumulated sum_m udot_fwd * lambdadot
-__global__ void sum_shots_kernel(const double* acc, int64_t np, int B, double dt, double* out, int accumulate) {
+__global__ void sum_shots_kernel(const double* acc, int64_t np, int B, int64_t pair_rows, double dt, double* out,
+                                 int accumulate) {
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < np; q += (int64_t)gridDim.x * blockDim.x) {
     double s = 0.0;
-    for (int b = 0; b < B; ++b) s += acc[q * B + b];
+    for (int b = 0; b < B; ++b) s += acc[shot_index(q, b, B, pair_rows)];
     s *= dt;
     out[q] = accumulate ? out[q] + s : s;
   }
@@ -980,7 +987,7 @@ __global__ void lfe_source_kernel(const double* M, const int32_t* dofs, const do
 // dt is applied at the end with the velocity term.
 __global__ void gradient_term_kernel(const int64_t* ptr, const int32_t* col, const double* val, int64_t np,
                                      int64_t n_int, int B, const double* u_fwd, const double* lam_int,
-                                     const double* lam_b, double c2, double* grad) {
+                                     const double* lam_b, double c2, int64_t pair_rows, double* grad) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < np * B; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t q = t / B;
     const int s = (int)(t - q * B);
@@ -997,7 +1004,8 @@ __global__ void gradient_term_kernel(const int64_t* ptr, const int32_t* col, con
       gu[d] = au;
       gl[d] = al;
     }
-    grad[t] = fma(c2, fma(gu[0], gl[0], gu[1] * gl[1]), grad[t]);
+    double& out = grad[shot_index(q, s, B, pair_rows)];
+    out = fma(c2, fma(gu[0], gl[0], gu[1] * gl[1]), out);
   }
 }
 
@@ -1345,6 +1353,10 @@ struct Stepper {
   int finalize_exact();
   int check_status();
   bool tensor_core_path() const { return use_tc; }
+  // v, z, q and the gradient's interior part in pairs of rows: the tensor-core kernels on every
+  // element, n_b even (a class of elements shares its arrays with the FP64 kernel's layout)
+  bool row_pairs() const { return use_tc && (nb & 1) == 0; }
+  int64_t pair_rows() const { return row_pairs() ? nint : 0; }
   // doubles per step and shot in a forward-field store, and where its boundary part starts:
   // every nodal point, or the boundary nodes alone for the comparison method (no radial interior)
   int64_t store_stride() const { return md.lfe ? N : np; }
@@ -1772,8 +1784,8 @@ int Stepper::element_launch(int down, int up, int64_t done_step) {
   }
   prof.begin(kPhaseElement, st);
   if (use_tc || use_mixed)
-    tc_element_launch(md, B, down, up, ea.u, ea.ud, ea.udd, rb.v.as<double>(), ea.ub, ea.udb, ea.uddb, ea.q, ea.fhat,
-                      ea.store_int, ea.fwd_int, ea.grad_int, ea.u_out, st, use_mixed ? elems_tc.as<int32_t>() : nullptr,
+    tc_element_launch(md, B, down, up, ea.ud, rb.v.as<double>(), ea.ub, ea.udb, ea.uddb, ea.q, ea.fhat, ea.store_int,
+                      ea.fwd_int, ea.grad_int, ea.u_out, row_pairs(), st, use_mixed ? elems_tc.as<int32_t>() : nullptr,
                       n_tc, pstatus.as<int>());
   if (!use_tc && (!use_mixed || n_fp > 0)) element_step_kernel<<<e_blocks, e_threads, e_smem, st>>>(ea);
   prof.end(kPhaseElement, st);
@@ -1787,7 +1799,7 @@ int Stepper::element_launch(int down, int up, int64_t done_step) {
     gradient_term_kernel<<<blocks, 256, 0, st>>>(mdev.grad_ptr.as<int64_t>(), mdev.grad_col.as<int32_t>(),
                                                  mdev.grad_val.as<double>(), np, nint, B,
                                                  fwd_u + (K - 1 - done_step - fwd_k0) * np * B, rb.lam.as<double>(),
-                                                 rb.ub.as<double>(), md.c * md.c, rb.grad_int.as<double>());
+                                                 rb.ub.as<double>(), md.c * md.c, pair_rows(), rb.grad_int.as<double>());
     prof.count(kPhaseOther);
   }
   return SBFWI_OK;
@@ -2015,14 +2027,15 @@ __global__ void session_field_kernel(const SlotDev* slots, int B, int64_t stride
   }
 }
 
-__global__ void column_zero_kernel(double* buf, int64_t rows, int B, int s) {
+__global__ void column_zero_kernel(double* buf, int64_t rows, int B, int s, int64_t pair_rows) {
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < rows; q += (int64_t)gridDim.x * blockDim.x)
-    buf[q * B + s] = 0.0;
+    buf[shot_index(q, s, B, pair_rows)] = 0.0;
 }
 
-__global__ void column_copy_kernel(const double* acc, int64_t rows, int B, int s, double scale, double* out) {
+__global__ void column_copy_kernel(const double* acc, int64_t rows, int B, int s, int64_t pair_rows, double scale,
+                                   double* out) {
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < rows; q += (int64_t)gridDim.x * blockDim.x)
-    out[q] = scale * acc[q * B + s];
+    out[q] = scale * acc[shot_index(q, s, B, pair_rows)];
 }
 
 int Stepper::zero_column(int s) {
@@ -2034,8 +2047,10 @@ int Stepper::zero_column(int s) {
   for (DevBuf* b : bufs) {
     const int64_t rows = (int64_t)(b->bytes / sizeof(double)) / B;
     if (rows == 0) continue;
+    // the interior arrays of the tensor-core kernels are in pairs of rows
+    const int64_t pairs = (b == &rb.v || b == &rb.ud || b == &rb.grad_int) ? pair_rows() : 0;
     column_zero_kernel<<<(unsigned)std::min<int64_t>((rows + 255) / 256, 152 * 8), 256, 0, st>>>(b->as<double>(), rows,
-                                                                                                 B, s);
+                                                                                                 B, s, pairs);
     profiler().count(kPhaseOther);
   }
   SBFWI_CUDA(cudaGetLastError());
@@ -2119,7 +2134,7 @@ static int emit_gradient(Model& md, const double* g_lib, double* grad, int mem, 
     // the padded layout gathered to the caller's
     gather_nodal_kernel<<<gb, 256, 0, st>>>(g_lib, md.dev().api_map.as<int64_t>(), nout, dst, accumulate ? 1 : 0);
   } else {
-    sum_shots_kernel<<<gb, 256, 0, st>>>(g_lib, nout, 1, 1.0, dst, accumulate ? 1 : 0);
+    sum_shots_kernel<<<gb, 256, 0, st>>>(g_lib, nout, 1, 0, 1.0, dst, accumulate ? 1 : 0);
   }
   profiler().count(kPhaseOther);
   SBFWI_CUDA(cudaGetLastError());
@@ -2448,7 +2463,8 @@ int sbfwi_adjoint_gradient(sbfwi_model* md, sbfwi_fwdstate* fs, const double* re
   DevBuf gn;
   SBFWI_CUDA(gn.alloc(sizeof(double) * np));
   const unsigned blocks = (unsigned)std::min<int64_t>((np + 255) / 256, 152 * 8);
-  sum_shots_kernel<<<blocks, 256, 0, st>>>(rb.grad_int.as<double>(), np, Bsum, scale, gn.as<double>(), 0);
+  sum_shots_kernel<<<blocks, 256, 0, st>>>(rb.grad_int.as<double>(), np, Bsum, exact ? 0 : adj.pair_rows(), scale,
+                                           gn.as<double>(), 0);
   profiler().count(kPhaseOther);
   rc = emit_gradient(*md, gn.as<double>(), grad, mem, accumulate, st);
   profiler().resolve();
@@ -2707,7 +2723,7 @@ int sbfwi_session_collect(sbfwi_session* S, int32_t slot, double* out, int mem) 
     DevBuf g;
     SBFWI_CUDA(g.alloc(sizeof(double) * np));
     column_copy_kernel<<<(unsigned)std::min<int64_t>((np + 255) / 256, 152 * 8), 256, 0, st>>>(
-        S->rb.grad_int.as<double>(), np, S->B, slot, md.dt, g.as<double>());
+        S->rb.grad_int.as<double>(), np, S->B, slot, S->sp->pair_rows(), md.dt, g.as<double>());
     profiler().count(kPhaseOther);
     rc = emit_gradient(md, g.as<double>(), out, mem, false, st);
   }

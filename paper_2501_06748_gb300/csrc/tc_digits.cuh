@@ -47,24 +47,6 @@ __device__ __forceinline__ int exp_bound(double a) {
 // out of line so that its FP64 conversion is not evaluated speculatively on the hot path
 static __device__ __noinline__ double int_to_double_scaled_slow(long long t, int E) { return ldexp((double)t, E); }
 
-// t * 2^E as a binary64, rounded to nearest-even like a conversion of t, built with
-// integer operations (the scaling by 2^E is exact unless the result is subnormal)
-__device__ __forceinline__ double int_to_double_scaled(long long t, int E) {
-  if (t == 0) return 0.0;
-  const unsigned long long sign = t < 0 ? 0x8000000000000000ULL : 0ULL;
-  unsigned long long m = t < 0 ? (unsigned long long)(-t) : (unsigned long long)t;
-  const int lz = __clzll((long long)m);
-  m <<= lz;                                   // top bit at position 63
-  unsigned long long hi = m >> 11;            // 53 bits
-  const unsigned long long rem = m & 0x7FFULL;
-  if (rem > 0x400ULL || (rem == 0x400ULL && (hi & 1ULL))) ++hi;
-  int bexp = E - lz + 11 + 52 + 1023;
-  if (hi == (1ULL << 53)) { hi >>= 1; ++bexp; }
-  if (bexp >= 1 && bexp <= 2046)
-    return __longlong_as_double((long long)(sign | ((unsigned long long)bexp << 52) | (hi & 0x000FFFFFFFFFFFFFULL)));
-  return int_to_double_scaled_slow(t, E);
-}
-
 // six balanced base-512 digits, most significant first, as FP16 bit patterns of 1536 + d
 // The 54-bit recurrence runs on two 32-bit halves: the low 27 bits give the three
 // least significant digits and a carry (0 or 1) into the high half, which gives the
@@ -95,75 +77,6 @@ __device__ __forceinline__ unsigned pack_digits(unsigned short lo, unsigned shor
   h = __hsub2(h, __halves2half2(__ushort_as_half(0x6600), __ushort_as_half(0x6600)));
   return *reinterpret_cast<const unsigned*>(&h);
 }
-
-__device__ __forceinline__ void mma16816(float (&c)[4], const uint4& a, unsigned b0, unsigned b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
-}
-
-// Sum of the levels as an int64 with weight 2^-52 relative to 2^(e_r + f).  Levels
-// 2..6 are added exactly; levels 7 and 8 are summed exactly apart and rounded once to
-// the nearest unit (flooring them with shifts biases every product by about -1 unit,
-// which the energy-conserving time loop then accumulates).
-// (kNeg: the negated sum, negated in the integer domain -- rounding is symmetric, so the
-// result is bit for bit the negation of the kNeg = false one.)
-template <bool kNeg = false>
-__device__ __forceinline__ double recombine(const float (&acc)[kLevels][4], int j, int e) {
-  long long t = 0;
-  t += (long long)__float2int_rn(acc[0][j]) << 36;
-  t += (long long)__float2int_rn(acc[1][j]) << 27;
-  t += (long long)__float2int_rn(acc[2][j]) << 18;
-  t += (long long)__float2int_rn(acc[3][j]) << 9;
-  t += (long long)__float2int_rn(acc[4][j]);
-  const long long low = ((long long)__float2int_rn(acc[5][j]) << 9) + (long long)__float2int_rn(acc[6][j]);
-  t += (low + (1LL << 17)) >> 18;
-  return int_to_double_scaled(kNeg ? -t : t, e - 52);
-}
-
-// Digits of an operand held in the B-fragment layout of m16n8k16: lane (g, t) holds
-// rows 2t, 2t+1, 2t+8, 2t+9 of column g.  f is that column's exponent.
-struct BDigits {
-  unsigned r[kSlices][2];
-};
-
-__device__ __forceinline__ void split_b(const double (&x)[4], int f, BDigits& d) {
-  unsigned short h[4][kSlices];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) digits(to_fixed(x[j], f), h[j]);
-#pragma unroll
-  for (int k = 0; k < kSlices; ++k) {
-    d.r[k][0] = pack_digits(h[0][k], h[1][k]);
-    d.r[k][1] = pack_digits(h[2][k], h[3][k]);
-  }
-}
-
-// column exponent: max over the four lanes of a column group (lanes 4g..4g+3)
-__device__ __forceinline__ int column_exponent(int e) {
-  e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
-  e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
-  return e;
-}
-
-// acc[L] += sum_{k + l = L} A_k x_l over the kept levels; A slices in fragment layout
-__device__ __forceinline__ void product(float (&acc)[kLevels][4], const uint4* Aslices, const BDigits& x) {
-#pragma unroll
-  for (int k = 0; k < kSlices; ++k) {
-    const uint4 a = Aslices[k * 32];
-#pragma unroll
-    for (int l = 0; l < kSlices; ++l)
-      if (k + l < kLevels) mma16816(acc[k + l], a, x.r[l][0], x.r[l][1]);
-  }
-}
-
-__device__ __forceinline__ void zero(float (&acc)[kLevels][4]) {
-#pragma unroll
-  for (int L = 0; L < kLevels; ++L)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[L][j] = 0.f;
-}
-
 
 // ---------------------------------------------------------------------------
 // The shot-major product of the element step: y^T = x^T A^T, shots in the rows of the
@@ -241,7 +154,7 @@ __device__ __forceinline__ void digit_pairs(uint2 a, uint2 b, unsigned (&d)[kSli
   d[0] = unbias(((w0 >> 5) & 0x03FF03FFu) | one, 0x66006600u);                // 1024 + field; 1536
 }
 
-__device__ __forceinline__ void split_rows(const double (&x)[4], int E, XDigits& d) {
+__device__ __forceinline__ void split_rows(const double* x, int E, XDigits& d) {   // x: 4 values
   unsigned lo[kSlices], hi[kSlices];
   digit_pairs(biased_fixed(x[0], E), biased_fixed(x[1], E), lo);
   digit_pairs(biased_fixed(x[2], E), biased_fixed(x[3], E), hi);
@@ -261,15 +174,24 @@ constexpr int kZeroExp = -8192;                   // a column of zeros (or below
 __device__ __forceinline__ int exp_of_key(int key) { return key > 0 ? max(key >> 20, 1) : kZeroExp; }
 __device__ __forceinline__ bool scale_small(int ex) { return ex > kZeroExp / 2 && ex < kScaledExp; }
 
-__device__ __forceinline__ int column_scale(double (&x)[4], int& adj) {
-  auto ex_of = [&] { return exp_of_key(quad_max(max4(mag_key(x[0]), mag_key(x[1]), mag_key(x[2]), mag_key(x[3])))); };
+template <int kV>
+__device__ __forceinline__ int key_max(const double (&x)[kV]) {
+  int k = 0;
+#pragma unroll
+  for (int j = 0; j < kV; j += 4) k = max(k, max4(mag_key(x[j]), mag_key(x[j + 1]), mag_key(x[j + 2]), mag_key(x[j + 3])));
+  return k;
+}
+
+template <int kV>
+__device__ __forceinline__ int column_scale(double (&x)[kV], int& adj) {
+  auto ex_of = [&] { return exp_of_key(quad_max(key_max(x))); };
   int ex = ex_of();
   adj = 0;
   if (__any_sync(0xffffffffu, scale_small(ex))) {
     if (scale_small(ex)) {
       adj = kScaleBits;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) x[j] *= 0x1p256;
+      for (int j = 0; j < kV; ++j) x[j] *= 0x1p256;
     }
     ex = ex_of();
   }
@@ -277,19 +199,16 @@ __device__ __forceinline__ int column_scale(double (&x)[4], int& adj) {
 }
 
 // the same for the joint operand [v ; q 2^bal]
-__device__ __forceinline__ int column_scale2(double (&v)[4], double (&q)[4], int bal, int& adj) {
-  auto ex_of = [&] {
-    const int ev = exp_of_key(max4(mag_key(v[0]), mag_key(v[1]), mag_key(v[2]), mag_key(v[3])));
-    const int eq = exp_of_key(max4(mag_key(q[0]), mag_key(q[1]), mag_key(q[2]), mag_key(q[3])));
-    return quad_max(max(ev, eq + bal));
-  };
+template <int kV>
+__device__ __forceinline__ int column_scale2(double (&v)[kV], double (&q)[kV], int bal, int& adj) {
+  auto ex_of = [&] { return quad_max(max(exp_of_key(key_max(v)), exp_of_key(key_max(q)) + bal)); };
   int ex = ex_of();
   adj = 0;
   if (__any_sync(0xffffffffu, scale_small(ex))) {
     if (scale_small(ex)) {
       adj = kScaleBits;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) { v[j] *= 0x1p256; q[j] *= 0x1p256; }
+      for (int j = 0; j < kV; ++j) { v[j] *= 0x1p256; q[j] *= 0x1p256; }
     }
     ex = ex_of();
   }
@@ -333,8 +252,8 @@ struct LevelSums {
   static constexpr int kMaxParts = parts_of(4, kOps);
   float acc[kLevels][kMaxParts][4];
 
-  template <int kOp>
-  __device__ __forceinline__ void add(const XDigits& x, const uint2* B, const float (&start)[4]) {
+  // op: constant after unrolling
+  __device__ __forceinline__ void add(int op, const XDigits& x, const uint2* B, const float (&start)[4]) {
 #pragma unroll
     for (int k = 0; k < kSlices; ++k) {
       const uint2 b = B[k * 32];
@@ -342,7 +261,7 @@ struct LevelSums {
       for (int p = 0; p < kPairs; ++p) {
         if (!pair_kept(k, p)) continue;
         const int m = k + 2 * p;
-        const int pos = kOp * pairs_of(m) + pairs_before(m, k);
+        const int pos = op * pairs_of(m) + pairs_before(m, k);
         if (pos % 4 == 0) mma_pair<true>(acc[m][pos / 4], x.f[p], b, start);
         else mma_pair<false>(acc[m][pos / 4], x.f[p], b, start);
       }
@@ -369,11 +288,11 @@ struct LevelSums {
     // levels 0, 1 of a product stay below 2^22 (kOps <= 2), so their sum fits 32 bits; the two lowest are
     // rounded once to the nearest unit (floor(floor(x / 2^9) + 2^8) / 2^9 = floor((x + 2^17) / 2^18))
     const int low = (L[5] + (L[6] >> 9) + 256) >> 9;
-    const int top = L[0] * 512 + L[1];
     long long t = (long long)(L[4] + low);
     t += (long long)L[3] * 512;
     t += (long long)L[2] * (1 << 18);
-    t += (long long)top * (1 << 27);
+    if constexpr (kOps <= 2) t += (long long)(L[0] * 512 + L[1]) * (1 << 27);
+    else t += ((long long)L[0] * 512 + L[1]) * (1 << 27);
     return t;
   }
 };
@@ -441,31 +360,23 @@ struct SliceArgs {
   int64_t E;
   const double* mats;     // [E][n][3][nb][nb]
   const double* rt;       // [E][2][nb][nb]
-  uint4* frag;            // [E][n][3: P, Q, H][tiles][kSlices][32], tiles = 1 (n_b <= 16) or 4 (<= 32)
-  uint4* frag_rt;         // [E][2: R, T][tiles][kSlices][32]
-  int* exps;              // [E][n][3][16 or 32] row exponents
-  int* exps_rt;           // [E][2][16 or 32]
+  unsigned char* ops;     // [E][3 n + 2] operator blocks (tc::OpBlock)
 };
 
 struct ElemTcArgs {
   int nb, n, B;
   int64_t E;
   double a0, a1, a2, c1, c2, dt;
-  const uint4* frag;
-  const uint4* frag_rt;
-  const int* exps;
-  const int* exps_rt;
+  const unsigned char* ops;
   const int32_t* dofs;
-  double* u; double* ud; double* udd; double* v;          // interior state [E][n][nb][B]: this kernel
-                                                          // keeps v (predictor) in v and z = u' + dt (1 - gamma) u''
-                                                          // in ud; u and udd are unused
+  double* ud; double* v;  // interior state: v the predictor, ud holds z = u' + dt (1 - gamma) u''; u, u'' are not kept
   const double* ub; const double* udb; const double* uddb;
   double* q;
   double* fhat;
   int do_down, do_up;
-  double* store_int;
+  double* store_int;      // nodal fields [E][n][nb][B]
   const double* fwd_int;
-  double* grad_int;
+  double* grad_int;       // gradient accumulators, in the state's layout
   double* u_out;          // full Frechet kernel: the new interior displacements (store or adjoint field)
   // the elements this launch steps: elems[0..n_elems) (an element class of a mesh with
   // uneven elements), or all E elements when elems is NULL
@@ -477,6 +388,6 @@ struct ElemTcArgs {
 // elements padded to 21..32 boundary nodes (tc2.cu)
 constexpr int kTwoTileMinNb = 21;
 int tc2_prepare(Model& md, cudaStream_t st);
-int tc2_element_launch(const ElemTcArgs& a, bool avg_accel, cudaStream_t st);
+void tc2_element_launch(const ElemTcArgs& a, bool avg_accel, bool pair, cudaStream_t st);
 
 }  // namespace sbfwi
