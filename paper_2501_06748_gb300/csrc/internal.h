@@ -343,11 +343,33 @@ bool tc_supported(int nb, int B);   // the tensor-core kernel is the default for
 bool tc_available(int nb, int B);   // a tensor-core kernel exists for these shapes
 int tc_prepare(Model& md, cudaStream_t st);
 int tc_prepare_one_tile(Model& md, cudaStream_t st);   // one-tile digits even when n_b is padded beyond 16
-// pair: v, z (ud), q and grad_int are in pairs of rows [row / 2][shot][row % 2] per radial point (tc_step.cuh)
-int tc_element_launch(const Model& md, int B, int down, int up, double* ud, double* v, const double* ub,
-                      const double* udb, const double* uddb, double* q, double* fhat, double* store_int,
-                      const double* fwd_int, double* grad_int, double* u_out, bool pair, cudaStream_t st,
-                      const int32_t* elems = nullptr, int64_t n_elems = 0, int* status = nullptr);
+// The interior state of the tensor-core element kernels, per element and radial point: whole tiles
+// [16 or 32 rows / 2][8 shots][2], zero beyond n_b(e) and the shots of the pass, or [n_b][B]
+constexpr int kTileShots = 8;
+struct TcState {
+  bool tiles = false;
+  int doubles = 0;        // of one point
+};
+TcState tc_state(const Model& md, int B, int64_t n_elems, int sms);
+struct TcLaunch {
+  int B, do_down, do_up;
+  bool tiles;             // the layout of the state (TcState)
+  double* v; double* z;   // the predictor v and z = u' + dt (1 - gamma) u'' (u, u'' are not kept)
+  double* q;
+  double* grad;           // adjoint: gradient accumulators, in the state's layout (nullable)
+  const double* ub; const double* udb; const double* uddb;
+  double* fhat;
+  double* store_int;      // nodal fields [E][n][nb][B] (nullable): forward velocities of this step,
+  const double* fwd_int;  // adjoint: the paired forward velocities,
+  double* u_out;          // full Frechet kernel: the new interior displacements (store or adjoint field)
+  // the elements this launch steps: elems[0..n_elems) (an element class of a mesh with uneven
+  // elements, its state in the same order), or all E elements when elems is NULL
+  const int32_t* elems;
+  int64_t n_elems;
+  int sms;                // SMs of the device
+  int* status;            // a bounded wait that gives up records SBFWI_ETIMEOUT here (nullable)
+};
+int tc_element_launch(const Model& md, const TcLaunch& l, cudaStream_t st);
 
 struct FwdState {
   Model* model = nullptr;

@@ -943,18 +943,36 @@ __global__ void sources_kernel(double* ext, int B, int nsrc, const int64_t* node
 // ---------------------------------------------------------------------------
 // gradient: shots summed, then optionally the transpose of the bilinear map
 // ---------------------------------------------------------------------------
-// Per-shot value of row q, shot s in a [row][shot] array whose first `pair_rows` rows are in pairs
-// [row / 2][shot][row % 2] (the interior state and gradient of the tensor-core element kernels)
-__device__ __forceinline__ int64_t shot_index(int64_t q, int s, int B, int64_t pair_rows) {
-  return q < pair_rows ? ((q >> 1) * B + s) * 2 + (q & 1) : q * B + s;
+// Place of (row, shot) in a tile of the tensor-core kernels' state
+__device__ __forceinline__ int tile_place(int row, int s) { return ((row >> 1) * kTileShots + s) * 2 + (row & 1); }
+
+// The per-shot gradient accumulators: rows [row][shot] from nodal point row0 on, and those of the
+// interior points of the tensor-core kernels' elements, in their state's layout
+struct GradCells {
+  double* acc;              // [n_nodal - row0][B]
+  int64_t row0;
+  double* tc;               // nullable
+  const int32_t* place;     // [E] the element's place in tc, -1: in acc (nullable: element e's is e)
+  int64_t n_int;
+  int n, nb, B;
+  TcState state;
+};
+__device__ __forceinline__ double* grad_cell(const GradCells& g, int64_t q, int s) {
+  if (g.tc && q < g.n_int) {
+    const int64_t ei = q / g.nb, e = ei / g.n;
+    const int64_t t = g.place ? (int64_t)g.place[e] : e;
+    const int row = (int)(q - ei * g.nb);
+    if (t >= 0)
+      return g.tc + (t * g.n + (ei - e * g.n)) * g.state.doubles + (g.state.tiles ? tile_place(row, s) : row * g.B + s);
+  }
+  return g.acc + (q - g.row0) * g.B + s;
 }
 
 // g(node) = dt * sum over shots of the accumulated sum_m udot_fwd * lambdadot
-__global__ void sum_shots_kernel(const double* acc, int64_t np, int B, int64_t pair_rows, double dt, double* out,
-                                 int accumulate) {
+__global__ void sum_shots_kernel(GradCells g, int64_t np, double dt, double* out, int accumulate) {
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < np; q += (int64_t)gridDim.x * blockDim.x) {
     double s = 0.0;
-    for (int b = 0; b < B; ++b) s += acc[shot_index(q, b, B, pair_rows)];
+    for (int b = 0; b < g.B; ++b) s += *grad_cell(g, q, b);
     s *= dt;
     out[q] = accumulate ? out[q] + s : s;
   }
@@ -987,7 +1005,7 @@ __global__ void lfe_source_kernel(const double* M, const int32_t* dofs, const do
 // dt is applied at the end with the velocity term.
 __global__ void gradient_term_kernel(const int64_t* ptr, const int32_t* col, const double* val, int64_t np,
                                      int64_t n_int, int B, const double* u_fwd, const double* lam_int,
-                                     const double* lam_b, double c2, int64_t pair_rows, double* grad) {
+                                     const double* lam_b, double c2, GradCells grad) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < np * B; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t q = t / B;
     const int s = (int)(t - q * B);
@@ -1004,7 +1022,7 @@ __global__ void gradient_term_kernel(const int64_t* ptr, const int32_t* col, con
       gu[d] = au;
       gl[d] = al;
     }
-    double& out = grad[shot_index(q, s, B, pair_rows)];
+    double& out = *grad_cell(grad, q, s);
     out = fma(c2, fma(gu[0], gl[0], gu[1] * gl[1]), out);
   }
 }
@@ -1281,9 +1299,10 @@ int build_level_tasks(const Model& md, LevelTasks& lt, int B, int grid) {
 namespace {
 
 struct RunBuffers {
-  DevBuf u, ud, udd, v, ub, udb, uddb, q, fhat, ext, ysep, ybnd, x;
+  DevBuf u, ud, udd, ub, udb, uddb, q, fhat, ext, ysep, ybnd, x;
+  DevBuf tv, tz, tq, tg;            // tensor-core kernels: v, z, q and the gradient accumulators (TcState)
   DevBuf lam;                       // full kernel, adjoint: interior displacements of the current step
-  DevBuf grad_int;                  // grad accumulators [n_nodal][B] (adjoint)
+  DevBuf grad_int;                  // grad accumulators [n_nodal][B] (adjoint; boundary nodes alone if tg holds the rest)
   // exact adjoint: mu of rows -1..n, v_bar_n per element, ghosts of the forward solution,
   // Gauss-point products, boundary station of the gradient per element
   DevBuf mu, vbn, ghost, gacc, gbnd;
@@ -1353,10 +1372,7 @@ struct Stepper {
   int finalize_exact();
   int check_status();
   bool tensor_core_path() const { return use_tc; }
-  // v, z, q and the gradient's interior part in pairs of rows: the tensor-core kernels on every
-  // element, n_b even (a class of elements shares its arrays with the FP64 kernel's layout)
-  bool row_pairs() const { return use_tc && (nb & 1) == 0; }
-  int64_t pair_rows() const { return row_pairs() ? nint : 0; }
+  GradCells grad_cells() const;
   // doubles per step and shot in a forward-field store, and where its boundary part starts:
   // every nodal point, or the boundary nodes alone for the comparison method (no radial interior)
   int64_t store_stride() const { return md.lfe ? N : np; }
@@ -1374,6 +1390,9 @@ struct Stepper {
   bool use_tc = false, persistent = false;
   bool use_mixed = false;            // per-class kernels (one-tile tensor-core + FP64) on an uneven mesh
   DevBuf elems_tc, elems_fp;         // the element classes of the mixed kernels
+  DevBuf place_tc;                   // and each element's place in the tensor-core class (-1: FP64 class)
+  TcState tcs;
+  int sms = 0;
   int64_t n_tc = 0, n_fp = 0;
   ElemStepArgs ea;
   SolveArgs sa;
@@ -1409,6 +1428,10 @@ int Stepper::init() {
   const Tree& t = m.tree;
   nb = md.nb; n = md.n;
   E = md.E; N = md.N; np = m.n_nodal; nint = m.n_int;
+  int device = 0, coop = 0, per_sm = 0;
+  SBFWI_CUDA(cudaGetDevice(&device));
+  SBFWI_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device));
+  SBFWI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
   // boundary state has one extra zero row: the padding dofs of uneven meshes read it
   const int64_t si = nint * B, sb = N * B, sb1 = (N + 1) * B;
   // element kernel: FP16 tensor cores with error-free splitting when the shapes allow,
@@ -1462,15 +1485,25 @@ int Stepper::init() {
     SBFWI_CUDA(cudaMemcpy(elems_fp.p, large.data(), sizeof(int32_t) * large.size(), cudaMemcpyHostToDevice));
     n_tc = (int64_t)small.size();
     n_fp = (int64_t)large.size();
+    std::vector<int32_t> of(E, -1);
+    for (size_t k = 0; k < small.size(); ++k) of[small[k]] = (int32_t)k;
+    SBFWI_CUDA(place_tc.alloc(sizeof(int32_t) * of.size()));
+    SBFWI_CUDA(cudaMemcpy(place_tc.p, of.data(), sizeof(int32_t) * of.size(), cudaMemcpyHostToDevice));
   }
-  // the tensor-core path carries the predictor v and z = u' + dt (1 - gamma) u'' (in ud), not u, u''
+  // the tensor-core path carries the predictor v and z = u' + dt (1 - gamma) u'', not u, u', u''
   // the comparison method keeps no interior state
-  const int64_t si_state = md.lfe ? 1 : si;
-  SBFWI_CUDA(rb.u.alloc(sizeof(double) * (use_tc ? 1 : si_state)));
-  SBFWI_CUDA(rb.ud.alloc(sizeof(double) * si_state));
-  SBFWI_CUDA(rb.udd.alloc(sizeof(double) * (use_tc ? 1 : si_state)));
-  SBFWI_CUDA(rb.q.alloc(sizeof(double) * si_state));
-  if (use_tc || use_mixed) SBFWI_CUDA(rb.v.alloc(sizeof(double) * si));
+  const int64_t si_state = (md.lfe || use_tc) ? 1 : si;
+  for (DevBuf* b : {&rb.u, &rb.ud, &rb.udd, &rb.q}) SBFWI_CUDA(b->alloc(sizeof(double) * si_state));
+  const int64_t n_state = use_tc ? E : use_mixed ? n_tc : 0;
+  if (n_state > 0) {
+    tcs = tc_state(md, B, n_state, sms);
+    const size_t bytes = sizeof(double) * (size_t)n_state * n * tcs.doubles;
+    for (DevBuf* b : {&rb.tv, &rb.tz, &rb.tq}) SBFWI_CUDA(b->alloc(bytes));
+    if (mode == Mode::Adjoint) {
+      SBFWI_CUDA(rb.tg.alloc(bytes));
+      SBFWI_CUDA(cudaMemsetAsync(rb.tg.p, 0, rb.tg.bytes, st));
+    }
+  }
   SBFWI_CUDA(rb.ub.alloc(sizeof(double) * sb1));
   SBFWI_CUDA(rb.udb.alloc(sizeof(double) * sb1));
   SBFWI_CUDA(rb.uddb.alloc(sizeof(double) * sb1));
@@ -1480,7 +1513,7 @@ int Stepper::init() {
   SBFWI_CUDA(rb.ysep.alloc(sizeof(double) * std::max<int64_t>(t.sep_rows, 1) * B));
   SBFWI_CUDA(rb.ybnd.alloc(sizeof(double) * std::max<int64_t>(t.bnd_rows, 1) * B));
   if (mode == Mode::Adjoint) {
-    SBFWI_CUDA(rb.grad_int.alloc(sizeof(double) * np * B));
+    SBFWI_CUDA(rb.grad_int.alloc(sizeof(double) * (use_tc ? N : np) * B));
     SBFWI_CUDA(cudaMemsetAsync(rb.grad_int.p, 0, rb.grad_int.bytes, st));
   }
   if (mode == Mode::Exact) {
@@ -1501,10 +1534,6 @@ int Stepper::init() {
   // the solve's tasks are built for 4 blocks per SM; a block task stages its front's
   // vectors and its rows of the factors in shared memory, a warp task the same for a
   // whole small front, one slice per warp
-  int device = 0, coop = 0, sms = 0, per_sm = 0;
-  SBFWI_CUDA(cudaGetDevice(&device));
-  SBFWI_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device));
-  SBFWI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
   const int grid = 4 * sms;
   lt = tasks_own ? tasks_own : &md.tasks;
   if (lt->shots != B || lt->grid != grid) {
@@ -1720,15 +1749,29 @@ int Stepper::launch_solve(const void* fn, unsigned grid, void** args, bool coope
 }
 
 int Stepper::zero_state() {
-  for (DevBuf* b : {&rb.u, &rb.ud, &rb.udd, &rb.v, &rb.q, &rb.ub, &rb.udb, &rb.uddb, &rb.ext, &rb.x, &rb.fhat})
+  for (DevBuf* b : {&rb.u, &rb.ud, &rb.udd, &rb.q, &rb.tv, &rb.tz, &rb.tq, &rb.ub, &rb.udb, &rb.uddb, &rb.ext, &rb.x, &rb.fhat})
     if (b->p) SBFWI_CUDA(cudaMemsetAsync(b->p, 0, b->bytes, st));
   return SBFWI_OK;
 }
 
 std::vector<DevBuf*> Stepper::state_bufs() const {
-  if (use_tc) return {&rb.v, &rb.ud, &rb.ub, &rb.udb, &rb.uddb};
-  if (use_mixed) return {&rb.u, &rb.ud, &rb.udd, &rb.v, &rb.ub, &rb.udb, &rb.uddb};
+  if (use_tc) return {&rb.tv, &rb.tz, &rb.ub, &rb.udb, &rb.uddb};
+  if (use_mixed) return {&rb.u, &rb.ud, &rb.udd, &rb.tv, &rb.tz, &rb.ub, &rb.udb, &rb.uddb};
   return {&rb.u, &rb.ud, &rb.udd, &rb.ub, &rb.udb, &rb.uddb};
+}
+
+GradCells Stepper::grad_cells() const {
+  GradCells g = {};
+  g.acc = rb.grad_int.as<double>();
+  g.B = mode == Mode::Exact ? 1 : B;
+  if (mode == Mode::Adjoint && rb.tg.p) {
+    g.row0 = use_tc ? nint : 0;
+    g.tc = rb.tg.as<double>();
+    g.place = use_mixed ? place_tc.as<int32_t>() : nullptr;
+    g.n_int = nint;
+    g.n = n; g.nb = nb; g.state = tcs;
+  }
+  return g;
 }
 
 int64_t Stepper::state_doubles() const {
@@ -1783,10 +1826,19 @@ int Stepper::element_launch(int down, int up, int64_t done_step) {
     ea.grad_int = rb.grad_int.as<double>();
   }
   prof.begin(kPhaseElement, st);
-  if (use_tc || use_mixed)
-    tc_element_launch(md, B, down, up, ea.ud, rb.v.as<double>(), ea.ub, ea.udb, ea.uddb, ea.q, ea.fhat, ea.store_int,
-                      ea.fwd_int, ea.grad_int, ea.u_out, row_pairs(), st, use_mixed ? elems_tc.as<int32_t>() : nullptr,
-                      n_tc, pstatus.as<int>());
+  if (use_tc || use_mixed) {
+    TcLaunch l;
+    l.B = B; l.do_down = down; l.do_up = up; l.tiles = tcs.tiles;
+    l.v = rb.tv.as<double>(); l.z = rb.tz.as<double>(); l.q = rb.tq.as<double>();
+    l.grad = ea.fwd_int ? rb.tg.as<double>() : nullptr;
+    l.ub = ea.ub; l.udb = ea.udb; l.uddb = ea.uddb; l.fhat = ea.fhat;
+    l.store_int = ea.store_int; l.fwd_int = ea.fwd_int; l.u_out = ea.u_out;
+    l.elems = use_mixed ? elems_tc.as<int32_t>() : nullptr;
+    l.n_elems = n_tc;
+    l.sms = sms;
+    l.status = pstatus.as<int>();
+    tc_element_launch(md, l, st);
+  }
   if (!use_tc && (!use_mixed || n_fp > 0)) element_step_kernel<<<e_blocks, e_threads, e_smem, st>>>(ea);
   prof.end(kPhaseElement, st);
   prof.count(kPhaseElement, use_mixed ? 2 : 1);
@@ -1799,7 +1851,7 @@ int Stepper::element_launch(int down, int up, int64_t done_step) {
     gradient_term_kernel<<<blocks, 256, 0, st>>>(mdev.grad_ptr.as<int64_t>(), mdev.grad_col.as<int32_t>(),
                                                  mdev.grad_val.as<double>(), np, nint, B,
                                                  fwd_u + (K - 1 - done_step - fwd_k0) * np * B, rb.lam.as<double>(),
-                                                 rb.ub.as<double>(), md.c * md.c, pair_rows(), rb.grad_int.as<double>());
+                                                 rb.ub.as<double>(), md.c * md.c, grad_cells());
     prof.count(kPhaseOther);
   }
   return SBFWI_OK;
@@ -1890,7 +1942,7 @@ int Stepper::run(int64_t k0, int64_t k1) {
       ba.store_ab = store_a ? store_a + (k - store_k0) * np * B + nint * B : nullptr;
     } else {
       ba.fwd_b = fwd + ((K - 1 - k - fwd_k0) * store_stride() + store_bnd_off()) * B;
-      ba.grad_b = rb.grad_int.as<double>() + nint * B;
+      ba.grad_b = rb.grad_int.as<double>() + (use_tc ? 0 : nint * B);
     }
     boundary_update_kernel<<<b_blocks, 256, 0, st>>>(ba);
     prof.count(kPhaseOther);
@@ -2027,15 +2079,20 @@ __global__ void session_field_kernel(const SlotDev* slots, int B, int64_t stride
   }
 }
 
-__global__ void column_zero_kernel(double* buf, int64_t rows, int B, int s, int64_t pair_rows) {
+__global__ void column_zero_kernel(double* buf, int64_t rows, int B, int s) {
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < rows; q += (int64_t)gridDim.x * blockDim.x)
-    buf[shot_index(q, s, B, pair_rows)] = 0.0;
+    buf[q * B + s] = 0.0;
 }
 
-__global__ void column_copy_kernel(const double* acc, int64_t rows, int B, int s, int64_t pair_rows, double scale,
-                                   double* out) {
+// the same for an array of tiles
+__global__ void tile_column_zero_kernel(double* buf, int64_t rows, int s) {
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < rows; q += (int64_t)gridDim.x * blockDim.x)
-    out[q] = scale * acc[shot_index(q, s, B, pair_rows)];
+    buf[((q >> 1) * kTileShots + s) * 2 + (q & 1)] = 0.0;
+}
+
+__global__ void column_copy_kernel(GradCells g, int64_t rows, int s, double scale, double* out) {
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < rows; q += (int64_t)gridDim.x * blockDim.x)
+    out[q] = scale * *grad_cell(g, q, s);
 }
 
 int Stepper::zero_column(int s) {
@@ -2043,14 +2100,17 @@ int Stepper::zero_column(int s) {
   // the sources kernel writes only the column's current source node: the previous
   // request's last sample at its node must not act on the next one
   bufs.push_back(&rb.ext);
-  if (mode == Mode::Adjoint) bufs.push_back(&rb.grad_int);
+  if (mode == Mode::Adjoint) {
+    bufs.push_back(&rb.grad_int);
+    bufs.push_back(&rb.tg);
+  }
   for (DevBuf* b : bufs) {
-    const int64_t rows = (int64_t)(b->bytes / sizeof(double)) / B;
+    const bool tile = tcs.tiles && (b == &rb.tv || b == &rb.tz || b == &rb.tg);
+    const int64_t rows = (int64_t)(b->bytes / sizeof(double)) / (tile ? kTileShots : B);
     if (rows == 0) continue;
-    // the interior arrays of the tensor-core kernels are in pairs of rows
-    const int64_t pairs = (b == &rb.v || b == &rb.ud || b == &rb.grad_int) ? pair_rows() : 0;
-    column_zero_kernel<<<(unsigned)std::min<int64_t>((rows + 255) / 256, 152 * 8), 256, 0, st>>>(b->as<double>(), rows,
-                                                                                                 B, s, pairs);
+    const unsigned blocks = (unsigned)std::min<int64_t>((rows + 255) / 256, 152 * 8);
+    if (tile) tile_column_zero_kernel<<<blocks, 256, 0, st>>>(b->as<double>(), rows, s);
+    else column_zero_kernel<<<blocks, 256, 0, st>>>(b->as<double>(), rows, B, s);
     profiler().count(kPhaseOther);
   }
   SBFWI_CUDA(cudaGetLastError());
@@ -2134,7 +2194,10 @@ static int emit_gradient(Model& md, const double* g_lib, double* grad, int mem, 
     // the padded layout gathered to the caller's
     gather_nodal_kernel<<<gb, 256, 0, st>>>(g_lib, md.dev().api_map.as<int64_t>(), nout, dst, accumulate ? 1 : 0);
   } else {
-    sum_shots_kernel<<<gb, 256, 0, st>>>(g_lib, nout, 1, 0, 1.0, dst, accumulate ? 1 : 0);
+    GradCells g = {};
+    g.acc = const_cast<double*>(g_lib);
+    g.B = 1;
+    sum_shots_kernel<<<gb, 256, 0, st>>>(g, nout, 1.0, dst, accumulate ? 1 : 0);
   }
   profiler().count(kPhaseOther);
   SBFWI_CUDA(cudaGetLastError());
@@ -2458,13 +2521,11 @@ int sbfwi_adjoint_gradient(sbfwi_model* md, sbfwi_fwdstate* fs, const double* re
   if (rc) return rc;
   // the paper's kernel accumulates per shot and applies dt at the end; the exact gradient is
   // already summed over shots (dt is in its misfit adjoint)
-  const int Bsum = exact ? 1 : B;
   const double scale = exact ? 1.0 : md->dt;
   DevBuf gn;
   SBFWI_CUDA(gn.alloc(sizeof(double) * np));
   const unsigned blocks = (unsigned)std::min<int64_t>((np + 255) / 256, 152 * 8);
-  sum_shots_kernel<<<blocks, 256, 0, st>>>(rb.grad_int.as<double>(), np, Bsum, exact ? 0 : adj.pair_rows(), scale,
-                                           gn.as<double>(), 0);
+  sum_shots_kernel<<<blocks, 256, 0, st>>>(adj.grad_cells(), np, scale, gn.as<double>(), 0);
   profiler().count(kPhaseOther);
   rc = emit_gradient(*md, gn.as<double>(), grad, mem, accumulate, st);
   profiler().resolve();
@@ -2723,7 +2784,7 @@ int sbfwi_session_collect(sbfwi_session* S, int32_t slot, double* out, int mem) 
     DevBuf g;
     SBFWI_CUDA(g.alloc(sizeof(double) * np));
     column_copy_kernel<<<(unsigned)std::min<int64_t>((np + 255) / 256, 152 * 8), 256, 0, st>>>(
-        S->rb.grad_int.as<double>(), np, S->B, slot, S->sp->pair_rows(), md.dt, g.as<double>());
+        S->sp->grad_cells(), np, slot, md.dt, g.as<double>());
     profiler().count(kPhaseOther);
     rc = emit_gradient(md, g.as<double>(), out, mem, false, st);
   }

@@ -72,27 +72,37 @@ int tc_prepare_one_tile(Model& md, cudaStream_t st) {
   return SBFWI_OK;
 }
 
-int tc_element_launch(const Model& md, int B, int down, int up, double* ud, double* v, const double* ub,
-                      const double* udb, const double* uddb, double* q, double* fhat, double* store_int,
-                      const double* fwd_int, double* grad_int, double* u_out, bool pair, cudaStream_t st,
-                      const int32_t* elems, int64_t n_elems, int* status) {
+int tc_tile_rows(const Model& md) { return md.nb > tc::kTile && !md.tc_one_tile ? 2 * tc::kTile : tc::kTile; }
+
+// Whole tiles save the bounds checks, rows save the traffic of the padding.  Fused launches, tiles | rows, ms:
+// 24 x 24 elements, N_r 16: n_b 16, 8 shots 0.055 | 0.060, n_b 8, 3 shots (5.3 times the values) 0.053 | 0.054,
+// n_b 4, 3 shots (10.7 times) 0.053 | 0.053, n_b 4, 1 shot 0.053 | 0.051; 64 x 64 elements: n_b 16, 8 shots
+// 0.217 | 0.219, 5 shots (1.6 times) 0.212 | 0.203, n_b 8, 8 shots (twice) 0.211 | 0.198.  Two tiles, 32 x 32
+// elements: n_b 24, 8 shots 0.243 | 0.254, n_b 32, 4 shots (twice) 0.243 | 0.249.
+TcState tc_state(const Model& md, int B, int64_t n_elems, int sms) {
+  TcState t;
+  const int rows = tc_tile_rows(md), nb = md.nb;
+  const double most = n_elems <= kFewElements * (int64_t)sms ? 5.4 : rows > tc::kTile ? 2.0 : 1.1;
+  t.tiles = rows * kTileShots <= most * nb * B;
+  t.doubles = t.tiles ? rows * kTileShots : nb * B;
+  return t;
+}
+
+int tc_element_launch(const Model& md, const TcLaunch& l, cudaStream_t st) {
   ElemTcArgs a;
-  a.nb = md.nb; a.n = md.n; a.B = B; a.E = md.E;
+  a.l = l;
+  a.nb = md.nb; a.n = md.n; a.E = md.E;
   a.a0 = md.a0; a.a1 = md.a1; a.a2 = md.a2; a.c1 = md.c1; a.c2 = md.c2; a.dt = md.dt;
   a.ops = md.tc_ops.as<unsigned char>();
   a.dofs = md.dev().dofs.as<int32_t>();
-  a.ud = ud; a.v = v; a.ub = ub; a.udb = udb; a.uddb = uddb; a.q = q; a.fhat = fhat;
-  a.do_down = down; a.do_up = up;
-  a.store_int = store_int; a.fwd_int = fwd_int; a.grad_int = grad_int; a.u_out = u_out;
-  a.elems = elems; a.n_elems = elems ? n_elems : md.E;
-  a.status = status;
-  if (a.n_elems == 0) return SBFWI_OK;
+  if (!l.elems) a.l.n_elems = md.E;
+  if (a.l.n_elems == 0) return SBFWI_OK;
   // average acceleration (beta = 1/4, gamma = 1/2): the shorter predictor update
   const bool avg = md.a2 == 1.0 && md.c1 == md.c2;
   // one 16-row tile: n_b <= 16, or the elements of n_b <= 16 of a mesh padded beyond (the
   // one-tile digits of its operators, prepared by tc_prepare_one_tile)
-  if (md.nb > tc::kTile && !md.tc_one_tile) tc2_element_launch(a, avg, pair, st);
-  else tc_launch_tiles<1>(a, avg, pair, st);
+  if (tc_tile_rows(md) > tc::kTile) tc2_element_launch(a, avg, st);
+  else tc_launch_tiles<1>(a, avg, st);
   return SBFWI_OK;
 }
 

@@ -9,8 +9,8 @@ namespace sbfwi {
 
 int tc2_prepare(Model& md, cudaStream_t st) { return tc_prepare_tiles<2>(md, st); }
 
-void tc2_element_launch(const ElemTcArgs& a, bool avg_accel, bool pair, cudaStream_t st) {
-  tc_launch_tiles<2>(a, avg_accel, pair, st);
+void tc2_element_launch(const ElemTcArgs& a, bool avg_accel, cudaStream_t st) {
+  tc_launch_tiles<2>(a, avg_accel, st);
 }
 
 }  // namespace sbfwi

@@ -95,14 +95,14 @@ __device__ __forceinline__ unsigned pack_digits(unsigned short lo, unsigned shor
 //  - accumulators start at 1.5 * 2^23, so the bits of a sum are the constant plus the sum
 //    (exact while |sum| <= 2^22: at most four mma of 16 products of |digit| <= 256 per
 //    accumulator) and the levels are added as 32-bit integers.
-// The digits, the kept levels and the rounding are those of split_b and recombine.
-// Measured (64 x 64 elements, n_b 16, N_r 32, 8 shots): fused launch 0.555 -> 0.463 ms,
-// 2124 -> 1665 instructions per warp and radial point of both sweeps, DRAM 5.5 TB/s.
+// Measured (64 x 64 elements, n_b 16, N_r 32, 8 shots), with the operator blocks, ring and tiled
+// state of tc_step.cuh: fused launch 0.555 -> 0.394 ms, 2124 -> 1500 instructions per warp and
+// radial point of both sweeps, DRAM 4.5 -> 6.2 TB/s (6.8 measured copy).
 // ---------------------------------------------------------------------------
 constexpr int kPairs = kSlices / 2;
 constexpr float kMagicF = 12582912.0f;            // 1.5 * 2^23: bits 0x4B400000
 constexpr unsigned kMagicBits = 0x4B400000u;
-constexpr int kMinExp = 64;                       // least biased exponent of a column's scale
+constexpr int kMinExp = 64;                       // least biased exponent of a nonzero column's scale
 constexpr int kScaledExp = 128;                   // columns below 2^(128 - 1023) are scaled up first
 constexpr int kScaleBits = 256;
 
@@ -165,7 +165,8 @@ __device__ __forceinline__ void split_rows(const double* x, int E, XDigits& d) {
 // Biased exponent E of the scale of a column (shot) of 16 rows: |x| < 2^(E - 1022) for its entries, shared
 // by the four lanes of the shot.  Columns near the bottom of the range are scaled up by 2^256 first
 // (adj = 256, a whole warp's branch that the path's fields rarely take), so that subnormal entries keep
-// their bits; E is at least kMinExp, which makes the shift of zero entries clear them.
+// their bits; then E > 62, which makes the shift of zero entries clear them (a column of zeros takes
+// E = 1022, whose results stay inside scaled_double's range).
 __device__ __forceinline__ int quad_max(int v) {
   v = max(v, __shfl_xor_sync(0xffffffffu, v, 1));
   return max(v, __shfl_xor_sync(0xffffffffu, v, 2));
@@ -195,7 +196,7 @@ __device__ __forceinline__ int column_scale(double (&x)[kV], int& adj) {
     }
     ex = ex_of();
   }
-  return max(ex, kMinExp);
+  return ex < kMinExp ? 1022 : ex;
 }
 
 // the same for the joint operand [v ; q 2^bal]
@@ -212,7 +213,7 @@ __device__ __forceinline__ int column_scale2(double (&v)[kV], double (&q)[kV], i
     }
     ex = ex_of();
   }
-  return max(ex, kMinExp);
+  return ex < kMinExp ? 1022 : ex;
 }
 
 // mma of a digit pair fragment and an operator digit, on top of c (kFirst: of the start value)
@@ -268,7 +269,8 @@ struct LevelSums {
     }
   }
 
-  // column c (0, 1) of this lane's row pair: the sum over the levels as an int64 (see recombine)
+  // column c (0, 1) of this lane's row pair: the sum over the levels as an int64 with weight 2^-52 relative to
+  // 2^(e_r + f)
   __device__ __forceinline__ long long total(int c) const {
     int L[kLevels];
 #pragma unroll
@@ -285,8 +287,10 @@ struct LevelSums {
     return combine(L);
   }
   static __device__ __forceinline__ long long combine(const int (&L)[kLevels]) {
-    // levels 0, 1 of a product stay below 2^22 (kOps <= 2), so their sum fits 32 bits; the two lowest are
-    // rounded once to the nearest unit (floor(floor(x / 2^9) + 2^8) / 2^9 = floor((x + 2^17) / 2^18))
+    // Levels 2..6 are added exactly; levels 7 and 8 are summed exactly apart and rounded once to the nearest
+    // unit (floor(floor(x / 2^9) + 2^8) / 2^9 = floor((x + 2^17) / 2^18)); flooring them with shifts biases
+    // every product by about -1 unit, which the energy-conserving time loop then accumulates.  Levels 2, 3
+    // stay below 2^22 for kOps <= 2, so that their sum fits 32 bits.
     const int low = (L[5] + (L[6] >> 9) + 256) >> 9;
     long long t = (long long)(L[4] + low);
     t += (long long)L[3] * 512;
@@ -297,21 +301,35 @@ struct LevelSums {
   }
 };
 
-// t * 2^(s) as a binary64, rounded to nearest-even (int_to_double_scaled with fewer operations: the
-// significand is normalised to bit 62 and a carry of the rounding moves into the exponent by itself)
+// t * 2^s as a binary64, rounded to nearest-even like a conversion of t, with integer operations (the
+// scaling by 2^s is exact unless the result is subnormal): the significand is normalised to bit 62 and a
+// carry of the rounding moves into the exponent by itself.  rare: the result may lie outside the normal
+// range.  (The conversion instruction takes the FP64 pipe for as long as this takes the integer one: with
+// it the fused launch took 0.459 instead of 0.433 ms.)
 template <bool kNeg>
-__device__ __forceinline__ double scaled_double(long long t, int s) {
-  const unsigned neg = kNeg ? ~0u : 0u;
-  const unsigned long long mag = (unsigned long long)(t < 0 ? -t : t);
-  const unsigned sign = (((unsigned)(t >> 32)) ^ neg) & 0x80000000u;
+__device__ __forceinline__ double scaled_double(long long t, int s, bool& rare) {
+  const int hi = (int)(t >> 32), sg = hi >> 31;
+  const unsigned long long mag = (unsigned long long)((t ^ (long long)sg) - (long long)sg);
   const int lz = __clzll((long long)mag);
   unsigned long long m = mag << ((lz - 1) & 63);
   m += 0x1FFULL + ((m >> 10) & 1ULL);
   const int be = s - lz + (1023 + 62);            // biased exponent - 1 (t != 0)
-  unsigned long long bits = (m >> 10) + ((unsigned long long)(unsigned)be << 52);
-  if (t == 0) return 0.0;
-  if ((unsigned)be > 2044u) return int_to_double_scaled_slow(kNeg ? -t : t, s);
-  return __longlong_as_double((long long)(bits | ((unsigned long long)sign << 32)));
+  const unsigned blo = (unsigned)(m >> 10), bhi = (unsigned)(m >> 42) + ((unsigned)be << 20);
+  const unsigned sgn = (kNeg ? ~(unsigned)hi : (unsigned)hi) & 0x80000000u;
+  rare |= (unsigned)be > 2044u;
+  return __hiloint2double((int)(lz == 64 ? 0u : bhi | sgn), (int)blo);
+}
+
+// kN of them with one branch for the rare ones (one branch each: 0.433 instead of 0.415 ms)
+template <int kN, bool kNeg>
+__device__ __forceinline__ void scaled_doubles(const long long (&t)[kN], const int (&s)[kN], double (&y)[kN]) {
+  bool rare = false;
+#pragma unroll
+  for (int j = 0; j < kN; ++j) y[j] = scaled_double<kNeg>(t[j], s[j], rare);
+  if (rare) {
+#pragma unroll
+    for (int j = 0; j < kN; ++j) y[j] = int_to_double_scaled_slow(kNeg ? -t[j] : t[j], s[j]);
+  }
 }
 
 // Bulk global -> shared copies by the TMA engine (cp.async.bulk), completing on an mbarrier
@@ -364,30 +382,20 @@ struct SliceArgs {
 };
 
 struct ElemTcArgs {
-  int nb, n, B;
+  int nb, n;
   int64_t E;
   double a0, a1, a2, c1, c2, dt;
   const unsigned char* ops;
   const int32_t* dofs;
-  double* ud; double* v;  // interior state: v the predictor, ud holds z = u' + dt (1 - gamma) u''; u, u'' are not kept
-  const double* ub; const double* udb; const double* uddb;
-  double* q;
-  double* fhat;
-  int do_down, do_up;
-  double* store_int;      // nodal fields [E][n][nb][B]
-  const double* fwd_int;
-  double* grad_int;       // gradient accumulators, in the state's layout
-  double* u_out;          // full Frechet kernel: the new interior displacements (store or adjoint field)
-  // the elements this launch steps: elems[0..n_elems) (an element class of a mesh with
-  // uneven elements), or all E elements when elems is NULL
-  const int32_t* elems;
-  int64_t n_elems;
-  int* status;            // a bounded wait that gives up records SBFWI_ETIMEOUT here (nullable)
+  TcLaunch l;
 };
+
+// up to this many elements per SM a launch is short of warps rather than of bandwidth (tc_launch_tiles, tc_state)
+constexpr int kFewElements = 13;
 
 // elements padded to 21..32 boundary nodes (tc2.cu)
 constexpr int kTwoTileMinNb = 21;
 int tc2_prepare(Model& md, cudaStream_t st);
-void tc2_element_launch(const ElemTcArgs& a, bool avg_accel, bool pair, cudaStream_t st);
+void tc2_element_launch(const ElemTcArgs& a, bool avg_accel, cudaStream_t st);
 
 }  // namespace sbfwi

@@ -24,33 +24,36 @@ struct OpBlock {
   static constexpr int kBytes = kFragBytes + kRows * 4;
 };
 
-// Radial slots of a warp: the pipeline depth in operators, and the launch shape.  Measured on
-// 64 x 64 elements, n_b 16, 8 shots: RING
-template <int kRT>
+// Operator slots per warp, warps (elements) per block and blocks per SM.  Shared memory taken by
+// the slots is lost to L1, which joins the two rows of a lane in the nodal fields, and deeper
+// rings pay only where few warps share an SM.  Two tiles: 12 KB an operator, so 3 slots and 6
+// warps per SM (0.72 ms on the 16^3 cube of n_b 26, 8 shots; 4 slots and 4 warps 0.89 ms).
+// One tile: kDeep false for many elements, true (one warp per block, so that the last elements
+// spread over the SMs) for few; see tc_launch_tiles for the line between them.
+template <int kRT, bool kDeep>
 struct Shape {
-  static constexpr int kSlots = kRT == 1 ? 4 : 3;
-  static constexpr int kWarps = kRT == 1 ? 4 : 2;          // warps (elements) per block
-  static constexpr int kBlocks = kRT == 1 ? 4 : 3;         // blocks per SM
+  static constexpr int kSlots = kRT == 1 && kDeep ? 4 : 3;
+  static constexpr int kWarps = kRT == 1 ? (kDeep ? 1 : 4) : 2;
+  static constexpr int kBlocks = kRT == 1 ? (kDeep ? 16 : 4) : 3;
 };
 
-template <int kRT>
+template <int kRT, int kSlots>
 struct __align__(16) WarpSmem {
-  unsigned char op[Shape<kRT>::kSlots][OpBlock<kRT>::kBytes];
-  uint64_t bar[Shape<kRT>::kSlots + (Shape<kRT>::kSlots & 1)];
+  unsigned char op[kSlots][OpBlock<kRT>::kBytes];
+  uint64_t bar[kSlots + (kSlots & 1)];
 };
 
 // A warp's ring of operator slots.  fetch, init: lane 0.
-template <int kRT>
+template <int kRT, int kSlots>
 struct Ring {
   using Op = OpBlock<kRT>;
-  static constexpr int kSlots = Shape<kRT>::kSlots;
-  WarpSmem<kRT>& W;
+  WarpSmem<kRT, kSlots>& W;
   const unsigned char* ops;   // the element's operators
   int n, item, end;           // next item to be read, end of the items
   int slot = 0;               // its slot
   unsigned parity = 0;        // of the ring's current round
 
-  __device__ __forceinline__ Ring(WarpSmem<kRT>& w, const unsigned char* o, int n_, int first, int last)
+  __device__ __forceinline__ Ring(WarpSmem<kRT, kSlots>& w, const unsigned char* o, int n_, int first, int last)
       : W(w), ops(o), n(n_), item(first), end(last) {}
   __device__ __forceinline__ void fetch(int k, int s) {
     const int j = k - n;
@@ -91,9 +94,8 @@ struct Ring {
 // last() runs once the digits are read; put(j, y_j, y_{j+1}) takes the lane's results in pairs.
 template <int kRT, int kOps, bool kNeg, class Last, class Put>
 __device__ __forceinline__ void product(const uint2* b0, const uint2* b1, const int* rexp, const XDigits* x, int f, int lane,
-                                        Last last, Put put) {
+                                        const float (&start)[4], Last last, Put put) {
   constexpr int kTile2 = OpBlock<kRT>::kTileFrags;
-  const float start[4] = {kMagicF, kMagicF, kMagicF, kMagicF};
   int2 er[2 * kRT];
 #pragma unroll
   for (int nt = 0; nt < 2 * kRT; ++nt) er[nt] = *reinterpret_cast<const int2*>(rexp + nt * 8 + 2 * (lane & 3));
@@ -107,50 +109,55 @@ __device__ __forceinline__ void product(const uint2* b0, const uint2* b1, const 
       for (int k = 0; k < kRT; ++k) sums.add(kRT + k, x[kRT + k], b1 + (nt * kRT + k) * kTile2 + lane, start);
     }
     if (nt == 2 * kRT - 1) last();
-    put(2 * nt, scaled_double<kNeg>(sums.total(0), er[nt].x + f - 52), scaled_double<kNeg>(sums.total(1), er[nt].y + f - 52));
+    const long long tt[2] = {sums.total(0), sums.total(1)};
+    const int sc[2] = {er[nt].x + f - 52, er[nt].y + f - 52};
+    double y[2];
+    scaled_doubles<2, kNeg>(tt, sc, y);
+    put(2 * nt, y[0], y[1]);
   }
 }
 
-// This lane's rows 16 r + {2t, 2t+1, 2t+8, 2t+9}, shot g, of vectors and nodal fields.
-// The state of the tensor-core kernels' interior (v, z, q and the gradient accumulators) is in
-// pairs of rows (kPair, n_b even), [row / 2][shot][row % 2]: a lane's two neighbouring rows are
-// one 16-byte access and a warp's are one contiguous range; [row][shot] otherwise.
-template <int kRT, bool kPair>
+// This lane's rows 16 r + {2t, 2t+1, 2t+8, 2t+9}, shot g, of the interior state and of nodal fields.
+// The interior state of the tensor-core kernels (v, z, q and the gradient accumulators) is kept either
+// in whole tiles (kTiles, internal.h): rows and shots beyond n_b and B stay zero, so a lane's two
+// neighbouring rows are one 16-byte access at a constant offset, without a bounds check, and a
+// warp's are one contiguous range; or as the nodal fields are, [row][shot].
+template <int kRT, bool kTiles>
 struct LaneRows {
   static constexpr int kV = 4 * kRT;
   int t2, B;
-  unsigned o0, p0;            // offsets of the lane's first row and first pair
+  unsigned o0, p0;            // offsets of the lane's first row in a nodal field and in the state of a point
   bool ok[kV];
   __device__ __forceinline__ LaneRows(int lane, int nb, int b) : t2(2 * (lane & 3)), B(b) {
     const int g = lane >> 2;
     o0 = (unsigned)(t2 * B + g);
-    p0 = (unsigned)(t2 * B + 2 * g);
+    p0 = kTiles ? (unsigned)(t2 * kCols + 2 * g) : o0;
 #pragma unroll
     for (int j = 0; j < kV; ++j) ok[j] = row(j) < nb && g < B;
   }
   static __device__ __forceinline__ constexpr int rel(int j) { return (j >> 2) * kTile + ((j >> 1) & 1) * 8 + (j & 1); }
   __device__ __forceinline__ int row(int j) const { return t2 + rel(j); }
   __device__ __forceinline__ unsigned off(int j) const { return o0 + (unsigned)(rel(j) * B); }
-  __device__ __forceinline__ unsigned poff(int j) const { return p0 + (unsigned)(rel(j) * B); }      // j even
-  __device__ __forceinline__ void load(const double* p, double (&x)[kV]) const {                     // state
+  // p: the lane's place in the state of a radial point
+  __device__ __forceinline__ void load(const double* p, double (&x)[kV]) const {
 #pragma unroll
     for (int j = 0; j < kV; j += 2) {
-      if (kPair) {
-        const double2 d = ok[j] ? *reinterpret_cast<const double2*>(p + poff(j)) : make_double2(0.0, 0.0);
+      if (kTiles) {
+        const double2 d = *reinterpret_cast<const double2*>(p + rel(j) * kCols);
         x[j] = d.x;
         x[j + 1] = d.y;
       } else {
-        x[j] = ok[j] ? p[off(j)] : 0.0;
-        x[j + 1] = ok[j + 1] ? p[off(j + 1)] : 0.0;
+        x[j] = ok[j] ? p[rel(j) * B] : 0.0;
+        x[j + 1] = ok[j + 1] ? p[rel(j + 1) * B] : 0.0;
       }
     }
   }
   __device__ __forceinline__ void store(double* p, int j, double x0, double x1) const {              // rows of j, j + 1
-    if (kPair) {
-      if (ok[j]) *reinterpret_cast<double2*>(p + poff(j)) = make_double2(x0, x1);
+    if (kTiles) {
+      *reinterpret_cast<double2*>(p + rel(j) * kCols) = make_double2(x0, x1);
     } else {
-      if (ok[j]) p[off(j)] = x0;
-      if (ok[j + 1]) p[off(j + 1)] = x1;
+      if (ok[j]) p[rel(j) * B] = x0;
+      if (ok[j + 1]) p[rel(j + 1) * B] = x1;
     }
   }
 };
@@ -198,7 +205,7 @@ __global__ void slice_operators_kernel(SliceArgs a) {
   } else {
     er = row_exp(h);
   }
-  if (which != 1 && lane < Op::kRows) eout[lane] = er;
+  if (which != 1 && lane < Op::kRows) eout[lane] = er > -1100 ? er : 0;
   for (int nt = 0; nt < 2 * kRT; ++nt) {
     const int ex = __shfl_sync(0xffffffffu, er, nt * 8 + g) + shift;
     for (int kt = 0; kt < kRT; ++kt) {
@@ -219,41 +226,46 @@ __global__ void slice_operators_kernel(SliceArgs a) {
 // P_{n-1}, Q_{n-1}, R, T); a slot is refilled as soon as its last digits are read, so the
 // copies of kSlots operators are in flight ahead of the products, across the turn of the
 // sweeps.  The state of a radial point is loaded before its product.
-template <int kRT, bool kAvgAccel, bool kPair>
-__global__ void __launch_bounds__(32 * tc::Shape<kRT>::kWarps, tc::Shape<kRT>::kBlocks)
+template <int kRT, bool kDeep, bool kTiles, bool kAvgAccel>
+__global__ void __launch_bounds__(32 * tc::Shape<kRT, kDeep>::kWarps, tc::Shape<kRT, kDeep>::kBlocks)
 element_step_tc_kernel(ElemTcArgs a) {
   using namespace tc;
+  constexpr int kSlots = Shape<kRT, kDeep>::kSlots;
   constexpr int kV = 4 * kRT;                 // values per lane
   extern __shared__ __align__(16) unsigned char tc_smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2;
-  const int64_t idx = (int64_t)blockIdx.x * Shape<kRT>::kWarps + warp;
-  if (idx >= a.n_elems) return;               // whole warp leaves together
-  const int64_t e = a.elems ? (int64_t)a.elems[idx] : idx;
-  const int nb = a.nb, n = a.n, B = a.B;
+  const int64_t idx = (int64_t)blockIdx.x * Shape<kRT, kDeep>::kWarps + warp;
+  if (idx >= a.l.n_elems) return;               // whole warp leaves together
+  const int64_t e = a.l.elems ? (int64_t)a.l.elems[idx] : idx;
+  const int nb = a.nb, n = a.n, B = a.l.B;
   const int per = nb * B;
-  Ring<kRT> ring(reinterpret_cast<WarpSmem<kRT>*>(tc_smem)[warp], a.ops + e * (3 * n + 2) * (int64_t)OpBlock<kRT>::kBytes,
-                 n, a.do_down ? 0 : n, a.do_up ? 3 * n + 2 : n);
+  Ring<kRT, kSlots> ring(reinterpret_cast<WarpSmem<kRT, kSlots>*>(tc_smem)[warp],
+                         a.ops + e * (3 * n + 2) * (int64_t)OpBlock<kRT>::kBytes, n, a.l.do_down ? 0 : n,
+                         a.l.do_up ? 3 * n + 2 : n);
   if (lane == 0) ring.start();
   __syncwarp();
-  const LaneRows<kRT, kPair> rows(lane, nb, B);
-  const int64_t base = e * (int64_t)n * per;
+  const LaneRows<kRT, kTiles> rows(lane, nb, B);
+  const int kT = kTiles ? kTile * kRT * kCols : per;          // the state of a radial point
+  const int64_t tile = idx * (int64_t)n * kT + rows.p0;       // the lane's place in that of point 0
+  const float start[4] = {kMagicF, kMagicF, kMagicF, kMagicF};
 
   double x[kV];       // the operand of the next product
-  if (a.do_down) {
+  if (a.l.do_down) {
 #pragma unroll
-    for (int j = 0; j < kV; ++j) x[j] = rows.ok[j] ? a.ub[(int64_t)a.dofs[e * nb + rows.row(j)] * B + g] : 0.0;
-    const bool grad = a.grad_int != nullptr;
+    for (int j = 0; j < kV; ++j) x[j] = rows.ok[j] ? a.l.ub[(int64_t)a.dofs[e * nb + rows.row(j)] * B + g] : 0.0;
+    const bool grad = a.l.grad != nullptr;
     for (int i = n - 1; i >= 0; --i) {
       // the state of this radial point, loaded ahead of the product
-      const int64_t o = base + (unsigned)(i * per);
+      const int64_t p = tile + i * kT;
+      const int64_t o = e * (int64_t)n * per + (unsigned)(i * per);
       double zo[kV], vo[kV], qo[kV], fw[kV], gr[kV];
-      rows.load(a.q + o, qo);
-      rows.load(a.v + o, vo);
-      rows.load(a.ud + o, zo);
+      rows.load(a.l.q + p, qo);
+      rows.load(a.l.v + p, vo);
+      rows.load(a.l.z + p, zo);
       if (grad) {
-        rows.load(a.grad_int + o, gr);
+        rows.load(a.l.grad + p, gr);
 #pragma unroll
-        for (int j = 0; j < kV; ++j) fw[j] = rows.ok[j] ? a.fwd_int[o + rows.off(j)] : 0.0;
+        for (int j = 0; j < kV; ++j) fw[j] = rows.ok[j] ? a.l.fwd_int[o + rows.off(j)] : 0.0;
       }
       int adj;
       const int E = column_scale<kV>(x, adj);
@@ -261,9 +273,9 @@ element_step_tc_kernel(ElemTcArgs a) {
 #pragma unroll
       for (int r = 0; r < kRT; ++r) split_rows(x + 4 * r, E, d[r]);
       const int s0 = ring.slot;
-      ring.wait(s0, a.status);
+      ring.wait(s0, a.l.status);
       product<kRT, 1, false>(
-          ring.frags(s0), nullptr, ring.exps(s0), d, E - 1022 - adj, lane, [&] { ring.template release<1>(lane); },
+          ring.frags(s0), nullptr, ring.exps(s0), d, E - 1022 - adj, lane, start, [&] { ring.template release<1>(lane); },
           [&](int j0, double h0, double h1) {
             double zs[2], vs[2], gs[2];
 #pragma unroll
@@ -285,32 +297,32 @@ element_step_tc_kernel(ElemTcArgs a) {
                 zs[c] = fma(a.c1, uddn, udn);
                 vs[c] = fma(a.a0, u_new, fma(a.a1, udn, a.a2 * uddn));
               }
-              if (a.store_int && rows.ok[j]) a.store_int[o + rows.off(j)] = udn;
+              if (a.l.store_int && rows.ok[j]) a.l.store_int[o + rows.off(j)] = udn;
               if (grad) gs[c] = fma(fw[j], udn, gr[j]);    // dt applied at the end
-              if (a.u_out && rows.ok[j]) a.u_out[o + rows.off(j)] = u_new;
-              x[j] = rows.ok[j] ? u_new : 0.0;
+              if (a.l.u_out && rows.ok[j]) a.l.u_out[o + rows.off(j)] = u_new;
+              x[j] = u_new;                                // zero beyond n_b and B: the operator's rows and q are
             }
-            rows.store(a.ud + o, j0, zs[0], zs[1]);
-            rows.store(a.v + o, j0, vs[0], vs[1]);
-            if (grad) rows.store(a.grad_int + o, j0, gs[0], gs[1]);
+            rows.store(a.l.z + p, j0, zs[0], zs[1]);
+            rows.store(a.l.v + p, j0, vs[0], vs[1]);
+            if (grad) rows.store(a.l.grad + p, j0, gs[0], gs[1]);
           });
     }
   }
-  if (!a.do_up) return;
+  if (!a.l.do_up) return;
   __syncwarp();
   // forward sweep: q_i = -(P_i v_i + Q_i q_{i-1}), as one product -[P | Q 2^-a][v ; q 2^a]: joint
   // row exponents in P's exponent slot, a in Q's
   double v[kV];
-  rows.load(a.v + base, v);
+  rows.load(a.l.v + tile, v);
 #pragma unroll
   for (int j = 0; j < kV; ++j) x[j] = 0.0;    // q of the previous radial point
   for (int i = 0; i < n; ++i) {
-    const int64_t o = base + (unsigned)(i * per);
+    const int64_t p = tile + i * kT;
     double vnext[kV];
-    if (i + 1 < n) rows.load(a.v + o + per, vnext);
+    if (i + 1 < n) rows.load(a.l.v + p + kT, vnext);
     const int s0 = ring.slot, s1 = ring.slot_after(1);
-    ring.wait(s0, a.status);
-    ring.wait(s1, a.status);
+    ring.wait(s0, a.l.status);
+    ring.wait(s1, a.l.status);
     const int bal = *ring.exps(s1);
     int adj;
     const int E = column_scale2<kV>(v, x, bal, adj);
@@ -320,11 +332,12 @@ element_step_tc_kernel(ElemTcArgs a) {
 #pragma unroll
     for (int r = 0; r < kRT; ++r) split_rows(x + 4 * r, max(E - bal, kMinExp), d[kRT + r]);
     product<kRT, 2, true>(
-        ring.frags(s0), ring.frags(s1), ring.exps(s0), d, E - 1022 - adj, lane, [&] { ring.template release<2>(lane); },
+        ring.frags(s0), ring.frags(s1), ring.exps(s0), d, E - 1022 - adj, lane, start,
+        [&] { ring.template release<2>(lane); },
         [&](int j0, double q0, double q1) {
-          rows.store(a.q + o, j0, q0, q1);
-          x[j0] = rows.ok[j0] ? q0 : 0.0;
-          x[j0 + 1] = rows.ok[j0 + 1] ? q1 : 0.0;
+          rows.store(a.l.q + p, j0, q0, q1);
+          x[j0] = q0;
+          x[j0 + 1] = q1;
         });
 #pragma unroll
     for (int j = 0; j < kV; ++j) v[j] = vnext[j];
@@ -335,7 +348,7 @@ element_step_tc_kernel(ElemTcArgs a) {
     v[j] = 0.0;
     if (rows.ok[j]) {
       const int64_t gi = (int64_t)a.dofs[e * nb + rows.row(j)] * B + g;
-      v[j] = fma(a.a0, a.ub[gi], fma(a.a1, a.udb[gi], a.a2 * a.uddb[gi]));
+      v[j] = fma(a.a0, a.l.ub[gi], fma(a.a1, a.l.udb[gi], a.a2 * a.l.uddb[gi]));
     }
   }
   double f[kV];
@@ -348,8 +361,8 @@ element_step_tc_kernel(ElemTcArgs a) {
 #pragma unroll
     for (int r = 0; r < kRT; ++r) split_rows(y + 4 * r, E, d[r]);
     const int s = ring.slot_after(k);
-    ring.wait(s, a.status);
-    product<kRT, 1, false>(ring.frags(s), nullptr, ring.exps(s), d, E - 1022 - adj, lane, [] {},
+    ring.wait(s, a.l.status);
+    product<kRT, 1, false>(ring.frags(s), nullptr, ring.exps(s), d, E - 1022 - adj, lane, start, [] {},
                            [&](int j0, double y0, double y1) {
                              f[j0] = k ? f[j0] + y0 : y0;
                              f[j0 + 1] = k ? f[j0 + 1] + y1 : y1;
@@ -357,10 +370,16 @@ element_step_tc_kernel(ElemTcArgs a) {
   }
 #pragma unroll
   for (int j = 0; j < kV; ++j)
-    if (rows.ok[j]) a.fhat[(e * nb + rows.row(j)) * B + g] = f[j];
+    if (rows.ok[j]) a.l.fhat[(e * nb + rows.row(j)) * B + g] = f[j];
 }
 
 // host side: the digits of every element's operators, and the launch
+template <int kRT, bool kDeep>
+constexpr int tc_block_smem() {
+  using S = tc::Shape<kRT, kDeep>;
+  return (int)sizeof(tc::WarpSmem<kRT, S::kSlots>) * S::kWarps;
+}
+
 template <int kRT>
 int tc_prepare_tiles(Model& md, cudaStream_t st) {
   using namespace tc;
@@ -374,21 +393,30 @@ int tc_prepare_tiles(Model& md, cudaStream_t st) {
   profiler().count(kPhaseSetup);
   SBFWI_CUDA(cudaGetLastError());
   // the slots need more than the default 48 KiB
-  for (const void* f : {(const void*)element_step_tc_kernel<kRT, true, true>, (const void*)element_step_tc_kernel<kRT, true, false>,
-                        (const void*)element_step_tc_kernel<kRT, false, true>, (const void*)element_step_tc_kernel<kRT, false, false>})
-    SBFWI_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(sizeof(WarpSmem<kRT>) * Shape<kRT>::kWarps)));
+  for (const void* f : {(const void*)element_step_tc_kernel<kRT, false, true, true>, (const void*)element_step_tc_kernel<kRT, false, true, false>,
+                        (const void*)element_step_tc_kernel<kRT, false, false, true>, (const void*)element_step_tc_kernel<kRT, false, false, false>})
+    SBFWI_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_block_smem<kRT, false>()));
   return SBFWI_OK;
 }
 
+template <int kRT, bool kDeep>
+void tc_launch_shape(const ElemTcArgs& a, bool avg_accel, cudaStream_t st) {
+  using S = tc::Shape<kRT, kDeep>;
+  const unsigned blocks = (unsigned)((a.l.n_elems + S::kWarps - 1) / S::kWarps);
+  auto launch = [&](auto kernel) { kernel<<<blocks, 32 * S::kWarps, tc_block_smem<kRT, kDeep>(), st>>>(a); };
+  if (a.l.tiles) avg_accel ? launch(element_step_tc_kernel<kRT, kDeep, true, true>) : launch(element_step_tc_kernel<kRT, kDeep, true, false>);
+  else avg_accel ? launch(element_step_tc_kernel<kRT, kDeep, false, true>) : launch(element_step_tc_kernel<kRT, kDeep, false, false>);
+}
+
+// One tile: the deep ring up to 13 elements per SM.  Fused launches, shallow | deep, n_b 16, 8 shots, ms:
+// 3.8 elements per SM (N_r 16) 0.061 | 0.055, 6.7 (N_r 32) 0.142 | 0.130, 10.5 0.177 | 0.173,
+// 12.7 0.215 | 0.210, 15.2 0.224 | 0.240, 20.6 0.348 | 0.371, 27 0.394 | 0.432.
 template <int kRT>
-void tc_launch_tiles(const ElemTcArgs& a, bool avg_accel, bool pair, cudaStream_t st) {
-  using S = tc::Shape<kRT>;
-  const int smem = (int)(sizeof(tc::WarpSmem<kRT>) * S::kWarps);
-  const unsigned blocks = (unsigned)((a.n_elems + S::kWarps - 1) / S::kWarps);
-  auto launch = [&](auto kernel) { kernel<<<blocks, 32 * S::kWarps, smem, st>>>(a); };
-  if (avg_accel) pair ? launch(element_step_tc_kernel<kRT, true, true>) : launch(element_step_tc_kernel<kRT, true, false>);
-  else pair ? launch(element_step_tc_kernel<kRT, false, true>) : launch(element_step_tc_kernel<kRT, false, false>);
+void tc_launch_tiles(const ElemTcArgs& a, bool avg_accel, cudaStream_t st) {
+  if constexpr (kRT == 1) {
+    if (a.l.n_elems <= kFewElements * (int64_t)a.l.sms) return tc_launch_shape<1, true>(a, avg_accel, st);
+  }
+  tc_launch_shape<kRT, false>(a, avg_accel, st);
 }
 
 }  // namespace sbfwi
