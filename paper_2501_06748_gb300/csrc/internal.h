@@ -74,22 +74,39 @@ struct TreeNodeDev {
   int32_t s, b;            // separator size (eliminated here), boundary size (passed up)
   int32_t child0, child1;  // -1 for leaves
   int32_t elem;            // leaf: its element; -1 otherwise
-  int32_t pad;
+  int32_t absorb;          // bit i: child i is merged into this node for the solve (Tree::snodes)
   int64_t sep_off;         // into sep_nodes (s ids) and ysep rows
   int64_t bnd_off;         // into bnd_nodes (b ids) and ybnd rows
   int64_t map_off;         // into map0/map1 (s+b entries)
-  int64_t X_off;           // factor storage: X (s*s) then G (s*b) then C (b*s)
+  int64_t X_off;           // factor storage: X (s*s) then G (s*b) then C (b*s); >= 0: in the model's factors,
+                           // else ~X_off in the set-up workspace
+  int64_t MX_off;          // the same of the node with its absorbed children merged (separator size ms)
+  int32_t ms;
+  int32_t pad;
   int64_t F_off;           // set-up workspace: front (f*f)
   int64_t U_off;           // set-up workspace: update matrix (b*b)
 };
+
+// A node of the solve's tree: a group of the elimination tree's nodes eliminated at once (see
+// group_levels in mesh.cpp)
+struct SolveNode {
+  int32_t s, b;            // separator and boundary sizes
+  int32_t kid0, kids;      // its children with solve tasks: skids[kid0 .. kid0 + kids)
+  int32_t parent, pass;    // pass: an element that eliminates nothing (no task, its parent reads f_hat)
+  int64_t sep_off, bnd_off, map_off, X_off;
+};
+struct Src4 {              // up to four sources of a front position (int4 on the device), see Tree::ssrc
+  int32_t v[4];
+};
+constexpr int32_t kMoreSources = INT32_MIN / 2;
 
 struct Task {               // a row range of one tree node, with the node's fields inline
   int32_t node;
   int32_t r0, r1;
   int32_t ksplit;           // lanes that share one output's dot product (1, 2, 4 or 8)
   int32_t s, b;             // separator and boundary sizes of the node
-  int32_t leaf;             // 1 if the node is an element (front values come from f_hat)
   int32_t pad;              // the node's height (the dataflow trace's phase)
+  int32_t kinds;            // sources of the front's positions: bit 0 f_hat rows, bit 1 ybnd rows
   int64_t sep_off, bnd_off, map_off, X_off;
 };
 
@@ -100,12 +117,21 @@ struct Tree {
   std::vector<int32_t> sep_nodes, bnd_nodes;
   std::vector<int32_t> map0, map1;     // per front position: child0 / child1 bnd index, -1 if absent;
                                        // leaves: map0 = local dof of the element
-  std::vector<int32_t> src0, src1;     // the same for the solve: >= 0 a row of ybnd (a child's
-                                       // boundary); <= -2 the f_hat row -2 - src (element * n_b +
-                                       // local dof) of the leaf's own element or of a child leaf
-                                       // that eliminates nothing (no solve task); -1 absent
   std::vector<std::vector<int32_t>> nodes_at_level;
-  int64_t X_total = 0, F_total = 0, U_total = 0, sep_rows = 0, bnd_rows = 0;
+  int64_t X_total = 0, F_total = 0, U_total = 0;
+  int64_t W_total = 0;                 // set-up workspace for factors that are merged further
+  // the tree of the solve: groups of the nodes above, children before parents
+  std::vector<SolveNode> snodes;
+  std::vector<int32_t> slevel_of;
+  int slevels = 0;
+  std::vector<int32_t> ssep_nodes, sbnd_nodes, skids;
+  // per front position (separator, then boundary) the rows it sums: >= 0 a row of ybnd (a child's
+  // boundary); <= -2 the f_hat row -2 - v (element * n_b + local dof) of an element below; -1 none.  More
+  // than four: the last is kMoreSources - k, and smore[k] counts the rest, which follow it.
+  std::vector<Src4> ssrc;
+  std::vector<int32_t> smore;
+  std::vector<std::vector<int32_t>> snodes_at_level;
+  int64_t sX_total = 0, sep_rows = 0, bnd_rows = 0;
   std::vector<int32_t> sep_owner;      // per global node: tree node that eliminates it
 };
 
@@ -117,7 +143,11 @@ struct Tree {
 struct MeshDevice {
   int device = -1;
   DevBuf xy, ctr, lines, lloc, dofs, xih, xil, tab;
-  DevBuf tree_nodes, sep_nodes, bnd_nodes, map0, map1, src0, src1, level_nodes;
+  DevBuf tree_nodes, map0, map1, level_nodes;
+  DevBuf snodes, ssep, sbnd, ssrc, smore;
+  DevBuf W;                          // factors that are merged further
+  DevBuf fmerge;                     // merge tiles {node, kind, r0, c0} (front_merge_kernel)
+  std::vector<int64_t> fmerge_start; // per level: first tile, first tile of the second phase, end
   std::vector<int64_t> level_start;
   DevBuf F, U;                       // factorisation workspaces
   DevBuf fgemm;                      // front product tiles {node, kind, r0, c0} (front_gemm_kernel)
@@ -173,6 +203,7 @@ struct Mesh {
 };
 
 int build_tree(Mesh& m);
+int build_solve_tree(Mesh& m);
 int ensure_gradient_operator(const Mesh& m, cudaStream_t st);   // MeshDevice::grad_* (setup.cu)
 int lfe_element(const double* E0, const double* E1, const double* E2, const double* M0, int nb, double* K,
                 double* M);                                        // lfe.cpp
@@ -194,8 +225,8 @@ struct LevelTasks {
   int max_level_items = 0;
   size_t block_doubles = 0;                     // largest staging area of a block task
   // the same tasks as one dataflow: items {first task, count, block?, direction} in
-  // topological order, and per tree node [forward tasks | backward tasks | child0 |
-  // child1 | nearest ancestor with backward tasks]
+  // topological order, and per solve node [forward tasks | backward tasks | first child |
+  // children | nearest ancestor with backward tasks], then the children's list
   DevBuf flow_items, node_info;
   int n_items = 0, nodes = 0;
   // the dataflow in up to three launches: items [seg[0], seg[1]) are the lower forward
@@ -227,11 +258,11 @@ struct Model {
   DevBuf S;         // [E][nb][nb]  dynamic stiffness
   DevBuf rho_nodal; // [n_nodal] FP64 (hi part of the set-up value)
   // global factors along the elimination tree, followed by copies of the solve's index
-  // arrays (src0, src1, sep_nodes, bnd_nodes): one range that the per-step solve
+  // arrays (sources, separator and boundary nodes): one range that the per-step solve
   // keeps resident in L2
   DevBuf factors;
-  const int32_t* solve_src0 = nullptr;
-  const int32_t* solve_src1 = nullptr;
+  const int4* solve_src = nullptr;
+  const int32_t* solve_more = nullptr;
   const int32_t* solve_sep = nullptr;
   const int32_t* solve_bnd = nullptr;
   size_t solve_bytes = 0;

@@ -80,6 +80,179 @@ struct Builder {
 
 }  // namespace
 
+// ---------------------------------------------------------------------------
+// the solve's tree
+// ---------------------------------------------------------------------------
+// Each level of the tree costs the per-step solve two dependent passes through L2 (its forward
+// and its backward tasks), whatever its size, and nested dissection makes one level per halving
+// of the mesh.  So consecutive levels are eliminated together where their factors are small: the
+// nodes of a group of levels become one node whose separator is all of theirs, with a dense
+// inverse.  That takes more factor entries (about 1.3 times when pairs of levels are merged on a
+// square mesh, 2 times for threes), so the grouping minimises
+//     kHopUs per level + kEntryUs per factor entry
+// over all partitions of the levels into consecutive ranges, each of at most kMaxMerged levels (an
+// entry's 8 shots at about half the FP64 rate of the device, and the two passes as traced).
+// Solve per step, every level apart | grouped, us: 4 x 4 elements, 1 shot 34 | 16; 24 x 24, 8 shots 135 | 69;
+// 1000 polygons, 2 shots 108 | 50; 64 x 64, 1 shot 152 | 101, 8 shots 222 | 184; 128 x 128, 8 shots (mostly
+// products) 624 | 647; 16^3 cube, 8 shots 922 | 872.  With 9 us and 2e-5 us the small meshes keep a level
+// more (24 x 24: 73, 4 x 4: 23); with 16 us the cube merges a pair of levels too many (930).
+constexpr double kHopUs = 12.0, kEntryUs = 2.4e-5;
+constexpr int kMaxMerged = 5;
+// the staging of a merged front (separator + boundary) fits the solve kernel at four blocks per SM
+constexpr int kMaxMergedFront = 777;
+
+// the group of every level
+static std::vector<int> group_levels(const Tree& t) {
+  const int H = t.levels, T = (int)t.nodes.size();
+  std::vector<int32_t> parent(T, -1);
+  for (int v = 0; v < T; ++v)
+    if (t.nodes[v].child0 >= 0) parent[t.nodes[v].child0] = parent[t.nodes[v].child1] = v;
+  std::vector<double> best(H + 1, 1e300);
+  std::vector<int> from(H + 1, 0);
+  best[0] = 0.0;
+  std::vector<int64_t> ms(T);
+  for (int a = 0; a < H; ++a)
+    for (int b = a; b < std::min(H, a + kMaxMerged); ++b) {
+      double cost = 0.0;
+      bool ok = true, work = false;
+      for (int v = 0; v < T && ok; ++v) {
+        const int h = t.level_of[v];
+        if (h < a || h > b) continue;
+        const TreeNodeDev& r = t.nodes[v];
+        ms[v] = r.s;
+        for (int32_t c : {r.child0, r.child1})
+          if (c >= 0 && t.level_of[c] >= a) ms[v] += ms[c];
+        if (parent[v] >= 0 && t.level_of[parent[v]] <= b) continue;     // not a group root
+        if (ms[v] > r.s && ms[v] + r.b > kMaxMergedFront) ok = false;
+        cost += kEntryUs * (double)(ms[v] * ms[v] + 2 * ms[v] * r.b);
+        if (ms[v] > 0) work = true;
+      }
+      if (!ok) break;                                                  // larger ranges only grow
+      if (work) cost += kHopUs;
+      if (best[a] + cost < best[b + 1]) { best[b + 1] = best[a] + cost; from[b + 1] = a; }
+    }
+  std::vector<int> group(H, 0);
+  for (int e = H, k = H; e > 0; e = from[e], --k)
+    for (int l = from[e]; l < e; ++l) group[l] = k;
+  return group;
+}
+
+int build_solve_tree(Mesh& m) {
+  Tree& t = m.tree;
+  const int T = (int)t.nodes.size();
+  const std::vector<int> group = group_levels(t);
+  std::vector<int32_t> parent(T, -1), solve_of(T, -1);
+  for (int v = 0; v < T; ++v)
+    if (t.nodes[v].child0 >= 0) parent[t.nodes[v].child0] = parent[t.nodes[v].child1] = v;
+  auto absorbed = [&](int v) { return parent[v] >= 0 && group[t.level_of[parent[v]]] == group[t.level_of[v]]; };
+  // factor places: the model's factors for group roots, the set-up workspace for the rest
+  t.W_total = t.sX_total = 0;
+  for (int v = 0; v < T; ++v) {
+    TreeNodeDev& r = t.nodes[v];
+    r.absorb = 0;
+    int64_t ms = r.s;
+    if (r.child0 >= 0) {
+      const int32_t ch[2] = {r.child0, r.child1};
+      for (int i = 0; i < 2; ++i)
+        if (absorbed(ch[i])) { r.absorb |= 1 << i; ms += t.nodes[ch[i]].ms; }
+    }
+    r.ms = (int32_t)ms;
+    auto place = [&](int64_t s, bool final) {
+      int64_t& total = final ? t.sX_total : t.W_total;
+      const int64_t off = total;
+      total += s * s + 2 * s * r.b;
+      return final ? off : ~off;
+    };
+    const bool root = !absorbed(v);
+    r.MX_off = place(ms, root);
+    r.X_off = r.absorb ? place(r.s, false) : r.MX_off;
+  }
+  // nodes, children and sources
+  t.snodes.clear(); t.ssep_nodes.clear(); t.sbnd_nodes.clear(); t.skids.clear(); t.ssrc.clear(); t.smore.clear();
+  t.slevel_of.clear();
+  std::vector<int32_t> pos(m.n_nodes, -1);
+  std::vector<std::vector<int32_t>> src;
+  for (int v = 0; v < T; ++v) {
+    if (absorbed(v)) continue;
+    const TreeNodeDev& r = t.nodes[v];
+    SolveNode n;
+    n.s = r.ms; n.b = r.b;
+    n.kid0 = (int32_t)t.skids.size(); n.kids = 0;
+    n.parent = -1;
+    n.pass = r.elem >= 0 && r.s == 0 ? 1 : 0;
+    n.sep_off = (int64_t)t.ssep_nodes.size();
+    n.bnd_off = (int64_t)t.sbnd_nodes.size();
+    n.map_off = (int64_t)t.ssrc.size();
+    n.X_off = r.MX_off;
+    const int id = (int)t.snodes.size();
+    solve_of[v] = id;
+    // members in the order of the merged separator: absorbed children first, then the node's own
+    std::vector<int32_t> members, kids, leaves;
+    std::vector<std::pair<int32_t, int>> stack = {{v, 0}};
+    while (!stack.empty()) {
+      const auto [u, k] = stack.back();
+      const TreeNodeDev& q = t.nodes[u];
+      if (k < 2 && q.child0 >= 0) {
+        stack.back().second = k + 1;
+        const int32_t c = k == 0 ? q.child0 : q.child1;
+        if (absorbed(c)) stack.push_back({c, 0});
+        else kids.push_back(c);
+      } else {
+        members.push_back(u);
+        if (q.elem >= 0) leaves.push_back(q.elem);
+        stack.pop_back();
+      }
+    }
+    for (int32_t u : members)
+      t.ssep_nodes.insert(t.ssep_nodes.end(), t.sep_nodes.begin() + t.nodes[u].sep_off,
+                          t.sep_nodes.begin() + t.nodes[u].sep_off + t.nodes[u].s);
+    t.sbnd_nodes.insert(t.sbnd_nodes.end(), t.bnd_nodes.begin() + r.bnd_off, t.bnd_nodes.begin() + r.bnd_off + r.b);
+    const int f = n.s + n.b;
+    for (int k = 0; k < n.s; ++k) pos[t.ssep_nodes[n.sep_off + k]] = k;
+    for (int k = 0; k < n.b; ++k) pos[t.sbnd_nodes[n.bnd_off + k]] = n.s + k;
+    if ((int)src.size() < f) src.resize(f);
+    for (int k = 0; k < f; ++k) src[k].clear();
+    int level = 0;
+    auto element = [&](int64_t e) {
+      for (int j = 0; j < m.nbe[e]; ++j) src[pos[m.dofs[e * m.nb + j]]].push_back((int32_t)(-2 - (e * m.nb + j)));
+    };
+    for (int32_t e : leaves) element(e);
+    for (int32_t c : kids) {
+      const SolveNode& q = t.snodes[solve_of[c]];
+      t.snodes[solve_of[c]].parent = id;
+      if (q.pass) {                       // eliminates nothing: its f_hat is read directly
+        element(t.nodes[c].elem);
+        continue;
+      }
+      t.skids.push_back(solve_of[c]);
+      ++n.kids;
+      level = std::max(level, t.slevel_of[solve_of[c]] + 1);
+      for (int k = 0; k < q.b; ++k) src[pos[t.sbnd_nodes[q.bnd_off + k]]].push_back((int32_t)(q.bnd_off + k));
+    }
+    for (int k = 0; k < f; ++k) {
+      Src4 q = {{-1, -1, -1, -1}};
+      const size_t cnt = src[k].size(), direct = cnt > 4 ? 3 : cnt;
+      for (size_t i = 0; i < direct; ++i) q.v[i] = src[k][i];
+      if (cnt > 4) {
+        q.v[3] = kMoreSources - (int32_t)t.smore.size();
+        t.smore.push_back((int32_t)(cnt - 3));
+        t.smore.insert(t.smore.end(), src[k].begin() + 3, src[k].end());
+      }
+      t.ssrc.push_back(q);
+    }
+    t.snodes.push_back(n);
+    t.slevel_of.push_back(level);
+  }
+  t.sep_rows = (int64_t)t.ssep_nodes.size();
+  t.bnd_rows = (int64_t)t.sbnd_nodes.size();
+  if (m.n_elem * m.nb > -(int64_t)kMoreSources - 4 || t.bnd_rows > INT32_MAX)
+    return fail(SBFWI_EUNSUPPORTED, "too many element boundary nodes for the solve's index arrays");
+  t.slevels = 1 + *std::max_element(t.slevel_of.begin(), t.slevel_of.end());
+  t.snodes_at_level.assign(t.slevels, {});
+  for (int k = 0; k < (int)t.snodes.size(); ++k) t.snodes_at_level[t.slevel_of[k]].push_back(k);
+  return SBFWI_OK;
+}
+
 int build_tree(Mesh& m) {
   Tree& t = m.tree;
   t = Tree();
@@ -143,7 +316,6 @@ int build_tree(Mesh& m) {
     r.child0 = bd.c0[nd];
     r.child1 = bd.c1[nd];
     r.elem = (bd.c0[nd] < 0) ? bd.order[bd.lo[nd]] : -1;
-    r.pad = 0;
     r.sep_off = sep_off;
     r.bnd_off = bnd_off;
     r.map_off = map_off;
@@ -166,31 +338,15 @@ int build_tree(Mesh& m) {
         const int32_t j = local.at(g);
         t.map0.push_back(j);
         t.map1.push_back(-1);
-        t.src0.push_back(-2 - (int32_t)(r.elem * m.nb + j));     // the element's own f_hat row
-        t.src1.push_back(-1);
       }
     } else {
       std::map<int32_t, int32_t> in0, in1;
       for (size_t k = 0; k < bnd[r.child0].size(); ++k) in0[bnd[r.child0][k]] = (int32_t)k;
       for (size_t k = 0; k < bnd[r.child1].size(); ++k) in1[bnd[r.child1][k]] = (int32_t)k;
-      const int64_t off0 = t.nodes[r.child0].bnd_off, off1 = t.nodes[r.child1].bnd_off;
-      // a child leaf that eliminates nothing passes its f_hat through unchanged: the
-      // solve reads f_hat directly (encoded -2 - row) and runs no task for it
-      auto src_of = [&](int32_t child, int64_t off, int32_t k, int32_t g) -> int32_t {
-        const TreeNodeDev& c = t.nodes[child];
-        if (c.elem >= 0 && c.s == 0) {
-          int32_t j = 0;
-          while (m.dofs[(int64_t)c.elem * m.nb + j] != g) ++j;
-          return -2 - (int32_t)(c.elem * m.nb + j);
-        }
-        return (int32_t)(off + k);
-      };
       for (int32_t g : front) {
         auto a = in0.find(g), b2 = in1.find(g);
         t.map0.push_back(a == in0.end() ? -1 : a->second);
         t.map1.push_back(b2 == in1.end() ? -1 : b2->second);
-        t.src0.push_back(a == in0.end() ? -1 : src_of(r.child0, off0, a->second, g));
-        t.src1.push_back(b2 == in1.end() ? -1 : src_of(r.child1, off1, b2->second, g));
       }
       t.level_of[nd] = 1 + std::max(t.level_of[r.child0], t.level_of[r.child1]);
     }
@@ -201,10 +357,8 @@ int build_tree(Mesh& m) {
   t.X_total = X_off;
   t.F_total = F_off;
   t.U_total = U_off;
-  t.sep_rows = sep_off;
-  t.bnd_rows = bnd_off;
   if (sep_off != m.n_nodes) return fail(SBFWI_EINVAL, "internal: separators do not cover the nodes");
-  return SBFWI_OK;
+  return build_solve_tree(m);
 }
 
 }  // namespace sbfwi

@@ -841,10 +841,15 @@ struct FactorArgs {
   double* F;                    // workspace fronts
   double* U;                    // workspace update matrices
   double* factors;
+  double* work;                 // factors that are merged further (TreeNodeDev::X_off < 0)
   int* status;
   int products;                 // 1: front_factor_kernel also forms G, C and U (else front_gemm_kernel)
   int big_s;                    // > 0: fronts with s >= big_s are inverted by front_invert_grid_kernel
 };
+
+__device__ __forceinline__ double* factor_at(const FactorArgs& a, int64_t off) {
+  return off >= 0 ? a.factors + off : a.work + ~off;
+}
 
 __global__ void front_assemble_kernel(FactorArgs a) {
   const TreeNodeDev nd = a.nodes[a.level_nodes[blockIdx.x]];
@@ -902,7 +907,7 @@ __global__ void front_factor_kernel(FactorArgs a) {
   const TreeNodeDev nd = a.nodes[a.level_nodes[blockIdx.x]];
   const int s = nd.s, b = nd.b, f = s + b;
   double* F = a.F + nd.F_off;
-  double* X = a.factors + nd.X_off;            // s x s
+  double* X = factor_at(a, nd.X_off);            // s x s
   double* G = X + (int64_t)s * s;              // s x b
   double* C = G + (int64_t)s * b;              // b x s
   double* U = a.U + nd.U_off;                  // b x b
@@ -997,7 +1002,7 @@ __global__ void __launch_bounds__(512) front_invert_grid_kernel(InvertArgs ia) {
   const TreeNodeDev nd = a.nodes[ia.node];
   const int s = nd.s, f = nd.s + nd.b;
   double* F = a.F + nd.F_off;
-  double* X = a.factors + nd.X_off;
+  double* X = factor_at(a, nd.X_off);
   const int tid = threadIdx.x, nt = blockDim.x;
   for (int64_t t = (int64_t)blockIdx.x * nt + tid; t < (int64_t)s * s; t += (int64_t)gridDim.x * nt)
     X[t] = ((t / s) == (t % s)) ? 1.0 : 0.0;
@@ -1081,7 +1086,7 @@ __global__ void __launch_bounds__(256) front_gemm_kernel(FactorArgs a, const int
   const TreeNodeDev nd = a.nodes[it.x];
   const int s = nd.s, b = nd.b, f = s + b;
   const double* F = a.F + nd.F_off;
-  double* X = a.factors + nd.X_off;
+  double* X = factor_at(a, nd.X_off);
   double* G = X + (int64_t)s * s;
   double* C = G + (int64_t)s * b;
   double* U = a.U + nd.U_off;
@@ -1126,12 +1131,109 @@ __global__ void __launch_bounds__(256) front_gemm_kernel(FactorArgs a, const int
   }
 }
 
-// Factors of the transposed global matrix from those of the matrix: the front of a tree node
+// The factors of a node with its absorbed children merged (TreeNodeDev::absorb), from its own (X, G, C
+// of separator size s) and theirs (merged before: X_i, G_i, C_i of size s_i).  With m_i the place of a
+// front position in child i's boundary, the block elimination of [children's separators; own one] gives
+//   X' = [ X_i (i = j) - G_i[:, m_i] X'[p, j] | -G_i[:, m_i] X ]      G' = [ G_i[:, m_i(bnd)] - G_i[:, m_i] G ]
+//        [ -X C_j[m_j, :]                    |  X             ]           [ G                               ]
+//   C' = [ C_i[m_i(bnd), :] - C C_i[m_i, :]  |  C ]
+// as 32 x 32 output tiles, item {node, kind, r0, c0}, kind = block + 8 i + 16 j: 0 X'[p, p], 1 X'[p, i],
+// 2 X'[i, p], 3 C'[:, p], 4 C'[:, i], 5 G'[p, :], 6 G'[i, :], and in a second launch, which reads
+// X'[p, j], 7 X'[i, j].  Forming the merged inverse from the factors this way costs products that fill the
+// grid; inverting the merged separators directly would lengthen the pivot chain of the set-up.
+__global__ void __launch_bounds__(256) front_merge_kernel(FactorArgs a, const int4* items) {
+  __shared__ double As[32][33];
+  __shared__ double Bs[32][33];
+  const int4 it = items[blockIdx.x];
+  const TreeNodeDev nd = a.nodes[it.x];
+  const int kind = it.y & 7, ci = (it.y >> 3) & 1, cj = (it.y >> 4) & 1, r0 = it.z, c0 = it.w;
+  const int s = nd.s, b = nd.b, ms = nd.ms, op = ms - s;
+  const double* X = factor_at(a, nd.X_off);
+  const double* G = X + (int64_t)s * s;
+  const double* C = G + (int64_t)s * b;
+  double* MX = factor_at(a, nd.MX_off);
+  double* MG = MX + (int64_t)ms * ms;
+  double* MC = MG + (int64_t)ms * b;
+  // child i (and j): sizes, factors, place in the merged separator, boundary places of this front
+  const TreeNodeDev ni = a.nodes[ci ? nd.child1 : nd.child0];
+  const int si = ni.ms, bi = ni.b;
+  const int first = (nd.absorb & 1) ? a.nodes[nd.child0].ms : 0;
+  const int oi = ci ? first : 0, oj = cj ? first : 0;
+  const bool child = kind != 0 && kind != 3 && kind != 5;
+  const double* Xi = child ? factor_at(a, ni.MX_off) : nullptr;
+  const double* Gi = child ? Xi + (int64_t)si * si : nullptr;
+  const double* Ci = child ? Gi + (int64_t)si * bi : nullptr;
+  const int32_t* mi = (ci ? a.map1 : a.map0) + nd.map_off;
+  const int sj = kind == 7 ? a.nodes[cj ? nd.child1 : nd.child0].ms : 0;
+  const int M = kind == 0 || kind == 1 || kind == 5 ? s : kind == 3 || kind == 4 ? b : si;
+  const int N = kind == 0 || kind == 2 || kind == 3 ? s : kind == 5 || kind == 6 ? b : kind == 7 ? sj : si;
+  // product A(r, k) B(k, c) over the own separator, subtracted from init(r, c)
+  auto A = [&](int r, int k) -> double {
+    if (kind == 1) return X[(int64_t)r * s + k];
+    if (kind == 4) return C[(int64_t)r * s + k];
+    const int q = mi[k];                                      // 2, 6, 7: G_i[:, m_i]
+    return q >= 0 ? Gi[(int64_t)r * bi + q] : 0.0;
+  };
+  auto B = [&](int k, int c) -> double {
+    if (kind == 2) return X[(int64_t)k * s + c];
+    if (kind == 6) return G[(int64_t)k * b + c];
+    if (kind == 7) return MX[(int64_t)(op + k) * ms + oj + c];
+    const int q = mi[k];                                      // 1, 4: C_i[m_i, :]
+    return q >= 0 ? Ci[(int64_t)q * si + c] : 0.0;
+  };
+  auto init = [&](int r, int c) -> double {
+    if (kind == 0) return X[(int64_t)r * s + c];
+    if (kind == 3) return C[(int64_t)r * s + c];
+    if (kind == 5) return G[(int64_t)r * b + c];
+    if (kind == 4) { const int q = mi[s + r]; return q >= 0 ? Ci[(int64_t)q * si + c] : 0.0; }
+    if (kind == 6) { const int q = mi[s + c]; return q >= 0 ? Gi[(int64_t)r * bi + q] : 0.0; }
+    if (kind == 7) return ci == cj ? Xi[(int64_t)r * si + c] : 0.0;
+    return 0.0;
+  };
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  double acc[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int r = r0 + ty + 8 * j, c = c0 + tx;
+    acc[j] = (r < M && c < N) ? init(r, c) : 0.0;
+  }
+  if (child)
+    for (int k0 = 0; k0 < s; k0 += 32) {
+      for (int t = threadIdx.x; t < 32 * 32; t += 256) {
+        const int i = t >> 5, j = t & 31;
+        As[i][j] = (r0 + i < M && k0 + j < s) ? A(r0 + i, k0 + j) : 0.0;
+        Bs[i][j] = (k0 + i < s && c0 + j < N) ? B(k0 + i, c0 + j) : 0.0;
+      }
+      __syncthreads();
+      const int kn = min(32, s - k0);
+      for (int kk = 0; kk < kn; ++kk) {
+        const double bv = Bs[kk][tx];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j] = fma(-As[ty + 8 * j][kk], bv, acc[j]);
+      }
+      __syncthreads();
+    }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int r = r0 + ty + 8 * j, c = c0 + tx;
+    if (r >= M || c >= N) continue;
+    if (kind <= 2 || kind == 7) {
+      const int rr = (kind == 0 || kind == 1 ? op : oi) + r, cc = (kind == 0 || kind == 2 ? op : kind == 7 ? oj : oi) + c;
+      MX[(int64_t)rr * ms + cc] = acc[j];
+    } else if (kind <= 4) {
+      MC[(int64_t)r * ms + (kind == 3 ? op : oi) + c] = acc[j];
+    } else {
+      MG[(int64_t)((kind == 5 ? op : oi) + r) * b + c] = acc[j];
+    }
+  }
+}
+
+// Factors of the transposed global matrix from those of the matrix: the front of a solve node
 // for A^T is the transpose of its front for A, so X' = F11^{-T} = X^T, G' = X' F21^T = C^T and
 // C' = F12^T X' = G^T (same storage layout: X' s x s, G' s x b, C' b x s).  One block per node.
-__global__ void transpose_factors_kernel(const TreeNodeDev* nodes, int n_nodes, const double* f, double* ft) {
+__global__ void transpose_factors_kernel(const SolveNode* nodes, int n_nodes, const double* f, double* ft) {
   for (int v = blockIdx.x; v < n_nodes; v += gridDim.x) {
-    const TreeNodeDev nd = nodes[v];
+    const SolveNode nd = nodes[v];
     const int s = nd.s, b = nd.b;
     if (s == 0) continue;
     const double* X = f + nd.X_off;
@@ -1240,12 +1342,13 @@ static int ensure_mesh_device(const Mesh& m, cudaStream_t st) {
   if ((rc = upload(d->tab, tab, st))) return rc;
   const Tree& t = m.tree;
   if ((rc = upload(d->tree_nodes, t.nodes, st))) return rc;
-  if ((rc = upload(d->sep_nodes, t.sep_nodes, st))) return rc;
-  if ((rc = upload(d->bnd_nodes, t.bnd_nodes, st))) return rc;
   if ((rc = upload(d->map0, t.map0, st))) return rc;
   if ((rc = upload(d->map1, t.map1, st))) return rc;
-  if ((rc = upload(d->src0, t.src0, st))) return rc;
-  if ((rc = upload(d->src1, t.src1, st))) return rc;
+  if ((rc = upload(d->snodes, t.snodes, st))) return rc;
+  if ((rc = upload(d->ssep, t.ssep_nodes, st))) return rc;
+  if ((rc = upload(d->sbnd, t.sbnd_nodes, st))) return rc;
+  if ((rc = upload(d->ssrc, t.ssrc, st))) return rc;
+  if ((rc = upload(d->smore, t.smore, st))) return rc;
   std::vector<int32_t> all;
   for (int l = 0; l < t.levels; ++l) {
     d->level_start.push_back((int64_t)all.size());
@@ -1284,6 +1387,44 @@ static int ensure_mesh_device(const Mesh& m, cudaStream_t st) {
     if (items.empty()) items.push_back(make_int4(0, 0, 0, 0));
     if ((rc = upload(d->fgemm, items, st))) return rc;
   }
+  {
+    std::vector<int4> items;
+    auto tiles = [&](int32_t nd, int kind, int M, int N) {
+      for (int r0 = 0; r0 < M; r0 += 32)
+        for (int c0 = 0; c0 < N; c0 += 32) items.push_back(make_int4(nd, kind, r0, c0));
+    };
+    for (int l = 0; l < t.levels; ++l) {
+      d->fmerge_start.push_back((int64_t)items.size());
+      for (int32_t nd : t.nodes_at_level[l]) {
+        const TreeNodeDev& r = t.nodes[nd];
+        if (!r.absorb) continue;
+        tiles(nd, 0, r.s, r.s);
+        tiles(nd, 3, r.b, r.s);
+        tiles(nd, 5, r.s, r.b);
+        for (int i = 0; i < 2; ++i) {
+          if (!(r.absorb >> i & 1)) continue;
+          const int si = t.nodes[i ? r.child1 : r.child0].ms;
+          tiles(nd, 1 + 8 * i, r.s, si);
+          tiles(nd, 2 + 8 * i, si, r.s);
+          tiles(nd, 4 + 8 * i, r.b, si);
+          tiles(nd, 6 + 8 * i, si, r.b);
+        }
+      }
+      d->fmerge_start.push_back((int64_t)items.size());
+      for (int32_t nd : t.nodes_at_level[l]) {
+        const TreeNodeDev& r = t.nodes[nd];
+        for (int i = 0; i < 2; ++i)
+          for (int j = 0; j < 2; ++j)
+            if ((r.absorb >> i & 1) && (r.absorb >> j & 1))
+              tiles(nd, 7 + 8 * i + 16 * j, t.nodes[i ? r.child1 : r.child0].ms, t.nodes[j ? r.child1 : r.child0].ms);
+      }
+      d->fmerge_start.push_back((int64_t)items.size());
+    }
+    if (items.empty()) items.push_back(make_int4(0, 0, 0, 0));
+    if ((rc = upload(d->fmerge, items, st))) return rc;
+    SBFWI_CUDA(cudaStreamSynchronize(st));     // items goes out of scope
+  }
+  SBFWI_CUDA(d->W.alloc(sizeof(double) * std::max<int64_t>(t.W_total, 1)));
   SBFWI_CUDA(d->F.alloc(sizeof(double) * std::max<int64_t>(t.F_total, 1)));
   SBFWI_CUDA(d->U.alloc(sizeof(double) * std::max<int64_t>(t.U_total, 1)));
   SBFWI_CUDA(cudaStreamSynchronize(st));     // host vectors above go out of scope
@@ -1622,29 +1763,27 @@ int setup_model(Model& md, const Mesh& m, const double* rho, int mem, cudaStream
   // global factorisation along the elimination tree
   const Tree& t = m.tree;
   {
-    const size_t fb = sizeof(double) * (size_t)std::max<int64_t>(t.X_total, 1);
-    const size_t nmap = t.src0.size(), nsep = t.sep_nodes.size(), nbnd = t.bnd_nodes.size();
-    const size_t ib = sizeof(int32_t) * (2 * nmap + nsep + nbnd);
+    // [factors | sources | separator nodes | boundary nodes | further sources]
+    const size_t fb = sizeof(double) * (size_t)((std::max<int64_t>(t.sX_total, 1) + 1) / 2 * 2);
+    const size_t nsrc = t.ssrc.size(), nsep = t.ssep_nodes.size(), nbnd = t.sbnd_nodes.size(), nmore = t.smore.size();
+    const size_t ib = sizeof(int32_t) * (4 * nsrc + nsep + nbnd + nmore);
     SBFWI_CUDA(md.factors.alloc(fb + ib));
     int32_t* tail = reinterpret_cast<int32_t*>(md.factors.as<char>() + fb);
-    md.solve_src0 = tail;
-    md.solve_src1 = tail + nmap;
-    md.solve_sep = tail + 2 * nmap;
-    md.solve_bnd = tail + 2 * nmap + nsep;
+    md.solve_src = reinterpret_cast<const int4*>(tail);
+    md.solve_sep = tail + 4 * nsrc;
+    md.solve_bnd = md.solve_sep + nsep;
+    md.solve_more = md.solve_bnd + nbnd;
     md.solve_bytes = fb + ib;
-    if (nmap) {
-      SBFWI_CUDA(cudaMemcpyAsync(tail, d.src0.p, sizeof(int32_t) * nmap, cudaMemcpyDeviceToDevice, st));
-      SBFWI_CUDA(cudaMemcpyAsync(tail + nmap, d.src1.p, sizeof(int32_t) * nmap, cudaMemcpyDeviceToDevice, st));
-    }
-    if (nsep) SBFWI_CUDA(cudaMemcpyAsync(tail + 2 * nmap, d.sep_nodes.p, sizeof(int32_t) * nsep, cudaMemcpyDeviceToDevice, st));
-    if (nbnd)
-      SBFWI_CUDA(cudaMemcpyAsync(tail + 2 * nmap + nsep, d.bnd_nodes.p, sizeof(int32_t) * nbnd, cudaMemcpyDeviceToDevice, st));
+    struct Part { const DevBuf& from; size_t at, n; };
+    for (const Part& p : {Part{d.ssrc, 0, 4 * nsrc}, Part{d.ssep, 4 * nsrc, nsep}, Part{d.sbnd, 4 * nsrc + nsep, nbnd},
+                          Part{d.smore, 4 * nsrc + nsep + nbnd, nmore}})
+      if (p.n) SBFWI_CUDA(cudaMemcpyAsync(tail + p.at, p.from.p, sizeof(int32_t) * p.n, cudaMemcpyDeviceToDevice, st));
   }
   {
     FactorArgs a;
     a.nodes = d.tree_nodes.as<TreeNodeDev>(); a.map0 = d.map0.as<int32_t>(); a.map1 = d.map1.as<int32_t>();
     a.S = md.S.as<double>(); a.nb = nb; a.F = d.F.as<double>(); a.U = d.U.as<double>();
-    a.factors = md.factors.as<double>(); a.status = status.as<int>();
+    a.factors = md.factors.as<double>(); a.work = d.W.as<double>(); a.status = status.as<int>();
     // the grid of the cooperative inversion: one block of 512 threads per SM, as many as fit
     DevBuf inv_bar;
     SBFWI_CUDA(inv_bar.alloc(2 * sizeof(unsigned)));
@@ -1684,6 +1823,12 @@ int setup_model(Model& md, const Mesh& m, const double* rho, int mem, cudaStream
         if (u0 > gc0) { front_gemm_kernel<<<(unsigned)(u0 - gc0), 256, 0, st>>>(a, items + gc0); prof.count(kPhaseSetup); }
         if (u1 > u0) { front_gemm_kernel<<<(unsigned)(u1 - u0), 256, 0, st>>>(a, items + u0); prof.count(kPhaseSetup); }
       }
+      for (int ph = 0; ph < 2; ++ph) {
+        const int64_t i0 = d.fmerge_start[3 * l + ph], i1 = d.fmerge_start[3 * l + ph + 1];
+        if (i1 == i0) continue;
+        front_merge_kernel<<<(unsigned)(i1 - i0), 256, 0, st>>>(a, d.fmerge.as<int4>() + i0);
+        prof.count(kPhaseSetup);
+      }
       SBFWI_CUDA(cudaGetLastError());
     }
   }
@@ -1720,9 +1865,9 @@ int prepare_exact(Model& md, cudaStream_t st) {
                                 md.xel.as<double>(), md.kq.as<double>(), status.as<int>(), st);
   if (rc) return rc;
   const Tree& t = m.tree;
-  SBFWI_CUDA(md.factors_t.alloc(sizeof(double) * (size_t)std::max<int64_t>(t.X_total, 1)));
-  const int tn = (int)t.nodes.size();
-  transpose_factors_kernel<<<(unsigned)std::min(tn, 152 * 8), 256, 0, st>>>(m.dev->tree_nodes.as<TreeNodeDev>(), tn,
+  SBFWI_CUDA(md.factors_t.alloc(sizeof(double) * (size_t)std::max<int64_t>(t.sX_total, 1)));
+  const int tn = (int)t.snodes.size();
+  transpose_factors_kernel<<<(unsigned)std::min(tn, 152 * 8), 256, 0, st>>>(m.dev->snodes.as<SolveNode>(), tn,
                                                                            md.factors.as<double>(),
                                                                            md.factors_t.as<double>());
   prof.count(kPhaseSetup);

@@ -146,9 +146,8 @@ __global__ void __launch_bounds__(512) element_step_kernel(ElemStepArgs a) {
 struct SolveArgs {
   const int32_t* sep_nodes;
   const int32_t* bnd_nodes;
-  const int32_t* src0;   // per front position: row of ybnd (or f_hat in a leaf); <= -2: f_hat row -2 - v
-                         // of a pass-through child leaf; -1 absent
-  const int32_t* src1;
+  const int4* src;       // per front position: its sources (Tree::ssrc)
+  const int32_t* more;   // further sources of positions with more than four
   const double* factors;
   const double* fhat;    // [E][nb][B]
   const double* ext;     // [N][B] external sources
@@ -160,17 +159,35 @@ struct SolveArgs {
   int warp_doubles;      // shared memory of one warp task (doubles)
 };
 
-// Sources of a front position: rows of f_hat (r <= -2: the leaf's own element, or a
-// pass-through child leaf) and the external sources are written before the solve
-// starts; rows of ybnd (r >= 0, a child's boundary) are written by other tasks of the
-// same solve (read through L2).  r = -1: absent.  Staging reads the first kind before
-// a task waits for its inputs and only the second kind after the wait.
-__device__ __forceinline__ double fhat_part(const SolveArgs& a, int32_t r, int s) {
-  return r <= -2 ? __ldcg(a.fhat + (int64_t)(-2 - r) * a.B + s) : 0.0;
+// Sources of a front position: rows of f_hat (r <= -2: an element below that no child task sums)
+// and the external sources are written before the solve starts; rows of ybnd (r >= 0, a child's
+// boundary) are written by other tasks of the same solve (read through L2).  r = -1: absent.
+// Staging reads the first kind before a task waits for its inputs and only the second kind
+// after the wait.
+// row of f_hat (kFhat) or ybnd that source r names, 0 for the other kind
+template <bool kFhat>
+__device__ __forceinline__ double source_row(const double* rows, int32_t r, int B, int s) {
+  if (kFhat) return r <= -2 ? __ldcg(rows + (int64_t)(-2 - r) * B + s) : 0.0;
+  return r >= 0 ? __ldcg(rows + (int64_t)r * B + s) : 0.0;
 }
-__device__ __forceinline__ double ybnd_part(const SolveArgs& a, int32_t r, int s) {
-  return r >= 0 ? __ldcg(a.ybnd + (int64_t)r * a.B + s) : 0.0;
+// the further sources of a position with more than four (elements meeting at a node)
+template <bool kFhat>
+__device__ __noinline__ double more_rows(const double* rows, const int32_t* list, int B, int s) {
+  double v = 0.0;
+  for (int k = 1; k <= list[0]; ++k) v += source_row<kFhat>(rows, list[k], B, s);
+  return v;
 }
+template <bool kFhat>
+__device__ __forceinline__ double sources(const SolveArgs& a, const int4& q, int s) {
+  const double* rows = kFhat ? a.fhat : a.ybnd;
+  const double v0 = source_row<kFhat>(rows, q.x, a.B, s), v1 = source_row<kFhat>(rows, q.y, a.B, s);
+  const double v2 = source_row<kFhat>(rows, q.z, a.B, s);
+  const double v3 = q.w <= kMoreSources ? more_rows<kFhat>(rows, a.more + (kMoreSources - q.w), a.B, s)
+                                        : source_row<kFhat>(rows, q.w, a.B, s);
+  return ((v0 + v1) + v2) + v3;
+}
+__device__ __forceinline__ double fhat_part(const SolveArgs& a, const int4& q, int s) { return sources<true>(a, q, s); }
+__device__ __forceinline__ double ybnd_part(const SolveArgs& a, const int4& q, int s) { return sources<false>(a, q, s); }
 
 // t / B for 0 <= t < 2^20: a multiply by floor(2^32 / B) + 1 and the high word (exact in
 // that range for B < 4096), instead of an integer division
@@ -184,6 +201,24 @@ __device__ __forceinline__ double lane_group_sum(double v, int ks) {
   return v;
 }
 
+// n doubles to shared memory, U loads per thread in flight
+template <int U>
+__device__ __forceinline__ void stage_copy(double* dst, const double* src, int n, int tid, int nthr) {
+  for (int base = 0; base < n; base += U * nthr) {
+    double v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int t = base + u * nthr + tid;
+      v[u] = t < n ? src[t] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int t = base + u * nthr + tid;
+      if (t < n) dst[t] = v[u];
+    }
+  }
+}
+
 // Shared-memory staging of a task, U values per thread at a time: all loads of a batch
 // are issued before any of its stores, so the loads of different positions overlap.
 // Every task stages in parts: the constant part (factor rows, index arrays, and the
@@ -193,49 +228,44 @@ __device__ __forceinline__ double lane_group_sum(double v, int ks) {
 //
 // Forward task (rows r0..r1 of the node's boundary):
 //   [front values: c_sep (s B), then c_bnd of the task's rows (rows B) | the task's rows
-//    of C (rows x s) | ybnd source rows of those s + rows positions (2 (s + rows) int32)]
+//    of C (rows x s) | sources of those s + rows positions (int4 each)]
 // c = ext + f_hat parts + ybnd parts, in this order for every schedule.
 struct FwdStage {
   double* vals;
   double* C;
-  int32_t* i0;
-  int32_t* i1;
+  int4* src;
   int P, rows;
 };
 __device__ __forceinline__ FwdStage fwd_layout(const Task& tk, double* sm, int B) {
   FwdStage f;
   f.rows = tk.r1 - tk.r0;
   f.P = tk.s + f.rows;
-  f.vals = sm;
-  f.C = sm + (size_t)f.P * B;
-  f.i0 = reinterpret_cast<int32_t*>(f.C + (size_t)f.rows * tk.s);
-  f.i1 = f.i0 + f.P;
+  f.src = reinterpret_cast<int4*>(sm);
+  f.vals = sm + 2 * (size_t)f.P;
+  f.C = f.vals + (size_t)f.P * B;
   return f;
 }
 
 template <int U>
-__device__ __forceinline__ void fwd_stage_const(const SolveArgs& a, const Task& tk, double* sm, int tid, int nthr) {
+__device__ __forceinline__ void fwd_stage_const(const SolveArgs& a, const Task& tk, double* sm, bool write_ysep, int tid,
+                                                int nthr) {
   const int B = a.B, S = tk.s;
+  const bool fhat = tk.kinds & 1, last = !(tk.kinds & 2);     // last: no ybnd parts follow
   const FwdStage f = fwd_layout(tk, sm, B);
   const double* C = a.factors + tk.X_off + (int64_t)S * S + (int64_t)S * tk.b + (int64_t)tk.r0 * S;
-  const int nv = f.P * B, n = nv + f.rows * S;
-  for (int base = 0; base < n; base += U * nthr) {
+  const int nv = f.P * B, nc = f.rows * S;
+  for (int base = 0; base < nv; base += U * nthr) {
+    int4 q[U];
     double v[U];
-    int32_t q0[U], q1[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int t = base + u * nthr + tid;
+      q[u] = make_int4(-1, -1, -1, -1);
       v[u] = 0.0;
-      q0[u] = -1;
-      q1[u] = -1;
       if (t < nv) {
         const int p = div_shots(a, t), sh = t - p * B;
-        const int pos = p < S ? p : S + tk.r0 + (p - S);
-        q0[u] = a.src0[tk.map_off + pos];
-        q1[u] = a.src1[tk.map_off + pos];
+        q[u] = a.src[tk.map_off + (p < S ? p : tk.r0 + p)];
         if (p < S) v[u] = __ldcg(a.ext + (int64_t)a.sep_nodes[tk.sep_off + p] * B + sh);
-      } else if (t < n) {
-        v[u] = C[t - nv];
       }
     }
 #pragma unroll
@@ -243,25 +273,14 @@ __device__ __forceinline__ void fwd_stage_const(const SolveArgs& a, const Task& 
       const int t = base + u * nthr + tid;
       if (t < nv) {
         const int p = div_shots(a, t), sh = t - p * B;
-        v[u] += fhat_part(a, q0[u], sh);
-        v[u] += fhat_part(a, q1[u], sh);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int t = base + u * nthr + tid;
-      if (t < nv) {
-        const int p = div_shots(a, t), sh = t - p * B;
+        if (fhat) v[u] += fhat_part(a, q[u], sh);
         f.vals[t] = v[u];
-        if (sh == 0) {
-          f.i0[p] = q0[u];
-          f.i1[p] = q1[u];
-        }
-      } else if (t < n) {
-        f.C[t - nv] = v[u];
+        if (last && write_ysep && t < S * B) a.ysep[tk.sep_off * B + t] = v[u];
+        if (!last && sh == 0) f.src[p] = q[u];
       }
     }
   }
+  stage_copy<2 * U>(f.C, C, nc, tid, nthr);
 }
 
 // the ybnd parts (children's boundaries); c_sep also goes to ysep if asked
@@ -270,7 +289,7 @@ __device__ __forceinline__ void fwd_stage_data(const SolveArgs& a, const Task& t
                                                int nthr) {
   const int B = a.B, S = tk.s;
   const FwdStage f = fwd_layout(tk, sm, B);
-  const int nv = f.P * B;
+  const int nv = (tk.kinds & 2) ? f.P * B : 0;
   for (int base = 0; base < nv; base += U * nthr) {
     double y[U];
 #pragma unroll
@@ -279,8 +298,7 @@ __device__ __forceinline__ void fwd_stage_data(const SolveArgs& a, const Task& t
       y[u] = 0.0;
       if (t < nv) {
         const int p = div_shots(a, t), sh = t - p * B;
-        y[u] = ybnd_part(a, f.i0[p], sh);
-        y[u] += ybnd_part(a, f.i1[p], sh);
+        y[u] = ybnd_part(a, f.src[p], sh);
       }
     }
 #pragma unroll
@@ -396,46 +414,31 @@ __device__ __forceinline__ void bwd_stage_data(const SolveArgs& a, const Task& t
 
 // Everything at once, for the schedules that have nothing to wait for (barrier, per
 // level): the same values in the same order of summation as the parts, so every schedule
-// gives the same bits, in one pass of dependent loads (index, then value).
+// gives the same bits.
 template <int U>
 __device__ __forceinline__ void fwd_stage_all(const SolveArgs& a, const Task& tk, double* sm, bool write_ysep, int tid,
                                               int nthr) {
   const int B = a.B, S = tk.s;
   const FwdStage f = fwd_layout(tk, sm, B);
   const double* C = a.factors + tk.X_off + (int64_t)S * S + (int64_t)S * tk.b + (int64_t)tk.r0 * S;
-  const int nv = f.P * B, n = nv + f.rows * S;
-  for (int base = 0; base < n; base += U * nthr) {
-    double v[U], y[U];
+  const int nv = f.P * B;
+  for (int base = 0; base < nv; base += U * nthr) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int t = base + u * nthr + tid;
-      v[u] = 0.0;
-      y[u] = 0.0;
       if (t < nv) {
         const int p = div_shots(a, t), sh = t - p * B;
-        const int pos = p < S ? p : S + tk.r0 + (p - S);
-        const int32_t q0 = a.src0[tk.map_off + pos], q1 = a.src1[tk.map_off + pos];
-        if (p < S) v[u] = __ldcg(a.ext + (int64_t)a.sep_nodes[tk.sep_off + p] * B + sh);
-        v[u] += fhat_part(a, q0, sh);
-        v[u] += fhat_part(a, q1, sh);
-        y[u] = ybnd_part(a, q0, sh);
-        y[u] += ybnd_part(a, q1, sh);
-      } else if (t < n) {
-        v[u] = C[t - nv];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int t = base + u * nthr + tid;
-      if (t < nv) {
-        const double c = v[u] + y[u];
+        const int4 q = a.src[tk.map_off + (p < S ? p : tk.r0 + p)];
+        const double v = p < S ? __ldcg(a.ext + (int64_t)a.sep_nodes[tk.sep_off + p] * B + sh) : 0.0;
+        double c = v;
+        if (tk.kinds & 1) c += fhat_part(a, q, sh);
+        if (tk.kinds & 2) c += ybnd_part(a, q, sh);
         f.vals[t] = c;
         if (write_ysep && t < S * B) a.ysep[tk.sep_off * B + t] = c;
-      } else if (t < n) {
-        f.C[t - nv] = v[u];
       }
     }
   }
+  stage_copy<U>(f.C, C, f.rows * S, tid, nthr);
 }
 
 template <int U>
@@ -559,7 +562,7 @@ __device__ void bwd_compute_warp(const SolveArgs& a, const Task& tk, const doubl
 // tasks end with __syncthreads (the staging area is reused by the block's next task),
 // warp tasks with __syncwarp.
 __device__ void solve_forward_task(const SolveArgs& a, const Task tk, double* sm) {
-  fwd_stage_all<8>(a, tk, sm, tk.r0 == 0, threadIdx.x, blockDim.x);
+  fwd_stage_all<4>(a, tk, sm, tk.r0 == 0, threadIdx.x, blockDim.x);
   __syncthreads();
   fwd_compute_block(a, tk, sm);
   __syncthreads();
@@ -573,7 +576,7 @@ __device__ void solve_backward_task(const SolveArgs& a, const Task tk, double* s
 }
 
 __device__ void solve_forward_warp(const SolveArgs& a, const Task tk, double* sm, int lane) {
-  fwd_stage_all<8>(a, tk, sm, true, lane, 32);
+  fwd_stage_all<4>(a, tk, sm, true, lane, 32);
   __syncwarp();
   fwd_compute_warp(a, tk, sm, lane);
   __syncwarp();
@@ -706,7 +709,8 @@ struct FlowArgs {
   const Task* bwd;
   const int4* items;          // {first task, count, block (1) or warp group (0), direction (0 fwd, 1 bwd)}
   int n_items;
-  const int32_t* node_info;   // [5][nodes]: forward tasks, backward tasks, child0, child1, backward dependency
+  const int32_t* node_info;   // [5][nodes]: forward tasks, backward tasks, first child, children, backward
+                              // dependency; then the list of children
   int nodes;
   unsigned* done_f;           // [nodes] forward tasks completed (cumulative)
   unsigned* done_b;           // [nodes] backward tasks completed (cumulative)
@@ -759,15 +763,19 @@ __device__ bool wait_count(const unsigned* counter, unsigned target, int* status
   return true;
 }
 
-// A forward task reads its children's boundaries: every forward task of both children.
-__device__ bool wait_children(const FlowArgs& a, int node) {
+// A forward task reads its children's boundaries: every forward task of every child (a whole
+// warp: each lane waits for a child)
+__device__ bool wait_children(const FlowArgs& a, int node, int lane) {
   const int T = a.nodes;
   const int32_t* nf = a.node_info;
-  const int ch[2] = {a.node_info[2 * T + node], a.node_info[3 * T + node]};
+  const int32_t* kids = a.node_info + 5 * T + a.node_info[2 * T + node];
+  const int n = a.node_info[3 * T + node];
   bool ok = true;
-  for (int k = 0; k < 2 && ok; ++k)
-    if (ch[k] >= 0) ok = wait_count(a.done_f + ch[k], a.gen * (unsigned)nf[ch[k]], a.status, a.budget);
-  return ok;
+  for (int k = lane; k < n; k += 32) {
+    const int c = kids[k];
+    ok = ok && wait_count(a.done_f + c, a.gen * (unsigned)nf[c], a.status, a.budget);
+  }
+  return __all_sync(0xffffffffu, ok);
 }
 
 // A backward task reads y_sep of its own node (that node's forward tasks) ...
@@ -823,12 +831,15 @@ __global__ void __launch_bounds__(256, 4) solve_flow_kernel(FlowArgs a) {
         __syncthreads();
         bwd_compute_block(a.s, tk, sm_f);
       } else {
-        fwd_stage_const<8>(a.s, tk, sm_f, threadIdx.x, blockDim.x);
-        if (threadIdx.x == 0) s_ok[0] = wait_children(a, tk.node) ? 1 : 0;
+        fwd_stage_const<4>(a.s, tk, sm_f, tk.r0 == 0, threadIdx.x, blockDim.x);
+        if (warp == 0) {
+          const bool ok = wait_children(a, tk.node, lane);
+          if (lane == 0) s_ok[0] = ok ? 1 : 0;
+        }
         __syncthreads();
         if (!s_ok[0]) return;
         if (tr && threadIdx.x == 0) t_ready = global_ns();
-        fwd_stage_data<8>(a.s, tk, sm_f, tk.r0 == 0, threadIdx.x, blockDim.x);
+        fwd_stage_data<4>(a.s, tk, sm_f, tk.r0 == 0, threadIdx.x, blockDim.x);
         __syncthreads();
         fwd_compute_block(a.s, tk, sm_f);
       }
@@ -858,13 +869,12 @@ __global__ void __launch_bounds__(256, 4) solve_flow_kernel(FlowArgs a) {
           bwd_compute_warp(a.s, tk, wsm, lane);
         }
       } else {
-        fwd_stage_const<8>(a.s, tk, wsm, lane, 32);
-        if (lane == 0) ok = wait_children(a, tk.node) ? 1 : 0;
-        ok = __shfl_sync(0xffffffffu, ok, 0);
+        fwd_stage_const<4>(a.s, tk, wsm, true, lane, 32);
+        ok = wait_children(a, tk.node, lane) ? 1 : 0;
         if (ok) {
           if (tr && lane == 0) t_ready = global_ns();
           __syncwarp();
-          fwd_stage_data<8>(a.s, tk, wsm, true, lane, 32);
+          fwd_stage_data<4>(a.s, tk, wsm, true, lane, 32);
           __syncwarp();
           fwd_compute_warp(a.s, tk, wsm, lane);
         }
@@ -1131,16 +1141,18 @@ static int pow2_floor(int v) {
 
 // Small fronts (s <= kWarpS, b <= kWarpB) are warp tasks: one warp does every row.
 static constexpr int kWarpS = 8, kWarpB = 32;
-static bool warp_front(const TreeNodeDev& r) { return r.s <= kWarpS && r.b <= kWarpB; }
+static bool warp_front(const SolveNode& r) { return r.s <= kWarpS && r.b <= kWarpB; }
 // staging area of one warp task: vectors (s + b) B, the factors s (s + b) and the node
-// ids or source rows (at most 2 (s + b) int32)
+// ids or sources (at most 4 (s + b) int32)
 size_t solve_warp_doubles(int B) {
-  return (size_t)(kWarpS + kWarpB) * (B + 1) + (size_t)kWarpS * (kWarpS + kWarpB);
+  return (size_t)(kWarpS + kWarpB) * (B + 2) + (size_t)kWarpS * (kWarpS + kWarpB);
 }
+// the staging area of a block that still runs four to an SM (228 KB, 1 KB of it reserved per block)
+static constexpr size_t kQuarterSm = (57 - 1) * 1024 / sizeof(double) - 16;
 // staging area of a block task (the layouts of fwd_layout / bwd_layout)
 static size_t block_task_doubles(const Task& t, int B, bool fwd) {
   const size_t rows = (size_t)(t.r1 - t.r0);
-  return fwd ? (t.s + rows) * B + rows * t.s + (t.s + rows)
+  return fwd ? (t.s + rows) * (B + 2) + rows * t.s
              : (size_t)(t.s + t.b) * B + rows * (t.s + t.b) + (t.b + rows + 1) / 2;
 }
 
@@ -1155,16 +1167,22 @@ int build_level_tasks(const Model& md, LevelTasks& lt, int B, int grid) {
   // are at most 32 nodes (their factor rows are short, so the staging stays small)
   const int rows_max = std::max(1, 256 / B), rows_max_short = std::max(1, 512 / B);
   const Tree& t = md.mesh->tree;
-  const int L = t.levels;
+  const int L = t.slevels;
   std::vector<Task> fwd, bwd;
   lt.fwd_start.assign(L + 1, 0); lt.bwd_start.assign(L + 1, 0);
   lt.fwd_wstart.assign(L, 0); lt.bwd_wstart.assign(L, 0);
   lt.fwd_group.assign(L, 1); lt.bwd_group.assign(L, 1);
+  std::vector<int32_t> kinds(t.snodes.size(), 0);     // of a node's sources: 1 f_hat rows, 2 ybnd rows
+  for (size_t nd = 0; nd < t.snodes.size(); ++nd) {
+    const SolveNode& r = t.snodes[nd];
+    for (int64_t k = r.map_off; k < r.map_off + r.s + r.b; ++k)
+      for (int32_t q : t.ssrc[k].v) kinds[nd] |= q <= kMoreSources ? 3 : q <= -2 ? 1 : q >= 0 ? 2 : 0;
+  }
   auto task = [&](int32_t nd, int32_t r0, int32_t r1, int ks) {
-    const TreeNodeDev& r = t.nodes[nd];
+    const SolveNode& r = t.snodes[nd];
     Task tk;
     tk.node = nd; tk.r0 = r0; tk.r1 = r1; tk.ksplit = ks;
-    tk.s = r.s; tk.b = r.b; tk.leaf = r.elem >= 0 ? 1 : 0; tk.pad = t.level_of[nd];   // height: the trace's phase
+    tk.s = r.s; tk.b = r.b; tk.pad = t.slevel_of[nd]; tk.kinds = kinds[nd];   // height: the trace's phase
     tk.sep_off = r.sep_off; tk.bnd_off = r.bnd_off; tk.map_off = r.map_off; tk.X_off = r.X_off;
     return tk;
   };
@@ -1182,13 +1200,13 @@ int build_level_tasks(const Model& md, LevelTasks& lt, int B, int grid) {
     lt.bwd_start[l] = (int32_t)bwd.size();
     int64_t rows_f = 0, rows_b = 0;
     int s_max = 0;
-    for (int32_t nd : t.nodes_at_level[l]) {
-      const TreeNodeDev& r = t.nodes[nd];
+    for (int32_t nd : t.snodes_at_level[l]) {
+      const SolveNode& r = t.snodes[nd];
       if (!warp_front(r)) { rows_f += r.b; rows_b += r.s; s_max = std::max(s_max, (int)r.s); }
     }
     const int rf = rows_for(rows_f, s_max <= 32 ? rows_max_short : rows_max), rb = rows_for(rows_b, rows_max);
-    for (int32_t nd : t.nodes_at_level[l]) {
-      const TreeNodeDev& r = t.nodes[nd];
+    for (int32_t nd : t.snodes_at_level[l]) {
+      const SolveNode& r = t.snodes[nd];
       if (warp_front(r)) continue;
       const int kf = lanes_for(rf, r.s), kb = lanes_for(rb, r.s + r.b);
       if (r.b == 0) fwd.push_back(task(nd, 0, 0, 1));
@@ -1197,11 +1215,11 @@ int build_level_tasks(const Model& md, LevelTasks& lt, int B, int grid) {
     }
     lt.fwd_wstart[l] = (int32_t)fwd.size();
     lt.bwd_wstart[l] = (int32_t)bwd.size();
-    for (int32_t nd : t.nodes_at_level[l]) {
-      const TreeNodeDev& r = t.nodes[nd];
+    for (int32_t nd : t.snodes_at_level[l]) {
+      const SolveNode& r = t.snodes[nd];
       if (!warp_front(r)) continue;
       // a leaf that eliminates nothing passes f_hat through (its parent reads f_hat)
-      if (!(r.elem >= 0 && r.s == 0)) fwd.push_back(task(nd, 0, r.b, 1));
+      if (!r.pass) fwd.push_back(task(nd, 0, r.b, 1));
       if (r.s > 0) bwd.push_back(task(nd, 0, r.s, 1));
     }
     lt.fwd_group[l] = group_for((int)fwd.size() - lt.fwd_wstart[l]);
@@ -1229,7 +1247,7 @@ int build_level_tasks(const Model& md, LevelTasks& lt, int B, int grid) {
     // the lower levels whose block tasks fit the warp tasks' staging area run at full
     // occupancy in their own launches; a few large fronts at the top (3-D separators are
     // planes) then no longer hold the whole solve at one block per SM
-    lt.small_doubles = 8 * solve_warp_doubles(B);
+    lt.small_doubles = std::max(8 * solve_warp_doubles(B), kQuarterSm);
     int low = -1;                                  // levels 0..low fit
     for (int l = 0; l < L; ++l) {
       size_t dl = 0;
@@ -1251,21 +1269,18 @@ int build_level_tasks(const Model& md, LevelTasks& lt, int B, int grid) {
     lt.flow_seg[3] = (int)items.size();
     if (low < 0) lt.flow_seg[2] = lt.flow_seg[3];                      // no level fits: one launch
     if (low + 1 >= L) lt.flow_seg[1] = lt.flow_seg[2] = lt.flow_seg[3];   // every level fits: one launch
-    const int T = (int)t.nodes.size();
-    std::vector<int32_t> info(5 * (size_t)T, 0), parent(T, -1);
+    const int T = (int)t.snodes.size();
+    std::vector<int32_t> info(5 * (size_t)T, 0);
     for (const Task& tk : fwd) info[tk.node] += 1;
     for (const Task& tk : bwd) info[T + tk.node] += 1;
     for (int nd = 0; nd < T; ++nd) {
-      info[2 * T + nd] = t.nodes[nd].child0;
-      info[3 * T + nd] = t.nodes[nd].child1;
-      if (t.nodes[nd].child0 >= 0) parent[t.nodes[nd].child0] = nd;
-      if (t.nodes[nd].child1 >= 0) parent[t.nodes[nd].child1] = nd;
-    }
-    for (int nd = 0; nd < T; ++nd) {
-      int a = parent[nd];
-      while (a >= 0 && info[T + a] == 0) a = parent[a];
+      info[2 * T + nd] = t.snodes[nd].kid0;
+      info[3 * T + nd] = t.snodes[nd].kids;
+      int a = t.snodes[nd].parent;
+      while (a >= 0 && info[T + a] == 0) a = t.snodes[a].parent;
       info[4 * T + nd] = a;
     }
+    info.insert(info.end(), t.skids.begin(), t.skids.end());
     SBFWI_CUDA(lt.flow_items.alloc(sizeof(int4) * std::max<size_t>(items.size(), 1)));
     if (!items.empty())
       SBFWI_CUDA(cudaMemcpy(lt.flow_items.p, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice));
@@ -1541,7 +1556,7 @@ int Stepper::init() {
     if (rc) return rc;
   }
   s_smem = sizeof(double) * std::max(lt->block_doubles, 8 * solve_warp_doubles(B));
-  if (s_smem > 200 * 1024) return fail(SBFWI_EUNSUPPORTED, "solve staging area exceeds shared memory");
+  if (s_smem > 226 * 1024) return fail(SBFWI_EUNSUPPORTED, "solve staging area exceeds shared memory");
   for (const void* f : {(const void*)solve_forward_kernel, (const void*)solve_backward_kernel,
                         (const void*)solve_persistent_kernel, (const void*)solve_flow_kernel<false>,
                         (const void*)solve_flow_kernel<true>})
@@ -1575,7 +1590,7 @@ int Stepper::init() {
 
   const MeshDevice& mdev = md.dev();
   sa.sep_nodes = md.solve_sep; sa.bnd_nodes = md.solve_bnd;
-  sa.src0 = md.solve_src0; sa.src1 = md.solve_src1;
+  sa.src = md.solve_src; sa.more = md.solve_more;
   // the exact adjoint solves with the transposed matrix: same tree, transposed factors
   sa.factors = mode == Mode::Exact ? md.factors_t.as<double>() : md.factors.as<double>();
   sa.fhat = rb.fhat.as<double>(); sa.ext = rb.ext.as<double>();
@@ -1614,7 +1629,7 @@ int Stepper::init() {
     pa.s = sa;
     pa.fwd = ftasks; pa.bwd = btasks;
     pa.fwd_meta = lt->fwd_meta.as<int32_t>(); pa.bwd_meta = lt->bwd_meta.as<int32_t>();
-    pa.levels = t.levels;
+    pa.levels = t.slevels;
     pa.bar = bar.as<unsigned>(); pa.status = pstatus.as<int>();
     pa.budget = 4000000000LL;            // ~2 s at 2 GHz
     pa.trace = nullptr;
@@ -1643,7 +1658,7 @@ int Stepper::init() {
     fa.claim = reinterpret_cast<unsigned long long*>(flow_counters.as<char>() + cb);
     fa.status = pstatus.as<int>();
     fa.budget = 4000000000LL;
-    fa.levels = md.mesh->tree.levels;
+    fa.levels = t.slevels;
     fa.trace = nullptr;
     p_grid = flow_grid[0];
     flow_gen = 0;
@@ -1863,7 +1878,7 @@ int Stepper::solve() {
   prof.begin(kPhaseSolve, st);
   if (flow) {
     ++flow_gen;
-    unsigned long long* trace = prof.flow_trace(2 * t.levels, st);
+    unsigned long long* trace = prof.flow_trace(2 * t.slevels, st);
     // up to three launches in stream order (lower forward levels, upper levels, lower backward
     // levels), each claiming its own range of the topologically ordered items
     for (int g = 0; g < 3; ++g) {
@@ -1883,7 +1898,7 @@ int Stepper::solve() {
       prof.count(kPhaseSolve);
     }
   } else if (persistent) {
-    pa.trace = prof.level_trace(6 * t.levels, st);
+    pa.trace = prof.level_trace(6 * t.slevels, st);
     if (pa.trace) ++prof.level_steps;
     void* kargs[] = {&pa};
     int rc = launch_solve((const void*)solve_persistent_kernel, (unsigned)p_grid, kargs, true);
@@ -1891,8 +1906,8 @@ int Stepper::solve() {
     prof.count(kPhaseSolve);
   } else {
     LevelKernelArgs la;
-    la.s = sa; la.levels = t.levels;
-    for (int l = 0; l < t.levels; ++l) {
+    la.s = sa; la.levels = t.slevels;
+    for (int l = 0; l < t.slevels; ++l) {
       const int cnt = lt->items(true, l);
       if (cnt == 0) continue;
       la.tasks = ftasks; la.meta = lt->fwd_meta.as<int32_t>(); la.level = l;
@@ -1901,7 +1916,7 @@ int Stepper::solve() {
       if (rc) return rc;
       prof.count(kPhaseSolve);
     }
-    for (int l = t.levels - 1; l >= 0; --l) {
+    for (int l = t.slevels - 1; l >= 0; --l) {
       const int cnt = lt->items(false, l);
       if (cnt == 0) continue;
       la.tasks = btasks; la.meta = lt->bwd_meta.as<int32_t>(); la.level = l;
