@@ -257,15 +257,16 @@ struct Model {
   DevBuf rt;        // [E][2][nb][nb]
   DevBuf S;         // [E][nb][nb]  dynamic stiffness
   DevBuf rho_nodal; // [n_nodal] FP64 (hi part of the set-up value)
-  // global factors along the elimination tree, followed by copies of the solve's index
-  // arrays (sources, separator and boundary nodes): one range that the per-step solve
-  // keeps resident in L2
+  // the solve tree's factors, followed by copies of the solve's index arrays (sources, separator and
+  // boundary nodes).  They are left to L2's own policy: marking them persisting gained the solve 0.7 %
+  // on the 64 x 64 mesh (45 MB) and took as much from the element kernel, and on larger meshes, whose
+  // factors do not fit, it cost the element kernel a third (96 x 96: 0.98 instead of 0.83 ms a step,
+  // 128 x 128: 2.28 instead of 1.42 ms)
   DevBuf factors;
   const int4* solve_src = nullptr;
   const int32_t* solve_more = nullptr;
   const int32_t* solve_sep = nullptr;
   const int32_t* solve_bnd = nullptr;
-  size_t solve_bytes = 0;
   DevBuf pts_hi, pts_lo; // [n_nodal][dim] dd location of every nodal point
   // the same operators split into FP16 digits for the tensor-core element kernels: one block
   // (digits, row exponents; tc::OpBlock) per operator, [E][P_0 Q_0 H_0 .. H_{n-1} R T]

@@ -1773,7 +1773,6 @@ int setup_model(Model& md, const Mesh& m, const double* rho, int mem, cudaStream
     md.solve_sep = tail + 4 * nsrc;
     md.solve_bnd = md.solve_sep + nsep;
     md.solve_more = md.solve_bnd + nbnd;
-    md.solve_bytes = fb + ib;
     struct Part { const DevBuf& from; size_t at, n; };
     for (const Part& p : {Part{d.ssrc, 0, 4 * nsrc}, Part{d.ssep, 4 * nsrc, nsep}, Part{d.sbnd, 4 * nsrc + nsep, nbnd},
                           Part{d.smore, 4 * nsrc + nsep + nbnd, nmore}})

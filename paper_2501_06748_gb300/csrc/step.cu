@@ -1429,9 +1429,6 @@ struct Stepper {
   ExactElemArgs xa;
   ExactBoundaryArgs xba;
   ExactGradArgs xga;
-  bool use_window = false;
-  cudaAccessPolicyWindow window = {};
-  int setup_l2_window(int device);
   int launch_solve(const void* fn, unsigned grid, void** args, bool cooperative, size_t smem = 0);
   std::vector<DevBuf*> state_bufs() const;
   int element_launch(int down, int up, int64_t done_step);
@@ -1617,8 +1614,6 @@ int Stepper::init() {
   }
   ftasks = lt->fwd.as<Task>();
   btasks = lt->bwd.as<Task>();
-  rc = mode == Mode::Exact ? SBFWI_OK : setup_l2_window(device);   // the window covers the forward factors
-  if (rc) return rc;
   // status word of the bounded device waits (the solve's barriers and counters, the element
   // kernels' copy barriers)
   SBFWI_CUDA(pstatus.alloc(sizeof(int)));
@@ -1706,55 +1701,17 @@ int Stepper::init() {
   return SBFWI_OK;
 }
 
-// The solve reads the same factors and index arrays every step, but the element
-// kernel streams gigabytes through L2 in between and would evict them.  Mark that one
-// range persisting (an access policy window on the solve launches) and, if the
-// context's persisting L2 set-aside is smaller, raise it to cover the range (a limit
-// of this process's context; SBFWI_L2_PERSIST=0 leaves L2 alone).
-int Stepper::setup_l2_window(int device) {
-  use_window = false;
-  const char* env = std::getenv("SBFWI_L2_PERSIST");
-  if (env && std::strcmp(env, "0") == 0) return SBFWI_OK;
-  int max_persist = 0, max_window = 0;
-  if (cudaDeviceGetAttribute(&max_persist, cudaDevAttrMaxPersistingL2CacheSize, device) != cudaSuccess ||
-      cudaDeviceGetAttribute(&max_window, cudaDevAttrMaxAccessPolicyWindowSize, device) != cudaSuccess) {
-    cudaGetLastError();
-    return SBFWI_OK;
-  }
-  if (max_persist <= 0 || max_window <= 0 || md.solve_bytes == 0) return SBFWI_OK;
-  const size_t want = std::min(md.solve_bytes, (size_t)max_persist);
-  size_t cur = 0;
-  SBFWI_CUDA(cudaDeviceGetLimit(&cur, cudaLimitPersistingL2CacheSize));
-  if (cur < want) {
-    SBFWI_CUDA(cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, want));
-    SBFWI_CUDA(cudaDeviceGetLimit(&cur, cudaLimitPersistingL2CacheSize));
-  }
-  if (cur == 0) return SBFWI_OK;
-  window.base_ptr = md.factors.p;
-  window.num_bytes = std::min(md.solve_bytes, (size_t)max_window);
-  window.hitRatio = (float)std::min(1.0, (double)cur / (double)window.num_bytes);
-  window.hitProp = cudaAccessPropertyPersisting;
-  window.missProp = cudaAccessPropertyStreaming;
-  use_window = true;
-  return SBFWI_OK;
-}
-
 int Stepper::launch_solve(const void* fn, unsigned grid, void** args, bool cooperative, size_t smem) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = smem ? smem : s_smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   int na = 0;
   if (cooperative) {
     attr[na].id = cudaLaunchAttributeCooperative;
     attr[na].val.cooperative = 1;
-    ++na;
-  }
-  if (use_window) {
-    attr[na].id = cudaLaunchAttributeAccessPolicyWindow;
-    attr[na].val.accessPolicyWindow = window;
     ++na;
   }
   cfg.attrs = attr;
