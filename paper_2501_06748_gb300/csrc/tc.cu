@@ -65,7 +65,8 @@ int tc_prepare(Model& md, cudaStream_t st) {
 // padded beyond 16 this is the whole operator of its elements with n_b <= 16, whose padded
 // rows and columns are zero)
 int tc_prepare_one_tile(Model& md, cudaStream_t st) {
-  const int rc = tc_prepare_tiles<1>(md, st);
+  int rc = tc_prepare_tiles<1>(md, st);
+  if (rc == SBFWI_OK) rc = tc_small_prepare();
   if (rc) return rc;
   md.tc_ready = true;
   md.tc_one_tile = md.nb > tc::kTile;
@@ -83,7 +84,7 @@ TcState tc_state(const Model& md, int B, int64_t n_elems, int sms) {
   TcState t;
   const int rows = tc_tile_rows(md), nb = md.nb;
   const double most = n_elems <= kFewElements * (int64_t)sms ? 5.4 : rows > tc::kTile ? 2.0 : 1.1;
-  t.tiles = rows * kTileShots <= most * nb * B;
+  t.tiles = rows * kTileShots <= most * nb * B && !(rows == tc::kTile && B <= kFewShots);
   t.doubles = t.tiles ? rows * kTileShots : nb * B;
   return t;
 }
@@ -102,6 +103,7 @@ int tc_element_launch(const Model& md, const TcLaunch& l, cudaStream_t st) {
   // one 16-row tile: n_b <= 16, or the elements of n_b <= 16 of a mesh padded beyond (the
   // one-tile digits of its operators, prepared by tc_prepare_one_tile)
   if (tc_tile_rows(md) > tc::kTile) tc2_element_launch(a, avg, st);
+  else if (l.B <= kFewShots) tc_small_launch(a, avg, st);
   else tc_launch_tiles<1>(a, avg, st);
   return SBFWI_OK;
 }

@@ -397,5 +397,9 @@ constexpr int kFewElements = 13;
 constexpr int kTwoTileMinNb = 21;
 int tc2_prepare(Model& md, cudaStream_t st);
 void tc2_element_launch(const ElemTcArgs& a, bool avg_accel, cudaStream_t st);
+// one or two shots, one tile (tc_small.cu)
+constexpr int kFewShots = 2;
+int tc_small_prepare();
+void tc_small_launch(const ElemTcArgs& a, bool avg_accel, cudaStream_t st);
 
 }  // namespace sbfwi
