@@ -897,6 +897,26 @@ __global__ void barrier_selftest_kernel(unsigned* bar, int* status, long long bu
     if (!grid_barrier(bar, bar + 1, status, budget)) return;
 }
 
+// external sources of one step: forward wavelets at the source nodes, or the
+// time-reversed residuals at the receivers
+struct SourceArgs {
+  double* ext;
+  int B, nsrc;
+  const int64_t* node;
+  const double* values;
+  int64_t stride_src, col;
+  int per_shot;             // one source per shot (node[s]); otherwise nsrc receivers shared by all shots
+};
+__device__ __forceinline__ void put_source(const SourceArgs& a, int t) {
+  const int s = t / a.nsrc, j = t - s * a.nsrc;
+  const int64_t g = a.per_shot ? a.node[s] : a.node[j];
+  a.ext[g * a.B + s] = a.values[(a.per_shot ? (int64_t)s : ((int64_t)s * a.nsrc + j)) * a.stride_src + a.col];
+}
+__global__ void sources_kernel(SourceArgs a) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < a.B * a.nsrc) put_source(a, t);
+}
+
 // ---------------------------------------------------------------------------
 // boundary nodes: Newmark update, receivers, store / gradient
 // ---------------------------------------------------------------------------
@@ -914,6 +934,7 @@ struct BoundaryArgs {
   double* store_ab;       // forward, exact adjoint: accelerations of this step at the boundary nodes [N][B]
   const double* fwd_b;    // adjoint: paired forward velocities [N][B]
   double* grad_b;         // adjoint accumulators [N][B]
+  SourceArgs next;        // the sources of the next step (nsrc = 0: none), which no kernel reads before its solve
 };
 
 __global__ void boundary_update_kernel(BoundaryArgs a) {
@@ -936,18 +957,8 @@ __global__ void boundary_update_kernel(BoundaryArgs a) {
       a.traces[((int64_t)s * a.R + r) * a.K + a.k] = a.x[a.rec[r] * a.B + s];
     }
   }
-}
-
-// external sources of one step: forward wavelets at the source nodes, or the
-// time-reversed residuals at the receivers
-__global__ void sources_kernel(double* ext, int B, int nsrc, const int64_t* node, const double* values,
-                               int64_t stride_src, int64_t col, int per_shot) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= B * nsrc) return;
-  const int s = t / nsrc, j = t - s * nsrc;
-  // per_shot: one source per shot (node[s]); otherwise nsrc receivers shared by all shots
-  const int64_t g = per_shot ? node[s] : node[j];
-  ext[g * B + s] = values[(per_shot ? (int64_t)s : ((int64_t)s * nsrc + j)) * stride_src + col];
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < a.next.B * a.next.nsrc; t += gridDim.x * blockDim.x)
+    put_source(a.next, t);
 }
 
 // ---------------------------------------------------------------------------
@@ -1639,7 +1650,8 @@ int Stepper::init() {
       int per_sm_flow = 0;
       SBFWI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_flow, solve_flow_kernel<true>, 256, flow_smem[g]));
       if (per_sm_flow < 1) return fail(SBFWI_EUNSUPPORTED, "the dataflow solve does not fit on an SM");
-      flow_grid[g] = std::max(1, std::min(per_sm_flow, 4) * sms);   // every block co-resident (cooperative launch)
+      const int items = lt->flow_seg[g + 1] - lt->flow_seg[g];
+      flow_grid[g] = std::max(1, std::min(std::min(per_sm_flow, 4) * sms, items));
     }
     const int T = lt->nodes;
     const size_t cb = ((sizeof(unsigned) * 2 * (size_t)T + 15) / 16) * 16;
@@ -1850,7 +1862,7 @@ int Stepper::solve() {
       f.base = (unsigned long long)(flow_gen - 1) * (unsigned long long)(f.n_items + flow_grid[g]);
       void* kargs[] = {&f};
       int rc = launch_solve(trace ? (const void*)solve_flow_kernel<true> : (const void*)solve_flow_kernel<false>,
-                            (unsigned)flow_grid[g], kargs, true, flow_smem[g]);
+                            (unsigned)flow_grid[g], kargs, false, flow_smem[g]);
       if (rc) return rc;
       prof.count(kPhaseSolve);
     }
@@ -1894,14 +1906,21 @@ int Stepper::run(int64_t k0, int64_t k1) {
   if (k0 > 0 || resume) element_launch(0, 1, k0 - 1);
   for (int64_t k = k0; k < k1; ++k) {
     if (k > k0) element_launch(1, 1, k - 1);
-    // sources of step k
-    if (mode == Mode::Forward) {
-      sources_kernel<<<(B + 127) / 128, 128, 0, st>>>(rb.ext.as<double>(), B, 1, nodes, values, K, k, 1);
-      prof.count(kPhaseOther);
-    } else if (R > 0) {
-      sources_kernel<<<(B * R + 127) / 128, 128, 0, st>>>(rb.ext.as<double>(), B, R, nodes, values, K, K - 1 - k, 0);
+    // sources of the window's first step; the others come with the boundary update before them
+    auto sources = [&](int64_t step) {
+      SourceArgs a = {};
+      a.ext = rb.ext.as<double>(); a.B = B; a.node = nodes; a.values = values; a.stride_src = K;
+      a.per_shot = mode == Mode::Forward ? 1 : 0;
+      a.nsrc = mode == Mode::Forward ? 1 : R;
+      a.col = mode == Mode::Forward ? step : K - 1 - step;
+      return a;
+    };
+    if (k == k0 && (mode == Mode::Forward || R > 0)) {
+      const SourceArgs a = sources(k);
+      sources_kernel<<<(a.B * a.nsrc + 127) / 128, 128, 0, st>>>(a);
       prof.count(kPhaseOther);
     }
+    ba.next = k + 1 < k1 ? sources(k + 1) : SourceArgs{};
     int rc = solve();
     if (rc) return rc;
     ba.k = k;
