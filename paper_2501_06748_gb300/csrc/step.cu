@@ -700,8 +700,9 @@ __global__ void __launch_bounds__(256, 4) solve_persistent_kernel(PersistentSolv
 // forward tasks of its own node and the backward tasks of its nearest ancestor that
 // has any.  Counters are cumulative over the launches of one time loop: after g
 // solves a node has g * n tasks done.  Every dependency of an item lies in an item
-// claimed earlier and all blocks are co-resident, so the earliest unfinished claimed
-// item can always proceed; every wait is still bounded and reports SBFWI_ETIMEOUT.
+// claimed earlier, by a block that runs, so the earliest unfinished claimed item can
+// always proceed, whether or not the other blocks have started (a plain launch); every
+// wait is still bounded and reports SBFWI_ETIMEOUT.
 // ---------------------------------------------------------------------------
 struct FlowArgs {
   SolveArgs s;
@@ -799,6 +800,7 @@ __global__ void __launch_bounds__(256, 4) solve_flow_kernel(FlowArgs a) {
   __shared__ unsigned long long s_tclaim;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr bool tr = kTrace;
+  grid_dependency_wait();
   if (tr && threadIdx.x == 0) atomicMin(a.trace, global_ns());
   for (;;) {
     // a wait that gave up anywhere stops every block at its next claim
@@ -810,7 +812,7 @@ __global__ void __launch_bounds__(256, 4) solve_flow_kernel(FlowArgs a) {
     __syncthreads();
     const long long it = s_item;
     __syncthreads();
-    if (it >= a.n_items) return;
+    if (it >= a.n_items) { grid_launch_next(); return; }
     const int4 im = a.items[it];
     const Task* tasks = im.w ? a.bwd : a.fwd;
     unsigned long long t_ready = tr ? s_tclaim : 0ULL;     // profiling: when the inputs were ready
@@ -913,6 +915,7 @@ __device__ __forceinline__ void put_source(const SourceArgs& a, int t) {
   a.ext[g * a.B + s] = a.values[(a.per_shot ? (int64_t)s : ((int64_t)s * a.nsrc + j)) * a.stride_src + a.col];
 }
 __global__ void sources_kernel(SourceArgs a) {
+  grid_dependency_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < a.B * a.nsrc) put_source(a, t);
 }
@@ -938,6 +941,7 @@ struct BoundaryArgs {
 };
 
 __global__ void boundary_update_kernel(BoundaryArgs a) {
+  grid_dependency_wait();
   const int64_t tot = a.N * a.B;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < tot; t += (int64_t)gridDim.x * blockDim.x) {
     const double un = a.x[t];
@@ -1860,10 +1864,8 @@ int Stepper::solve() {
       f.n_items = i1 - i0;
       f.claim = fa.claim + g;
       f.base = (unsigned long long)(flow_gen - 1) * (unsigned long long)(f.n_items + flow_grid[g]);
-      void* kargs[] = {&f};
-      int rc = launch_solve(trace ? (const void*)solve_flow_kernel<true> : (const void*)solve_flow_kernel<false>,
-                            (unsigned)flow_grid[g], kargs, false, flow_smem[g]);
-      if (rc) return rc;
+      SBFWI_CUDA(launch_next(trace ? solve_flow_kernel<true> : solve_flow_kernel<false>, (unsigned)flow_grid[g], 256,
+                             flow_smem[g], st, f));
       prof.count(kPhaseSolve);
     }
   } else if (persistent) {
@@ -1917,7 +1919,7 @@ int Stepper::run(int64_t k0, int64_t k1) {
     };
     if (k == k0 && (mode == Mode::Forward || R > 0)) {
       const SourceArgs a = sources(k);
-      sources_kernel<<<(a.B * a.nsrc + 127) / 128, 128, 0, st>>>(a);
+      SBFWI_CUDA(launch_next(sources_kernel, (unsigned)(a.B * a.nsrc + 127) / 128, 128, 0, st, a));
       prof.count(kPhaseOther);
     }
     ba.next = k + 1 < k1 ? sources(k + 1) : SourceArgs{};
@@ -1935,7 +1937,7 @@ int Stepper::run(int64_t k0, int64_t k1) {
       ba.fwd_b = fwd + ((K - 1 - k - fwd_k0) * store_stride() + store_bnd_off()) * B;
       ba.grad_b = rb.grad_int.as<double>() + (use_tc ? 0 : nint * B);
     }
-    boundary_update_kernel<<<b_blocks, 256, 0, st>>>(ba);
+    SBFWI_CUDA(launch_next(boundary_update_kernel, b_blocks, 256, 0, st, ba));
     prof.count(kPhaseOther);
   }
   element_launch(1, 0, k1 - 1);

@@ -152,9 +152,10 @@ element_step_small_kernel(ElemTcArgs a) {
   const int per = nb * B;
   Ring<1, kSlots> ring(M.ring, a.ops + e * (3 * n + 2) * (int64_t)OpBlock<1>::kBytes, n, a.l.do_down ? 0 : n,
                        a.l.do_up ? 3 * n + 2 : n);
-  if (lane == 0) ring.start();
+  if (lane == 0) ring.start();                // constant operators
   for (int k = lane; k < (int)(sizeof(M.dig) / 4); k += 32) reinterpret_cast<unsigned*>(M.dig)[k] = 0u;
   __syncwarp();
+  grid_dependency_wait();
   const bool ok = row < nb && s < B;
   const int64_t at = (int64_t)row * B + s;                    // this lane's place in a radial point
   const int64_t st = idx * (int64_t)n * per + at;             // in the state
@@ -255,8 +256,8 @@ static void small_launch(const ElemTcArgs& a, bool avg_accel, cudaStream_t st) {
   constexpr int kWarps = tc::SmallShape<kDeep>::kWarps;
   const int smem = (int)sizeof(tc::SmallSmem<kDeep>) * kWarps;
   const unsigned blocks = (unsigned)((a.l.n_elems + kWarps - 1) / kWarps);
-  if (avg_accel) element_step_small_kernel<kDeep, true><<<blocks, 32 * kWarps, smem, st>>>(a);
-  else element_step_small_kernel<kDeep, false><<<blocks, 32 * kWarps, smem, st>>>(a);
+  if (avg_accel) launch_next(element_step_small_kernel<kDeep, true>, blocks, 32 * kWarps, smem, st, a);
+  else launch_next(element_step_small_kernel<kDeep, false>, blocks, 32 * kWarps, smem, st, a);
 }
 
 void tc_small_launch(const ElemTcArgs& a, bool avg_accel, cudaStream_t st) {

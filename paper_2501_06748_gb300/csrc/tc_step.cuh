@@ -7,6 +7,7 @@
 
 #include "internal.h"
 #include "prof.h"
+#include "sync.cuh"
 #include "tc_digits.cuh"
 
 namespace sbfwi {
@@ -242,8 +243,9 @@ element_step_tc_kernel(ElemTcArgs a) {
   Ring<kRT, kSlots> ring(reinterpret_cast<WarpSmem<kRT, kSlots>*>(tc_smem)[warp],
                          a.ops + e * (3 * n + 2) * (int64_t)OpBlock<kRT>::kBytes, n, a.l.do_down ? 0 : n,
                          a.l.do_up ? 3 * n + 2 : n);
-  if (lane == 0) ring.start();
+  if (lane == 0) ring.start();                // constant operators
   __syncwarp();
+  grid_dependency_wait();
   const LaneRows<kRT, kTiles> rows(lane, nb, B);
   const int kT = kTiles ? kTile * kRT * kCols : per;          // the state of a radial point
   const int64_t tile = idx * (int64_t)n * kT + rows.p0;       // the lane's place in that of point 0
@@ -403,7 +405,7 @@ template <int kRT, bool kDeep>
 void tc_launch_shape(const ElemTcArgs& a, bool avg_accel, cudaStream_t st) {
   using S = tc::Shape<kRT, kDeep>;
   const unsigned blocks = (unsigned)((a.l.n_elems + S::kWarps - 1) / S::kWarps);
-  auto launch = [&](auto kernel) { kernel<<<blocks, 32 * S::kWarps, tc_block_smem<kRT, kDeep>(), st>>>(a); };
+  auto launch = [&](auto kernel) { launch_next(kernel, blocks, 32 * S::kWarps, tc_block_smem<kRT, kDeep>(), st, a); };
   if (a.l.tiles) avg_accel ? launch(element_step_tc_kernel<kRT, kDeep, true, true>) : launch(element_step_tc_kernel<kRT, kDeep, true, false>);
   else avg_accel ? launch(element_step_tc_kernel<kRT, kDeep, false, true>) : launch(element_step_tc_kernel<kRT, kDeep, false, false>);
 }
