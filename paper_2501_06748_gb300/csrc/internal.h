@@ -65,6 +65,7 @@ struct DevBuf {
 cudaError_t store_alloc(DevBuf& b, size_t bytes);
 void store_release(DevBuf& b);
 void store_cache_clear();
+void misfit_pool_clear();      // the misfit calls' idle scratch (step.cu)
 
 // ---------------------------------------------------------------------------
 // elimination tree of the global boundary system (nested dissection by

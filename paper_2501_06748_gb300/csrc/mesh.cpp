@@ -560,6 +560,7 @@ int sbfwi_profile_solve_flow(double* us, int32_t cap, int32_t* n_slots, int64_t*
 
 int sbfwi_release_cache(void) {
   store_cache_clear();
+  misfit_pool_clear();
   return SBFWI_OK;
 }
 
