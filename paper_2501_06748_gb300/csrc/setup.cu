@@ -283,7 +283,8 @@ struct ElemArgs {
   int64_t e0;                 // first element of this launch
   const int32_t* nbe;         // [E] n_b of each element
   const int64_t* lptr;        // [E+1] first line of each element
-  dd* mat_ws;                 // global workspace for the 16 matrices (nullptr: shared memory)
+  dd* mat_ws;                 // global workspace for the kSetupMats matrices (nullptr: shared memory)
+  int scratch;                // dd entries of the area that ElemSmem::Eline shares with th, ph, ps, Gm
   double* E_out;              // comparison method: E0, E1, E2, M0 of radial point 0 [E][4][nb][nb], then stop
   int64_t n_elem, n_int;
   double c;
@@ -316,13 +317,15 @@ struct ElemSmem {
               // c^2 w det (b2.b2), w det.  3-D: c^2 w det times b1.b1, b2.b1, b3.b1, b2.b2,
               // b2.b3, b3.b3, then w det
   dd* KR;     // [L][ng][nk] the same times rho at the Gauss point
+  dd* prod;   // (2-D) [3][ng][fpp][fpp] products phi phi, dphi phi, dphi dphi
   dd* Eline;  // [L][fpp][fpp][4] per-line (face) contributions
   dd* phi;    // [ng][fpp]
   dd* dphi;   // [ng][fpp]
   dd* dphz;   // [ng][fpp] (3-D)
-  dd* mat;    // 16 matrices of n_b(e)^2 (placed nb*nb apart)
-  dd* col;    // [nb] Gauss-Jordan factor column
-  int* piv;
+  dd* mat;    // 11 matrices of n_b(e)^2 (placed nb*nb apart); th, ph, ps and Gm follow in the scratch area
+  dd* row;    // [nb] Gauss-Jordan pivot row
+  int* piv;   // pivot row, then [nb] the columns of the inverse
+  signed char* loc;   // [L][nb] position of a boundary node on a line (face), -1 if it is not on it
   int nb, L;  // this element's boundary nodes and lines
   int64_t l0; // its first line
 };
@@ -345,6 +348,18 @@ struct DDOps {
   static __device__ __forceinline__ dd fma(dd acc, dd x, dd y) { return dd_fma(acc, x, y); }
   static __device__ __forceinline__ dd div(dd x, dd y) { return dd_div(x, y); }
   static __device__ __forceinline__ dd neg(dd x) { return dd_neg(x); }
+  // Terms of a sum: the high parts by TwoSum, all errors in the low part (the compensated dot product of
+  // Ogita, Rump and Oishi with the low parts' products): 12 operations, against 28 of fma, for an error of
+  // n^2 2^-106 sum |x y|.  norm makes the sum a dd.
+  static __device__ __forceinline__ dd mac(dd acc, dd x, dd y) {
+    const double p = __dmul_rn(x.hi, y.hi);
+    const double e = ::fma(x.lo, y.hi, ::fma(x.hi, y.lo, ::fma(x.hi, y.hi, -p)));
+    const dd s = two_sum(acc.hi, p);
+    return dd{s.hi, acc.lo + (s.lo + e)};
+  }
+  static __device__ __forceinline__ dd norm(dd x) { return fast_two_sum(x.hi, x.lo); }
+  // a - x y
+  static __device__ __forceinline__ dd fms(dd a, dd x, dd y) { return norm(mac(a, neg(x), y)); }
 };
 struct F64Ops {
   static __device__ __forceinline__ dd make(double a) { return dd{a, 0.0}; }
@@ -355,9 +370,24 @@ struct F64Ops {
   static __device__ __forceinline__ dd fma(dd acc, dd x, dd y) { return dd{::fma(x.hi, y.hi, acc.hi), 0.0}; }
   static __device__ __forceinline__ dd div(dd x, dd y) { return dd{x.hi / y.hi, 0.0}; }
   static __device__ __forceinline__ dd neg(dd x) { return dd{-x.hi, 0.0}; }
+  static __device__ __forceinline__ dd mac(dd acc, dd x, dd y) { return fma(acc, x, y); }
+  static __device__ __forceinline__ dd norm(dd x) { return x; }
+  static __device__ __forceinline__ dd fms(dd a, dd x, dd y) { return dd{::fma(-x.hi, y.hi, a.hi), 0.0}; }
 };
+constexpr int kSetupMats = 15;       // working matrices of the element set-up
 constexpr int kExtendedPoints = 4;   // coefficient matrices of points 0..3 in double-double
 constexpr int kExtendedRows = 2;     // rows 0, 1 of the condensation in double-double
+
+// ElemSmem::prod
+template <class Op>
+__device__ void shape_products(const ElemArgs& a, const ElemSmem& sm) {
+  const int ng = a.ng, pp = a.fpp;
+  for (int t = threadIdx.x; t < 3 * ng * pp * pp; t += blockDim.x) {
+    const int k = t / (ng * pp * pp), gab = t - k * ng * pp * pp, g = gab / (pp * pp), ab = gab - g * pp * pp;
+    const int aa = g * pp + ab / pp, bb = g * pp + ab % pp;
+    sm.prod[t] = Op::mul(k == 0 ? sm.phi[aa] : sm.dphi[aa], k == 2 ? sm.dphi[bb] : sm.phi[bb]);
+  }
+}
 
 // E0, E1, E2, M0 of element e at radial point i into the four given matrices
 template <class Op>
@@ -372,39 +402,38 @@ __device__ void coefficient_matrices(const ElemArgs& a, const ElemSmem& sm, int6
     for (int q = 0; q < pp; ++q) {
       const int j = a.line_local[(sm.l0 + l) * pp + q];
       const int64_t idx = (i < a.n) ? e * (int64_t)a.n * nbs + (int64_t)i * nbs + j : a.n_int + a.dofs[e * nbs + j];
-      r = Op::fma(r, sm.phi[g * pp + q], ldd(a.rho_hi, a.rho_lo, idx));
+      r = Op::mac(r, sm.phi[g * pp + q], ldd(a.rho_hi, a.rho_lo, idx));
     }
+    r = Op::norm(r);
     for (int k = 0; k < nk; ++k) sm.KR[(l * ng + g) * nk + k] = Op::mul(sm.K[(l * ng + g) * nk + k], r);
   }
   __syncthreads();
-  // per-line (face) matrices: sum over Gauss points
-  for (int t = tid; t < L * pp * pp; t += nt) {
-    const int l = t / (pp * pp), ab = t - l * pp * pp, aa = ab / pp, bb = ab - aa * pp;
-    dd s0 = Op::make(0.0), s1 = s0, s2 = s0, sm0 = s0;
-    for (int g = 0; g < ng; ++g) {
-      const dd* kr = sm.KR + (l * ng + g) * nk;
-      const dd pa = sm.phi[g * pp + aa], pb = sm.phi[g * pp + bb];
-      const dd da = sm.dphi[g * pp + aa], db = sm.dphi[g * pp + bb];
-      const dd papb = Op::mul(pa, pb);
-      s0 = Op::fma(s0, kr[0], papb);
-      if (a.dim == 2) {
-        s1 = Op::fma(s1, kr[1], Op::mul(da, pb));
-        s2 = Op::fma(s2, kr[2], Op::mul(da, db));
-        sm0 = Op::fma(sm0, kr[3], papb);
-      } else {
+  // per-line (face) matrices: sum over Gauss points, one thread per entry of one matrix
+  for (int t = tid; t < L * pp * pp * 4; t += nt) {
+    const int k = t & 3, lab = t >> 2, l = lab / (pp * pp), ab = lab - l * pp * pp, aa = ab / pp, bb = ab - aa * pp;
+    dd s = Op::make(0.0);
+    if (a.dim == 2) {
+      const dd* tab = sm.prod + (k == 3 ? 0 : k) * ng * pp * pp + ab;
+      for (int g = 0; g < ng; ++g) s = Op::mac(s, sm.KR[(l * ng + g) * nk + k], tab[g * pp * pp]);
+    } else {
+      for (int g = 0; g < ng; ++g) {
+        const dd* kr = sm.KR + (l * ng + g) * nk;
+        const dd pa = sm.phi[g * pp + aa], pb = sm.phi[g * pp + bb];
+        const dd da = sm.dphi[g * pp + aa], db = sm.dphi[g * pp + bb];
         // B2 = b2 N_eta + b3 N_zeta: E1 += (b2.b1 N_eta,a + b3.b1 N_zeta,a) N_b,
         // E2 += b2.b2 N_eta,a N_eta,b + b2.b3 (N_eta,a N_zeta,b + N_zeta,a N_eta,b) + b3.b3 N_zeta,a N_zeta,b
         const dd za = sm.dphz[g * pp + aa], zb = sm.dphz[g * pp + bb];
-        s1 = Op::fma(s1, Op::add(Op::mul(kr[1], da), Op::mul(kr[2], za)), pb);
-        dd q2 = Op::mul(kr[3], Op::mul(da, db));
-        q2 = Op::fma(q2, kr[4], Op::add(Op::mul(da, zb), Op::mul(za, db)));
-        q2 = Op::fma(q2, kr[5], Op::mul(za, zb));
-        s2 = Op::add(s2, q2);
-        sm0 = Op::fma(sm0, kr[6], papb);
+        if (k == 0 || k == 3) s = Op::mac(s, kr[2 * k], Op::mul(pa, pb));
+        else if (k == 1) s = Op::mac(s, Op::add(Op::mul(kr[1], da), Op::mul(kr[2], za)), pb);
+        else {
+          dd q2 = Op::mul(kr[3], Op::mul(da, db));
+          q2 = Op::fma(q2, kr[4], Op::add(Op::mul(da, zb), Op::mul(za, db)));
+          q2 = Op::fma(q2, kr[5], Op::mul(za, zb));
+          s = Op::add(s, q2);
+        }
       }
     }
-    dd* out = sm.Eline + (size_t)t * 4;
-    out[0] = s0; out[1] = s1; out[2] = s2; out[3] = sm0;
+    sm.Eline[t] = Op::norm(s);
   }
   __syncthreads();
   // assemble the element matrices from the lines (faces)
@@ -412,12 +441,7 @@ __device__ void coefficient_matrices(const ElemArgs& a, const ElemSmem& sm, int6
     const int A = t / nb, B = t - A * nb;
     dd s0 = Op::make(0.0), s1 = s0, s2 = s0, s3 = s0;
     for (int l = 0; l < L; ++l) {
-      int pa = -1, pb = -1;
-      for (int q = 0; q < pp; ++q) {
-        const int j = a.line_local[(sm.l0 + l) * pp + q];
-        if (j == A) pa = q;
-        if (j == B) pb = q;
-      }
+      const int pa = sm.loc[l * nb + A], pb = sm.loc[l * nb + B];
       if (pa < 0 || pb < 0) continue;
       const dd* v = sm.Eline + ((size_t)(l * pp + pa) * pp + pb) * 4;
       s0 = Op::add(s0, v[0]); s1 = Op::add(s1, v[1]); s2 = Op::add(s2, v[2]); s3 = Op::add(s3, v[3]);
@@ -427,52 +451,77 @@ __device__ void coefficient_matrices(const ElemArgs& a, const ElemSmem& sm, int6
   __syncthreads();
 }
 
-// Inv = A^{-1} by Gauss-Jordan with partial pivoting; A is destroyed.
+// Warp 0: the pivot of column k of M (its first largest entry from row k on), the pivot row divided by it,
+// with the inverse of the pivot in column k, and the column of the inverse that column k will hold.
 template <class Op>
-__device__ void gj_inverse(int nb, dd* A, dd* Inv, dd* col, int* piv, int* status) {
+__device__ void gj_pivot(int nb, int k, const dd* M, dd* row, int* piv, int* status) {
+  const int lane = threadIdx.x;
+  unsigned long long bv = 0;
+  int best = k;
+  for (int r = k + lane; r < nb; r += 32) {
+    const double v = fabs(M[r * nb + k].hi);
+    // NaN: nothing below it, but chosen on the diagonal, where it is reported
+    const unsigned long long key = v == v ? (unsigned long long)__double_as_longlong(v) + 1 : r == k ? ~0ULL : 0ULL;
+    if (key > bv) { bv = key; best = r; }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long ov = __shfl_xor_sync(0xffffffffu, bv, o);
+    const int ob = __shfl_xor_sync(0xffffffffu, best, o);
+    if (ov > bv || (ov == bv && ob < best)) { bv = ov; best = ob; }
+  }
+  const dd p = M[best * nb + k];
+  if (lane == 0) {
+    if (!(fabs(p.hi) > 0.0) || !isfinite(p.hi)) atomic_flag(status, SBFWI_ESINGULAR);
+    piv[0] = best;
+    const int o = piv[1 + best];
+    piv[1 + best] = piv[1 + k];
+    piv[1 + k] = o;
+  }
+  const dd pinv = Op::div(Op::make(1.0), p);
+  for (int c = lane; c < nb; c += 32) row[c] = c == k ? pinv : Op::mul(M[best * nb + c], pinv);
+}
+
+// Inv = A^{-1} by Gauss-Jordan with partial pivoting, in place: column k of the identity takes the place of
+// column k of A as it is eliminated, so a step is one multiply-add per entry (of [A | I] it was two, and as
+// many products with the unnormalised pivot row); each step writes the other of the two matrices, with the
+// row exchange in its indices.  A and Inv are exchanged where that leaves the result in A; A is destroyed.
+template <class Op>
+__device__ void gj_inverse(int nb, dd*& A, dd*& Inv, dd* row, int* piv, int* status) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int t = tid; t < nb * nb; t += nt) Inv[t] = Op::make((t / nb) == (t % nb) ? 1.0 : 0.0);
+  dd *src = A, *dst = Inv;
+  if (tid < 32) {
+    for (int c = tid; c < nb; c += 32) piv[1 + c] = c;
+    __syncwarp();
+    gj_pivot<Op>(nb, 0, src, row, piv, status);
+  }
   __syncthreads();
   for (int k = 0; k < nb; ++k) {
-    if (tid == 0) {
-      int best = k;
-      double bv = fabs(A[k * nb + k].hi);
-      for (int r = k + 1; r < nb; ++r) {
-        const double v = fabs(A[r * nb + k].hi);
-        if (v > bv) { bv = v; best = r; }
-      }
-      if (!(bv > 0.0) || !isfinite(bv)) atomic_flag(status, SBFWI_ESINGULAR);
-      *piv = best;
-    }
-    __syncthreads();
-    const int pr = *piv;
-    if (pr != k) {
-      for (int c = tid; c < nb; c += nt) {
-        dd t1 = A[k * nb + c]; A[k * nb + c] = A[pr * nb + c]; A[pr * nb + c] = t1;
-        dd t2 = Inv[k * nb + c]; Inv[k * nb + c] = Inv[pr * nb + c]; Inv[pr * nb + c] = t2;
-      }
-    }
-    __syncthreads();
-    for (int r = tid; r < nb; r += nt) col[r] = A[r * nb + k];
-    __syncthreads();
-    const dd pinv = Op::div(Op::make(1.0), col[k]);
+    const int pr = piv[0];
     for (int t = tid; t < nb * nb; t += nt) {
       const int r = t / nb, c = t - r * nb;
-      // row k is only read here; it is normalised after the barrier below
-      const dd ak = Op::mul(A[k * nb + c], pinv), ik = Op::mul(Inv[k * nb + c], pinv);
+      dd v = row[c];
       if (r != k) {
-        const dd f = col[r];
-        A[t] = Op::sub(A[t], Op::mul(f, ak));
-        Inv[t] = Op::sub(Inv[t], Op::mul(f, ik));
+        const int from = r == pr ? k : r;
+        v = Op::fms(c == k ? Op::make(0.0) : src[from * nb + c], src[from * nb + k], v);
       }
+      dst[t] = v;
     }
     __syncthreads();
-    for (int c = tid; c < nb; c += nt) {
-      A[k * nb + c] = Op::mul(A[k * nb + c], pinv);
-      Inv[k * nb + c] = Op::mul(Inv[k * nb + c], pinv);
+    dd* const s = src;
+    src = dst;
+    dst = s;
+    if (k + 1 < nb) {
+      if (tid < 32) gj_pivot<Op>(nb, k + 1, src, row, piv, status);
+      __syncthreads();
     }
-    __syncthreads();
   }
+  for (int t = tid; t < nb * nb; t += nt) {
+    const int r = t / nb, c = t - r * nb;
+    dst[r * nb + piv[1 + c]] = src[t];
+  }
+  __syncthreads();
+  A = src;
+  Inv = dst;
 }
 
 // C = A * B (all nb x nb, distinct buffers)
@@ -481,13 +530,20 @@ __device__ void mm(int nb, const dd* A, const dd* B, dd* C) {
   for (int t = threadIdx.x; t < nb * nb; t += blockDim.x) {
     const int r = t / nb, c = t - r * nb;
     dd s = Op::make(0.0);
-    for (int k = 0; k < nb; ++k) s = Op::fma(s, A[r * nb + k], B[k * nb + c]);
-    C[t] = s;
+    for (int k = 0; k < nb; ++k) s = Op::mac(s, A[r * nb + k], B[k * nb + c]);
+    C[t] = Op::norm(s);
   }
   __syncthreads();
 }
 
-__global__ void element_setup_kernel(ElemArgs a) {
+// Bound by the FP64 pipe (2 operations per clock and SM): 77 % of it busy, 21 ms for 4096 elements of
+// 16 boundary nodes and 32 radial points (54 ms before), three quarters of the operations in the
+// eliminations and products of the binary64 points.  So operations are what is saved: eliminations in
+// place (1 instead of 4 per entry and step), extended sums by compensated dot products (12 instead of
+// 28 a term), the shape functions' products formed once.  The 15 working matrices leave room for three
+// blocks per SM at 80 registers (with 96, two blocks: 24 ms); one block barrier per elimination step is
+// for warp 0, which finds the next pivot.
+__global__ void __launch_bounds__(768) element_setup_kernel(ElemArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int64_t e = a.e0 + blockIdx.x;
   const int ng = a.ng, pp = a.fpp, nk = a.nk, n = a.n, nbs = a.nb;
@@ -500,29 +556,39 @@ __global__ void element_setup_kernel(ElemArgs a) {
   dd* base = reinterpret_cast<dd*>(smem_raw);
   sm.K = base;                     base += a.L * ng * nk;
   sm.KR = base;                    base += a.L * ng * nk;
-  sm.Eline = base;                 base += a.L * pp * pp * 4;
   sm.phi = base;                   base += ng * pp;
   sm.dphi = base;                  base += ng * pp;
   sm.dphz = base;                  base += a.dim == 3 ? ng * pp : 0;
-  sm.col = base;                   base += nbs;
+  sm.row = base;                   base += nbs;
+  sm.prod = base;                  base += a.dim == 2 ? 3 * ng * pp * pp : 0;
+  sm.Eline = base;                 // never alive together with th, ph, ps, Gm
+  dd* work = base;                 base += a.scratch;
   if (a.mat_ws) {
-    sm.mat = a.mat_ws + (int64_t)blockIdx.x * 16 * nns;
+    sm.mat = a.mat_ws + (int64_t)blockIdx.x * kSetupMats * nns;
+    work = sm.mat + 11 * nns;
   } else {
-    sm.mat = base;                 base += 16 * nns;
+    sm.mat = base;                 base += 11 * nns;
   }
   sm.piv = reinterpret_cast<int*>(base);
+  sm.loc = reinterpret_cast<signed char*>(sm.piv + 1 + nbs);
   const int ms = (int)nns;
   dd* E0w[3] = {sm.mat + 0 * ms, sm.mat + 1 * ms, sm.mat + 2 * ms};
   dd* E1w[3] = {sm.mat + 3 * ms, sm.mat + 4 * ms, sm.mat + 5 * ms};
   dd* E2w[2] = {sm.mat + 6 * ms, sm.mat + 7 * ms};
   dd* M0w[2] = {sm.mat + 8 * ms, sm.mat + 9 * ms};
-  dd* th = sm.mat + 10 * ms;
-  dd* ph = sm.mat + 11 * ms;
-  dd* ps = sm.mat + 12 * ms;
-  dd* Hp = sm.mat + 13 * ms;
-  dd* Gm = sm.mat + 14 * ms;
-  dd* T1 = sm.mat + 15 * ms;
+  dd* Hp = sm.mat + 10 * ms;
+  dd* th = work;
+  dd* ph = work + ms;
+  dd* ps = work + 2 * ms;
+  dd* Gm = work + 3 * ms;
 
+  for (int t = tid; t < L * nb; t += nt) {
+    const int l = t / nb, A = t - l * nb;
+    int p = -1;
+    for (int q = 0; q < pp; ++q)
+      if (a.line_local[(sm.l0 + l) * pp + q] == A) p = q;
+    sm.loc[t] = (signed char)p;
+  }
   // Lagrange tables and line geometry (Section 3 preamble)
   for (int t = tid; t < ng * pp; t += nt) {
     const int g = t / pp, q = t - g * pp;
@@ -532,6 +598,7 @@ __global__ void element_setup_kernel(ElemArgs a) {
       sm.dphz[t] = dd{a.tab[2 * (ng + 2 * ng * pp + g * pp + q)], a.tab[2 * (ng + 2 * ng * pp + g * pp + q) + 1]};
   }
   __syncthreads();
+  if (a.dim == 2) shape_products<DDOps>(a, sm);
   const dd c2 = two_prod(a.c, a.c);
   if (a.dim == 3) {
     // face geometry: J_b rows r_b = x_b - x0, x_b,eta, x_b,zeta; b1, b2, b3 the columns of
@@ -670,20 +737,22 @@ __global__ void element_setup_kernel(ElemArgs a) {
       __syncthreads();
       if (i == 0) {
         // row -1: theta = -xi_0 E0/(2h), phi = E1^T, psi = xi_0 E0/(2h).  rho_0 = theta_0 theta_{-1}^{-1}
+        dd* T1 = E0w[s_prev];                                     // no point before this one
         for (int t = tid; t < nn; t += nt) T1[t] = Op::mul(Op::neg(Op::mul(xi, E0w[s_cur][t])), inv_2h);
         __syncthreads();
-        gj_inverse<Op>(nb, T1, Gm, sm.col, sm.piv, a.status);
-        mm<Op>(nb, th, Gm, Hp);                                   // Hp <- rho_0
+        dd* G = Gm;                                               // (Gm itself stays in its place)
+        gj_inverse<Op>(nb, T1, G, sm.row, sm.piv, a.status);
+        mm<Op>(nb, th, G, Hp);                                   // Hp <- rho_0
         if (a.xel) {
           // rho_0, and the ghost u_{-1} = u_1 + Gamma u_0 from row -1: Gamma = -theta_{-1}^{-1} E1_0^T
           double* X = a.xel + e * 6 * nns;
           for (int t = tid; t < nn; t += nt) {
             const int r = t / nb, cc = t - r * nb;
             dd g = Op::make(0.0);
-            for (int k = 0; k < nb; ++k) g = Op::fma(g, Gm[r * nb + k], E1w[s_cur][cc * nb + k]);
+            for (int k = 0; k < nb; ++k) g = Op::mac(g, G[r * nb + k], E1w[s_cur][cc * nb + k]);
             const int64_t to = (int64_t)r * nbs + cc;
             X[to] = Hp[t].hi;
-            X[2 * nns + to] = -g.hi;
+            X[2 * nns + to] = -Op::norm(g).hi;
           }
           __syncthreads();
         }
@@ -693,16 +762,11 @@ __global__ void element_setup_kernel(ElemArgs a) {
           dd s1 = Op::make(0.0), s2 = Op::make(0.0);
           for (int k = 0; k < nb; ++k) {
             const dd rk = Hp[r * nb + k];
-            s1 = Op::fma(s1, rk, E1w[s_cur][cc * nb + k]);               // phi_{-1}[k][c] = E1[c][k]
-            s2 = Op::fma(s2, rk, Op::mul(Op::mul(xi, E0w[s_cur][k * nb + cc]), inv_2h));
+            s1 = Op::mac(s1, rk, E1w[s_cur][cc * nb + k]);               // phi_{-1}[k][c] = E1[c][k]
+            s2 = Op::mac(s2, rk, E0w[s_cur][k * nb + cc]);               // psi_{-1} = E0 xi / (2h)
           }
-          T1[t] = s1;
-          Gm[t] = s2;
-        }
-        __syncthreads();
-        for (int t = tid; t < nn; t += nt) {
-          ph[t] = Op::sub(ph[t], T1[t]);
-          ps[t] = Op::sub(ps[t], Gm[t]);
+          ph[t] = Op::sub(ph[t], Op::norm(s1));
+          ps[t] = Op::fms(ps[t], Op::norm(s2), Op::mul(xi, inv_2h));
         }
         __syncthreads();
       } else {
@@ -712,12 +776,16 @@ __global__ void element_setup_kernel(ElemArgs a) {
           __syncthreads();
         }
         // Thomas sweep: phi_i -= theta_i phi_{i-1}^{-1} psi_{i-1} = theta_i H_{i-1}
-        mm<Op>(nb, th, Hp, T1);
-        for (int t = tid; t < nn; t += nt) ph[t] = Op::sub(ph[t], T1[t]);
+        for (int t = tid; t < nn; t += nt) {
+          const int r = t / nb, cc = t - r * nb;
+          dd s = Op::make(0.0);
+          for (int k = 0; k < nb; ++k) s = Op::mac(s, th[r * nb + k], Hp[k * nb + cc]);
+          ph[t] = Op::sub(ph[t], Op::norm(s));
+        }
         __syncthreads();
       }
       if (i < n) {
-        gj_inverse<Op>(nb, ph, Gm, sm.col, sm.piv, a.status);     // G_i, destroys ph
+        gj_inverse<Op>(nb, ph, Gm, sm.row, sm.piv, a.status);     // G_i, destroys ph
         if (a.xops) {
           double* Gi = a.xops + (e * (int64_t)n + i) * nns;
           for (int t = tid; t < nn; t += nt) Gi[(int64_t)(t / nb) * nbs + (t % nb)] = Gm[t].hi;
@@ -728,32 +796,31 @@ __global__ void element_setup_kernel(ElemArgs a) {
           dd sp = Op::make(0.0), sq = Op::make(0.0), sh = Op::make(0.0);
           for (int k = 0; k < nb; ++k) {
             const dd gk = Gm[r * nb + k];
-            sp = Op::fma(sp, gk, M0w[w_cur][k * nb + cc]);
-            sq = Op::fma(sq, gk, th[k * nb + cc]);
-            sh = Op::fma(sh, gk, ps[k * nb + cc]);
+            sp = Op::mac(sp, gk, M0w[w_cur][k * nb + cc]);
+            sq = Op::mac(sq, gk, th[k * nb + cc]);
+            sh = Op::mac(sh, gk, ps[k * nb + cc]);
           }
-          sp = Op::mul(sp, x2);
+          sp = Op::mul(Op::norm(sp), x2);
+          sq = Op::norm(sq);
+          sh = Op::norm(sh);
           const int64_t to = (int64_t)r * nbs + cc;
           Pi[to] = sp.hi;
           Pi[nns + to] = (i == 0) ? 0.0 : sq.hi;
           Pi[2 * nns + to] = sh.hi;
-          T1[t] = sh;                                         // H_i kept in double-double
+          Hp[t] = sh;                                         // H_i kept in double-double
         }
-        __syncthreads();
-        for (int t = tid; t < nn; t += nt) Hp[t] = T1[t];
         __syncthreads();
       } else {
         // i == n: th = theta_n, ph = modified phi_n, ps = psi_n, Hp = H_{n-1}
-        for (int t = tid; t < nn; t += nt) T1[t] = ps[t];
-        __syncthreads();
-        gj_inverse<Op>(nb, T1, Gm, sm.col, sm.piv, a.status);     // Gm = psi_n^{-1}
+        gj_inverse<Op>(nb, ps, Gm, sm.row, sm.piv, a.status);     // Gm = psi_n^{-1}
+        dd* T1 = ps;
         // W = psi_{n+1} psi_n^{-1}, psi_{n+1} = xi_n E0_n / (2h)
         for (int t = tid; t < nn; t += nt) {
           const int r = t / nb, cc = t - r * nb;
           dd s = Op::make(0.0);
           for (int k = 0; k < nb; ++k)
-            s = Op::fma(s, Op::mul(Op::mul(xi, E0w[s_cur][r * nb + k]), inv_2h), Gm[k * nb + cc]);
-          T1[t] = s;
+            s = Op::mac(s, Op::mul(Op::mul(xi, E0w[s_cur][r * nb + k]), inv_2h), Gm[k * nb + cc]);
+          T1[t] = Op::norm(s);
         }
         __syncthreads();
         if (a.xel) {
@@ -767,10 +834,11 @@ __global__ void element_setup_kernel(ElemArgs a) {
             for (int k = 0; k < nb; ++k) {
               const dd gk = Gm[r * nb + k];
               const dd mk = Op::mul(x2, M0w[w_cur][k * nb + cc]);
-              yt = Op::fma(yt, gk, th[k * nb + cc]);
-              yp = Op::fma(yp, gk, Op::add(E0w[s_next][k * nb + cc], Op::mul(a.mass, mk)));
-              ym = Op::fma(ym, gk, mk);
+              yt = Op::mac(yt, gk, th[k * nb + cc]);
+              yp = Op::mac(yp, gk, Op::add(E0w[s_next][k * nb + cc], Op::mul(a.mass, mk)));
+              ym = Op::mac(ym, gk, mk);
             }
+            yt = Op::norm(yt); yp = Op::norm(yp); ym = Op::norm(ym);
             const int64_t to = (int64_t)r * nbs + cc;
             X[nns + to] = T1[t].hi;
             X[3 * nns + to] = yt.hi;
@@ -784,8 +852,8 @@ __global__ void element_setup_kernel(ElemArgs a) {
           const int r = t / nb, cc = t - r * nb;
           dd s = E1w[s_cur][cc * nb + r];
           for (int k = 0; k < nb; ++k)
-            s = Op::add(s, Op::mul(Op::mul(Op::mul(xi, E0w[s_cur][r * nb + k]), inv_2h), Hp[k * nb + cc]));
-          Gm[t] = s;
+            s = Op::mac(s, Op::mul(Op::mul(xi, E0w[s_cur][r * nb + k]), inv_2h), Hp[k * nb + cc]);
+          Gm[t] = Op::norm(s);
         }
         __syncthreads();
         double* Se = a.S + e * nns;
@@ -795,10 +863,11 @@ __global__ void element_setup_kernel(ElemArgs a) {
           dd s = Gm[t], rr = Op::mul(Op::mul(xi, E0w[s_cur][t]), inv_2h), tt = Op::make(0.0);  // -theta_{n+1} = xi E0/(2h)
           for (int k = 0; k < nb; ++k) {
             const dd wk = T1[r * nb + k];
-            s = Op::sub(s, Op::mul(wk, ph[k * nb + cc]));
-            rr = Op::fma(rr, wk, th[k * nb + cc]);
-            tt = Op::fma(tt, wk, M0w[w_cur][k * nb + cc]);
+            s = Op::mac(s, Op::neg(wk), ph[k * nb + cc]);
+            rr = Op::mac(rr, wk, th[k * nb + cc]);
+            tt = Op::mac(tt, wk, M0w[w_cur][k * nb + cc]);
           }
+          s = Op::norm(s); rr = Op::norm(rr); tt = Op::norm(tt);
           const int64_t to = (int64_t)r * nbs + cc;
           Se[to] = s.hi;
           Re[to] = rr.hi;
@@ -819,6 +888,8 @@ __global__ void element_setup_kernel(ElemArgs a) {
       w_cur = w_next;
       w_next = ow;
       if (i + 2 <= n) {
+        // read after the barrier behind the density of coefficient_matrices
+        if (i + 2 == kExtendedPoints && a.dim == 2) shape_products<F64Ops>(a, sm);
         if (i + 2 < kExtendedPoints)
           coefficient_matrices<DDOps>(a, sm, e, i + 2, E0w[s_next], E1w[s_next], E2w[w_next], M0w[w_next]);
         else
@@ -1627,13 +1698,18 @@ static int launch_element_setup(Model& md, const Mesh& m, const double* rho_hi, 
   a.rho_hi = rho_hi; a.rho_lo = rho_lo;
   a.xi_hi = d.xih.as<double>(); a.xi_lo = d.xil.as<double>(); a.tab = d.tab.as<double>();
   a.mats = md.mats.as<double>(); a.rt = md.rt.as<double>(); a.S = md.S.as<double>(); a.status = status;
-  // the 16 working matrices live in shared memory up to n_b = 24; beyond, in a global
+  // the working matrices live in shared memory up to n_b = 24; beyond, in a global
   // workspace, with the elements set up in chunks that bound its size
-  const size_t small =
-      sizeof(dd) * ((size_t)L * ng * 2 * nk + (size_t)L * pp * pp * 4 + (m.dim == 3 ? 3 : 2) * (size_t)ng * pp + nb) + 16;
-  const size_t mat_bytes = sizeof(dd) * 16 * (size_t)nn;
-  const bool in_smem = small + mat_bytes <= 160 * 1024;
-  const size_t smem = in_smem ? small + mat_bytes : small;
+  const size_t temps = (size_t)L * pp * pp * 4;
+  const size_t shapes = (size_t)ng * pp * (m.dim == 3 ? 3 : 2 + 3 * pp);
+  const size_t tables = sizeof(dd) * ((size_t)L * ng * 2 * nk + shapes + nb) +
+                        sizeof(int) * (1 + (size_t)nb) + (size_t)L * nb + 16;
+  const size_t mat_bytes = sizeof(dd) * kSetupMats * (size_t)nn;
+  const size_t scratch_smem = std::max(temps, 4 * (size_t)nn);
+  const size_t smem_all = tables + sizeof(dd) * (scratch_smem + 11 * (size_t)nn);
+  const bool in_smem = smem_all <= 160 * 1024;
+  a.scratch = (int)(in_smem ? scratch_smem : temps);
+  const size_t smem = in_smem ? smem_all : tables + sizeof(dd) * temps;
   SBFWI_CUDA(cudaFuncSetAttribute(element_setup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   cudaFuncAttributes fattr;
   SBFWI_CUDA(cudaFuncGetAttributes(&fattr, element_setup_kernel));
