@@ -12,6 +12,7 @@
 //  3. multifrontal factorisation of the global boundary matrix sum_e S_e along
 //     the elimination tree (FP64, one CTA per front, Gauss-Jordan with partial
 //     pivoting inside each separator block).
+#include <cooperative_groups.h>
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -914,21 +915,20 @@ struct FactorArgs {
   double* factors;
   double* work;                 // factors that are merged further (TreeNodeDev::X_off < 0)
   int* status;
-  int products;                 // 1: front_factor_kernel also forms G, C and U (else front_gemm_kernel)
-  int big_s;                    // > 0: fronts with s >= big_s are inverted by front_invert_grid_kernel
 };
 
 __device__ __forceinline__ double* factor_at(const FactorArgs& a, int64_t off) {
   return off >= 0 ? a.factors + off : a.work + ~off;
 }
 
+// gridDim.y blocks per front (one block took 0.4 ms for the largest fronts of the 64 x 64 mesh)
 __global__ void front_assemble_kernel(FactorArgs a) {
   const TreeNodeDev nd = a.nodes[a.level_nodes[blockIdx.x]];
   const int f = nd.s + nd.b;
   double* F = a.F + nd.F_off;
   const int32_t* m0 = a.map0 + nd.map_off;
   const int32_t* m1 = a.map1 + nd.map_off;
-  for (int64_t t = threadIdx.x; t < (int64_t)f * f; t += blockDim.x) {
+  for (int64_t t = blockIdx.y * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)f * f; t += (int64_t)gridDim.y * blockDim.x) {
     const int r = (int)(t / f), c = (int)(t - (int64_t)r * f);
     double v;
     if (nd.elem >= 0) {
@@ -971,6 +971,130 @@ __device__ int block_pivot(const double* F, int f, int k, int s, double* redv, i
   return (v > 0.0 && isfinite(v)) ? r : -1;
 }
 
+// X = F11^{-1} of a front by a cluster of blocks: Gauss-Jordan with row pivoting inside F11, in place in shared memory
+// (column k of the identity takes the place of column k as it is eliminated).  Block q holds a slab of columns, so
+// the pivot is found by one warp of the block that holds the pivot column: it updates that column first, finds the
+// next pivot and sends the column (rows exchanged), the pivot and its inverse to every block's shared memory while
+// the other warps update theirs; one cluster barrier ends the step.  Two buffers alternate: a block writes the one
+// that every block read in the step before the last barrier.  Each entry sees the operations of the elimination of
+// [F11 | I] in memory (front_factor_kernel), so X has the same bits.
+// What bounds it: s steps of a barrier, a pivot search and w s products on an SM (w columns a block).  One block
+// working in memory took 3.8 ms for s = 129 (2 to 4 fronts a level), the whole grid with its barriers 3.0 ms for
+// s = 257; clusters of 8 take 0.63 and 2.0 ms.
+constexpr size_t kInvertSmem = 200 * 1024;
+constexpr int kInvertCluster = 8;             // the portable cluster size
+constexpr size_t invert_bytes(int s, int w) {  // slab, two columns, pivot row | pivots, exchanged columns
+  return sizeof(double) * ((size_t)s * w + 2 * (size_t)s + w + 2) + sizeof(int) * ((size_t)s + 2);
+}
+constexpr int largest_invert_s() {
+  int s = 1;
+  while (invert_bytes(s + 1, (s + kInvertCluster) / kInvertCluster) <= kInvertSmem) ++s;
+  return s;
+}
+constexpr int kClusterInvertS = largest_invert_s();   // larger separators: front_factor_kernel, front_invert_grid_kernel
+
+__global__ void __launch_bounds__(256) front_invert_kernel(FactorArgs a) {
+  namespace cg = cooperative_groups;
+  extern __shared__ double sm_inv[];
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = (int)cl.num_blocks(), q = (int)cl.block_rank();
+  const TreeNodeDev nd = a.nodes[a.level_nodes[blockIdx.x / cs]];
+  const int s = nd.s, f = nd.s + nd.b;
+  if (s == 0 || s > kClusterInvertS) return;           // the whole cluster
+  const double* F = a.F + nd.F_off;
+  double* X = factor_at(a, nd.X_off);
+  const int W = (s + cs - 1) / cs, c0 = min(q * W, s), w = min(W, s - c0);   // w = 0: a block without columns
+  double* M = sm_inv;                    // [s][W]
+  double* colb = M + (size_t)s * W;      // [2][s]
+  double* row = colb + 2 * s;            // [W]
+  double* pinvb = row + W;               // [2]
+  int* pivb = reinterpret_cast<int*>(pinvb + 2);   // [2]
+  int* own = pivb + 2;                   // [s]
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  for (int c = tid; c < s; c += nt) own[c] = c;
+  for (int r = tid >> 5; r < s; r += nt >> 5)
+    for (int j = lane; j < w; j += 32) M[r * W + j] = F[(int64_t)r * f + c0 + j];
+  cl.sync();
+
+  // warp 0 of the block that holds column k: the pivot, its inverse and the column to buffer k & 1 of every block
+  auto send_pivot = [&](int k) {
+    const int j = k - c0, buf = k & 1;
+    double bv = -1.0;
+    int best = s;
+    for (int r = k + lane; r < s; r += 32) {
+      const double v = fabs(M[r * W + j]);
+      if (v > bv) { bv = v; best = r; }
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+      const double ov = __shfl_xor_sync(0xffffffffu, bv, off);
+      const int oi = __shfl_xor_sync(0xffffffffu, best, off);
+      if (ov > bv || (ov == bv && oi < best)) { bv = ov; best = oi; }
+    }
+    const bool ok = bv > 0.0 && isfinite(bv);
+    const double pinv = ok ? 1.0 / M[best * W + j] : 0.0;
+    for (int b = 0; b < cs; ++b) {
+      double* col = cl.map_shared_rank(colb, b) + buf * s;
+      if (ok)
+        for (int r = lane; r < s; r += 32) col[r] = r == k ? 0.0 : M[(r == best ? k : r) * W + j];
+      if (lane == 0) {
+        cl.map_shared_rank(pivb, b)[buf] = ok ? best : -1;
+        cl.map_shared_rank(pinvb, b)[buf] = pinv;
+      }
+    }
+  };
+  if (q == 0 && tid < 32) send_pivot(0);
+  cl.sync();
+  for (int k = 0; k < s; ++k) {
+    const int pr = pivb[k & 1];
+    const double pinv = pinvb[k & 1];
+    const double* col = colb + (k & 1) * s;
+    if (pr < 0) {                        // every block reads the same
+      if (tid == 0 && q == 0) atomic_flag(a.status, SBFWI_ESINGULAR);
+      return;
+    }
+    for (int j = tid; j < w; j += nt) {
+      const double v = M[pr * W + j];
+      if (pr != k) M[pr * W + j] = M[k * W + j];
+      row[j] = c0 + j == k ? pinv : v * pinv;
+    }
+    if (tid == 0) {
+      const int o = own[pr];
+      own[pr] = own[k];
+      own[k] = o;
+    }
+    __syncthreads();
+    const int jk = k - c0, jn = k + 1 - c0;                  // this and the next pivot column's places
+    auto update = [&](int r, int j) {
+      const double fr = col[r];
+      const double v = j == jk ? 0.0 : M[r * W + j];
+      M[r * W + j] = r == k ? row[j] : fr != 0.0 ? fma(-fr, row[j], v) : v;
+    };
+    const bool next = k + 1 < s && jn >= 0 && jn < w;        // this block sends the next pivot
+    if (next && tid < 32) {
+      for (int r = lane; r < s; r += 32) update(r, jn);
+      __syncwarp();
+      send_pivot(k + 1);
+    } else {
+      const int first = next ? tid - 32 : tid, step = next ? nt - 32 : nt;
+      if (w > 0) {
+        int r = first / w, j = first - r * w;
+        const int dr = step / w, dj = step - dr * w;
+        while (r < s) {
+          if (!next || j != jn) update(r, j);
+          r += dr;
+          j += dj;
+          if (j >= w) { j -= w; ++r; }
+        }
+      }
+    }
+    cl.sync();
+  }
+  for (int r = tid >> 5; r < s; r += nt >> 5)
+    for (int j = lane; j < w; j += 32) X[(int64_t)r * s + own[c0 + j]] = M[r * W + j];
+}
+
+// G, C and U of the fronts of a level with many fronts, one block each (else front_gemm_kernel), after the
+// inverses of separators too large for front_invert_kernel
 __global__ void front_factor_kernel(FactorArgs a) {
   __shared__ double redv[32];
   __shared__ int redi[32];
@@ -983,8 +1107,7 @@ __global__ void front_factor_kernel(FactorArgs a) {
   double* C = G + (int64_t)s * b;              // b x s
   double* U = a.U + nd.U_off;                  // b x b
   const int tid = threadIdx.x, nt = blockDim.x;
-  if (a.big_s > 0 && s >= a.big_s) return;     // inverted over the whole grid; products by tiles
-  if (s > 0) {
+  if (s > kClusterInvertS) {                   // smaller ones: front_invert_kernel
     // X = F11^{-1}: Gauss-Jordan on [F11 | I] with row pivoting inside F11
     for (int64_t t = tid; t < (int64_t)s * s; t += nt) X[t] = ((t / s) == (t % s)) ? 1.0 : 0.0;
     __syncthreads();
@@ -1024,7 +1147,8 @@ __global__ void front_factor_kernel(FactorArgs a) {
         __syncthreads();
       }
     }
-    if (!a.products) return;
+  }
+  if (s > 0) {
     // G = X F12 (s x b), C = F21 X (b x s)
     for (int64_t t = tid; t < (int64_t)s * b; t += nt) {
       const int r = (int)(t / b), c = (int)(t - (int64_t)r * b);
@@ -1040,7 +1164,6 @@ __global__ void front_factor_kernel(FactorArgs a) {
     }
     __syncthreads();
   }
-  if (!a.products) return;
   // update matrix U = F22 - C F12 (b x b)
   for (int64_t t = tid; t < (int64_t)b * b; t += nt) {
     const int r = (int)(t / b), c = (int)(t - (int64_t)r * b);
@@ -1142,8 +1265,6 @@ __global__ void __launch_bounds__(512) front_invert_grid_kernel(InvertArgs ia) {
     if (!grid_barrier(ia.bar, ia.bar + 1, a.status, ia.budget)) return;
   }
 }
-
-constexpr int kGridInvertS = 192;     // separators from this size up are inverted over the whole grid
 
 // The products of front_factor_kernel as 32 x 32 output tiles spread over many blocks (a
 // level's large fronts would otherwise each keep one SM busy): item {node, kind, r0, c0},
@@ -1862,9 +1983,9 @@ int setup_model(Model& md, const Mesh& m, const double* rho, int mem, cudaStream
     // the grid of the cooperative inversion: one block of 512 threads per SM, as many as fit
     DevBuf inv_bar;
     SBFWI_CUDA(inv_bar.alloc(2 * sizeof(unsigned)));
-    int inv_grid = 0;
+    int inv_grid = 0, sms = 0;
     {
-      int dev_id = 0, sms = 0, per_sm = 0;
+      int dev_id = 0, per_sm = 0;
       SBFWI_CUDA(cudaGetDevice(&dev_id));
       SBFWI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id));
       SBFWI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, front_invert_grid_kernel, 512, 0));
@@ -1877,14 +1998,35 @@ int setup_model(Model& md, const Mesh& m, const double* rho, int mem, cudaStream
       // per front would leave most SMs idle); levels with many small fronts keep them in
       // front_factor_kernel
       const int64_t gc0 = d.fgemm_start[3 * l], u0 = d.fgemm_start[3 * l + 1], u1 = d.fgemm_start[3 * l + 2];
-      a.products = d.fgemm_level[l] ? 0 : 1;
-      a.big_s = d.fgemm_level[l] ? kGridInvertS : 0;
-      front_assemble_kernel<<<cnt, 256, 0, st>>>(a);
-      front_factor_kernel<<<cnt, 512, 0, st>>>(a);
-      prof.count(kPhaseSetup, 2);
-      if (a.big_s > 0)
+      int s_inv = 0;                                   // largest separator of front_invert_kernel
+      for (int32_t v : t.nodes_at_level[l])
+        if (t.nodes[v].s <= kClusterInvertS) s_inv = std::max(s_inv, (int)t.nodes[v].s);
+      const unsigned split = std::max(1u, std::min(32u, 4u * (unsigned)sms / cnt));
+      front_assemble_kernel<<<dim3(cnt, split), 256, 0, st>>>(a);
+      prof.count(kPhaseSetup);
+      if (s_inv > 0) {
+        // clusters as large as the level leaves SMs for, of at least 8 columns a block; larger where the front needs it
+        int cs = 1;
+        while (cs < kInvertCluster && (invert_bytes(s_inv, (s_inv + cs - 1) / cs) > kInvertSmem ||
+                                       (2 * cs * cnt <= (unsigned)sms && 16 * cs <= s_inv)))
+          cs *= 2;
+        const size_t bytes = invert_bytes(s_inv, (s_inv + cs - 1) / cs);
+        SBFWI_CUDA(cudaFuncSetAttribute(front_invert_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvertSmem));
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)cs; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(cnt * (unsigned)cs); cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = bytes; cfg.stream = st;
+        cfg.attrs = &attr; cfg.numAttrs = 1;
+        SBFWI_CUDA(cudaLaunchKernelEx(&cfg, front_invert_kernel, a));
+        prof.count(kPhaseSetup);
+      }
+      if (!d.fgemm_level[l]) {
+        front_factor_kernel<<<cnt, 512, 0, st>>>(a);
+        prof.count(kPhaseSetup);
+      } else {
         for (int32_t v : t.nodes_at_level[l]) {
-          if (t.nodes[v].s < kGridInvertS) continue;
+          if (t.nodes[v].s <= kClusterInvertS) continue;
           InvertArgs ia;
           ia.f = a; ia.node = v; ia.bar = inv_bar.as<unsigned>(); ia.budget = 4000000000LL;
           SBFWI_CUDA(cudaMemsetAsync(inv_bar.p, 0, inv_bar.bytes, st));
@@ -1893,7 +2035,6 @@ int setup_model(Model& md, const Mesh& m, const double* rho, int mem, cudaStream
                                                  0, st));
           prof.count(kPhaseSetup);
         }
-      if (!a.products) {
         const int4* items = d.fgemm.as<int4>();
         if (u0 > gc0) { front_gemm_kernel<<<(unsigned)(u0 - gc0), 256, 0, st>>>(a, items + gc0); prof.count(kPhaseSetup); }
         if (u1 > u0) { front_gemm_kernel<<<(unsigned)(u1 - u0), 256, 0, st>>>(a, items + u0); prof.count(kPhaseSetup); }
