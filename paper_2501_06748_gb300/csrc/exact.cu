@@ -23,9 +23,10 @@
 // radial point and of the radial differences of E0, E1 (central inside, one-sided at the
 // ends), and these are linear in the densities of the point: E0 = sum_j rho_j E0hat_j with
 // E0hat_j = int phi_j c^2 (b1.b1) phi^T phi det J_b d eta (Eq. (Es)).  So each row's share
-// is a sum of Gauss-point products of the interpolated mu and u fields (and their eta
-// derivatives), accumulated per radial point, line element and Gauss point over the time
-// loop and projected onto phi_j once at the end.
+// is a sum over Gauss points of products of the interpolated mu and u fields (and their eta
+// derivatives), bilinear in a line's nodal values: the time loop accumulates the products
+// of the nodal values per row and line, which are interpolated and projected onto phi_j
+// once at the end.
 #include <algorithm>
 #include <cstdint>
 
@@ -219,155 +220,143 @@ __global__ void exact_boundary_post_kernel(ExactBoundaryArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// gradient: Gauss-point products of one step
+// gradient: products of one step
 // ---------------------------------------------------------------------------
-struct Acc4 {
-  double e0, e1, e2, m;
-};
-__device__ __forceinline__ void zero4(Acc4& x) { x.e0 = x.e1 = x.e2 = x.m = 0.0; }
-
-// sum over the Bp lanes of one (element, line, Gauss point), then one lane adds the station's
-// four sums to the accumulators
-__device__ __forceinline__ void flush4(const ExactGradArgs& a, Acc4 v, int64_t e, int st, int l, int g, int lane,
-                                       int Bp, bool live) {
-  for (int off = Bp >> 1; off > 0; off >>= 1) {
-    v.e0 += __shfl_xor_sync(0xffffffffu, v.e0, off);
-    v.e1 += __shfl_xor_sync(0xffffffffu, v.e1, off);
-    v.e2 += __shfl_xor_sync(0xffffffffu, v.e2, off);
-    v.m += __shfl_xor_sync(0xffffffffu, v.m, off);
+// Row r = -1..n+1 of one element per block: for every line and pair (a, b) of its nodes the
+// products sum_shots mu_a w_b, added to the accumulators, with w = u_{r-1} - 2 u_r + u_{r+1},
+// u_{r+1} - u_{r-1}, u_r and u'' (rows -1 and n+1: the two in the middle, with the fields of rows
+// 0 and n).  The two in the middle are also differentiated along the line: there the values of a line are its
+// first node's and the others' differences from it, so that the derivatives lose nothing where a field is
+// nearly constant around the element (towards the scaling centre, as xi).
+// Why nodal products: interpolating the fields to the Gauss points and multiplying there takes about 70
+// FP64 operations per Gauss point, row and shot (seven points a line of order 4), the products 4 (p + 1)^2
+// per line, row and shot without a reduction over lanes; the pipe does 2 a clock and SM.  576 elements of
+// order 4, 32 radial points, 8 shots: 0.75 -> 0.15 ms a step.
+__global__ void __launch_bounds__(128) exact_gradient_kernel(ExactGradArgs a) {
+  extern __shared__ double shw[];          // [5][B][nb]: the four w and mu; [3][B][L][pp]: the middle two and mu by line
+  const int nb = a.nb, n = a.n, B = a.B, per = nb * B, pp = a.pp, p2 = pp * pp;
+  const int64_t e = blockIdx.x / (n + 3);
+  const int r = (int)(blockIdx.x - e * (n + 3)) - 1;
+  const int rr = min(max(r, 0), n);
+  const bool inner = r == rr;
+  const int32_t* dofs = a.dofs + e * nb;
+  const double* fu = a.fu_int + e * (int64_t)n * per;
+  const double* gh = a.ghost + e * 2 * per;
+  for (int t = threadIdx.x; t < per; t += blockDim.x) {
+    const int j = t / B, s = t - j * B;
+    const int32_t gn = dofs[j];
+    const bool node = gn < a.N;            // padding dofs point at node N
+    // row q of the forward solution: ghosts, interior, boundary nodes
+    auto u = [&](int q) {
+      if (q < 0) return gh[t];
+      if (q < n) return fu[(int64_t)q * per + t];
+      if (q == n) return node ? a.fu_b[(int64_t)gn * B + s] : 0.0;
+      return gh[per + t];
+    };
+    const double uA = u(rr - 1), uB = u(rr), uC = u(rr + 1);
+    double w3 = 0.0;
+    if (inner) w3 = r < n ? a.fa_int[(e * n + r) * (int64_t)per + t] : node ? a.fa_b[(int64_t)gn * B + s] : 0.0;
+    const double mu = r <= n ? a.mu[(e * (n + 2) + r + 1) * (int64_t)per + t] : node ? a.fbar[(int64_t)gn * B + s] : 0.0;
+    const int o = s * nb + j;
+    shw[o] = uA - 2.0 * uB + uC;
+    shw[per + o] = uC - uA;
+    shw[2 * per + o] = uB;
+    shw[3 * per + o] = w3;
+    shw[4 * per + o] = mu;
   }
-  if (live && lane == 0) {
-    const int64_t LG = (int64_t)a.L * a.ng;
-    double* acc = a.gacc + ((e * (a.n + 1) + st) * 4) * LG + (int64_t)l * a.ng + g;
-    acc[0] += v.e0;
-    acc[LG] += v.e1;
-    acc[2 * LG] += v.e2;
-    acc[3 * LG] += v.m;
+  __syncthreads();
+  const int64_t l0 = a.lptr[e];
+  const int L = (int)(a.lptr[e + 1] - l0);
+  const int lp = L * pp;
+  double* line = shw + 5 * per;
+  for (int t = threadIdx.x; t < 3 * B * lp; t += blockDim.x) {
+    const int v = t / (B * lp), sq = t - v * B * lp, s = sq / lp, q = sq - s * lp;
+    const double* f = shw + (v < 2 ? v + 1 : 4) * per + s * nb;
+    const int32_t* loc = a.line_local + l0 * pp;
+    const double x = f[loc[q]];
+    line[t] = q % pp ? x - f[loc[q / pp * pp]] : x;
+  }
+  __syncthreads();
+  double* out = a.prod + (int64_t)blockIdx.x * a.L * 4 * p2;
+  for (int o = threadIdx.x; o < L * 4 * p2; o += blockDim.x) {
+    const int lk = o / p2, ab = o - lk * p2, l = lk >> 2, k = lk & 3, ia = ab / pp, ib = ab - ia * pp;
+    if (!inner && (k == 0 || k == 3)) continue;
+    const int32_t* loc = a.line_local + (l0 + l) * pp;
+    const bool by_line = k == 1 || k == 2;
+    const double* m = by_line ? line + 2 * B * lp + l * pp + ia : shw + 4 * per + loc[ia];
+    const double* w = by_line ? line + (k - 1) * B * lp + l * pp + ib : shw + k * per + loc[ib];
+    const int stride = by_line ? lp : nb;
+    double acc = out[o];
+    for (int s = 0; s < B; ++s) acc = fma(m[s * stride], w[s * stride], acc);
+    out[o] = acc;
   }
 }
 
-template <int PP>
-__global__ void __launch_bounds__(256) exact_gradient_kernel(ExactGradArgs a) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int Bp = a.Bp;
-  const int lane = (int)(t % Bp);
-  const int64_t grp = t / Bp;                      // (e, line, Gauss point)
-  const int ng = a.ng;
-  const int g = (int)(grp % ng);
-  const int64_t el = grp / ng;
-  const int l = (int)(el % a.L);
-  const int64_t e = el / a.L;
-  const bool in_range = e < a.E;
-  const int64_t ee = in_range ? e : 0;
-  const int L_e = (int)(a.lptr[ee + 1] - a.lptr[ee]);
-  // a whole warp takes part in the shuffles: lanes outside the problem compute zeros
-  const bool live = in_range && l < L_e;
-  const int s = lane < a.B ? lane : 0;
-  const bool shot = live && lane < a.B;
-  const int nb = a.nb, n = a.n, B = a.B;
-  const int per = nb * B;
-  double ph[PP], dph[PP];
-  int loc[PP];
-#pragma unroll
-  for (int q = 0; q < PP; ++q) {
-    ph[q] = a.tab[2 * (ng + g * PP + q)];
-    dph[q] = a.tab[2 * (ng + ng * PP + g * PP + q)];
-    loc[q] = live ? a.line_local[(a.lptr[ee] + l) * PP + q] : 0;
+// The Gauss-point sums of every station (radial point) from the nodal products of its row and its neighbours:
+// a row's terms in E0 and E1 at its own point, and in their radial differences (forward at row 0, backward at
+// row n, central inside)
+__global__ void exact_collect_kernel(ExactFinalArgs a) {
+  const int n = a.n, pp = a.pp, p2 = pp * pp, ng = a.ng;
+  const int64_t tot = a.E * (int64_t)(n + 1) * a.L * ng;
+  const double inv_2h = 0.5 / a.h;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < tot; t += (int64_t)gridDim.x * blockDim.x) {
+    const int g = (int)(t % ng);
+    const int64_t tl = t / ng;
+    const int l = (int)(tl % a.L);
+    const int64_t es = tl / a.L, e = es / (n + 1);
+    const int st = (int)(es - e * (n + 1));
+    if (l >= (int)(a.lptr[e + 1] - a.lptr[e])) continue;
+    const double* ph = a.tab + 2 * (ng + g * pp);                 // double-double pairs: the high parts
+    const double* dph = a.tab + 2 * (ng + ng * pp + g * pp);
+    auto row = [&](int r, int k) { return a.prod + (((e * (n + 3) + r + 1) * a.L + l) * 4 + k) * p2; };
+    // sum_ab x_a y_b prod_ab, with x0 and y0 for the first node's functions
+    auto contract = [&](const double* pr, double x0, const double* x, double y0, const double* y) {
+      double v = 0.0;
+      for (int ia = 0; ia < pp; ++ia) {
+        double q = 0.0;
+        for (int ib = 0; ib < pp; ++ib) q = fma(ib ? y[2 * ib] : y0, pr[ia * pp + ib], q);
+        v = fma(ia ? x[2 * ia] : x0, q, v);
+      }
+      return v;
+    };
+    // values and derivatives of the products by line: the first node's value has the functions 1 and 0
+    auto vv = [&](int r, int k) { return contract(row(r, k), 1.0, ph, 1.0, ph); };
+    auto vd = [&](int r, int k) { return contract(row(r, k), 1.0, ph, 0.0, dph); };
+    auto dv = [&](int r, int k) { return contract(row(r, k), 0.0, dph, 1.0, ph); };
+    auto nodal = [&](int r, int k) { return contract(row(r, k), ph[0], ph, ph[0], ph); };
+    const double xi = a.xi[st];
+    double e0 = xi * xi / (a.h * a.h) * nodal(st, 0) + xi * inv_2h * vv(st, 1);
+    double e1 = xi * inv_2h * (vd(st, 1) - dv(st, 1));
+    const double e2 = -contract(row(st, 2), 0.0, dph, 0.0, dph);
+    const double m = -xi * xi * nodal(st, 3);
+    // times the weight w that row r's difference gives this station
+    auto differences = [&](int r, double w) {
+      const double x = a.xi[r];
+      e0 = fma(w, x * x * inv_2h * vv(r, 1), e0);
+      e1 = fma(w, x * vd(r, 2), e1);
+    };
+    if (st == 0) differences(0, -1.0 / a.h);
+    if (st == n) differences(n, 1.0 / a.h);
+    if (st >= 1) differences(st - 1, st == 1 ? 1.0 / a.h : inv_2h);
+    if (st < n) differences(st + 1, st + 1 == n ? -1.0 / a.h : -inv_2h);
+    // rows -1 and n+1: xi E0 (u_{r+1} - u_{r-1}) / (2h) + E1^T u
+    for (int end = 0; end < 2; ++end)
+      if (st == (end ? n : 0)) {
+        const int r = end ? n + 1 : -1;
+        e0 = fma(xi * inv_2h, vv(r, 1), e0);
+        e1 += vd(r, 2);
+      }
+    const int64_t LG = (int64_t)a.L * ng;
+    double* acc = a.gacc + es * 4 * LG + (int64_t)l * ng + g;
+    acc[0] = e0;
+    acc[LG] = e1;
+    acc[2 * LG] = e2;
+    acc[3 * LG] = m;
   }
-  const double h = a.h;
-  const double* fu_int = a.fu_int + ee * (int64_t)n * per;
-  const double* fa_int = a.fa_int + ee * (int64_t)n * per;
-  const double* mu = a.mu + ee * (int64_t)(n + 2) * per;
-  const double* gh = a.ghost + ee * 2 * per;
-  const int32_t* dofs = a.dofs + ee * nb;
-  // value and eta-derivative at this Gauss point of a field row given per local dof
-  auto interp_row = [&](const double* row, double& v, double& d) {
-    v = 0.0; d = 0.0;
-#pragma unroll
-    for (int q = 0; q < PP; ++q) {
-      const double x = shot ? row[loc[q] * B + s] : 0.0;
-      v = fma(ph[q], x, v);
-      d = fma(dph[q], x, d);
-    }
-  };
-  auto interp_nodes = [&](const double* glob, double& v, double& d) {   // a row on the global nodes
-    v = 0.0; d = 0.0;
-#pragma unroll
-    for (int q = 0; q < PP; ++q) {
-      const int32_t gn = dofs[loc[q]];
-      const double x = (shot && gn < a.N) ? glob[(int64_t)gn * B + s] : 0.0;
-      v = fma(ph[q], x, v);
-      d = fma(dph[q], x, d);
-    }
-  };
-  // the forward solution's row r = -1..n+1 (ghosts, interior, boundary nodes)
-  auto u_row = [&](int r, double& v, double& d) {
-    if (r == -1) interp_row(gh, v, d);
-    else if (r < n) interp_row(fu_int + (int64_t)r * per, v, d);
-    else if (r == n) interp_nodes(a.fu_b, v, d);
-    else interp_row(gh + per, v, d);
-  };
-  double uA, uAd, uB, uBd, uC, uCd, mv, md, av, ad;
-  Acc4 prv, cur, nxt;
-  zero4(prv); zero4(cur); zero4(nxt);
-  u_row(-1, uA, uAd);
-  u_row(0, uB, uBd);
-  u_row(1, uC, uCd);
-  const double inv_2h = 0.5 / h;
-  // row -1 (station 0): xi_0 E0_0 (u_1 - u_{-1}) / (2h) + E1_0^T u_0
-  interp_row(mu, mv, md);
-  {
-    const double x0 = a.xi[0];
-    cur.e0 = fma(x0 * inv_2h * mv, uC - uA, cur.e0);
-    cur.e1 = fma(uBd, mv, cur.e1);
-  }
-  for (int r = 0; r <= n; ++r) {
-    if (r > 0) {
-      uA = uB; uAd = uBd; uB = uC; uBd = uCd;
-      u_row(r + 1, uC, uCd);
-    }
-    interp_row(mu + (int64_t)(r + 1) * per, mv, md);
-    if (r < n) interp_row(fa_int + (int64_t)r * per, av, ad);
-    else interp_nodes(a.fa_b, av, ad);
-    const double xi = a.xi[r];
-    const double d1 = uC - uA, d1d = uCd - uAd, d2 = uA - 2.0 * uB + uC;
-    cur.e0 = fma(mv, fma(xi * xi / (h * h), d2, xi * inv_2h * d1), cur.e0);
-    cur.e1 = fma(xi * inv_2h, fma(d1d, mv, -md * d1), cur.e1);
-    cur.e2 = fma(-md, uBd, cur.e2);
-    cur.m = fma(-xi * xi * mv, av, cur.m);
-    // radial differences of E0 and E1: forward at r = 0, backward at r = n, central inside
-    const double te0 = xi * xi * inv_2h * mv * d1;     // times the weight of E0 at a station
-    const double te1 = xi * uBd * mv;                  // times the weight of E1 at a station
-    if (r == 0) {
-      const double w = 1.0 / h;
-      nxt.e0 = fma(w, te0, nxt.e0); nxt.e1 = fma(w, te1, nxt.e1);
-      cur.e0 = fma(-w, te0, cur.e0); cur.e1 = fma(-w, te1, cur.e1);
-    } else if (r == n) {
-      const double w = 1.0 / h;
-      cur.e0 = fma(w, te0, cur.e0); cur.e1 = fma(w, te1, cur.e1);
-      prv.e0 = fma(-w, te0, prv.e0); prv.e1 = fma(-w, te1, prv.e1);
-    } else {
-      nxt.e0 = fma(inv_2h, te0, nxt.e0); nxt.e1 = fma(inv_2h, te1, nxt.e1);
-      prv.e0 = fma(-inv_2h, te0, prv.e0); prv.e1 = fma(-inv_2h, te1, prv.e1);
-    }
-    if (r == n) break;
-    // station r - 1 is complete
-    if (r >= 1) flush4(a, prv, ee, r - 1, l, g, lane, Bp, live);
-    prv = cur; cur = nxt; zero4(nxt);
-  }
-  // row n+1 (station n): xi_n E0_n (u_{n+1} - u_{n-1}) / (2h) + E1_n^T u_n, mu_{n+1} on the global nodes
-  interp_nodes(a.fbar, mv, md);
-  {
-    const double xn = a.xi[n];
-    cur.e0 = fma(xn * inv_2h * mv, uC - uA, cur.e0);
-    cur.e1 = fma(uBd, mv, cur.e1);
-  }
-  flush4(a, prv, ee, n - 1, l, g, lane, Bp, live);
-  flush4(a, cur, ee, n, l, g, lane, Bp, live);
 }
 
-// dE/drho at every radial point and boundary node of every element from the accumulated
-// products: -sum_lines sum_g phi_j(g) (k0 A0 + k1 A1 + k2 A2 + km Am); interior points go to
+// dE/drho at every radial point and boundary node of every element from the Gauss-point
+// sums: -sum_lines sum_g phi_j(g) (k0 A0 + k1 A1 + k2 A2 + km Am); interior points go to
 // the library's nodal layout, the boundary station to a per-element slot (gathered per node)
 __global__ void exact_finalize_kernel(ExactFinalArgs a) {
   const int nb = a.nb, n = a.n, pp = a.pp, ng = a.ng;
@@ -440,26 +429,20 @@ int exact_boundary_launch(const ExactBoundaryArgs& a, bool post, cudaStream_t st
   return SBFWI_OK;
 }
 
-int exact_gradient_launch(const ExactGradArgs& a, int p, cudaStream_t st) {
-  const int64_t threads = a.E * (int64_t)a.L * a.ng * a.Bp;
-  const unsigned blocks = (unsigned)((threads + 255) / 256);
-  switch (p + 1) {
-    case 2: exact_gradient_kernel<2><<<blocks, 256, 0, st>>>(a); break;
-    case 3: exact_gradient_kernel<3><<<blocks, 256, 0, st>>>(a); break;
-    case 4: exact_gradient_kernel<4><<<blocks, 256, 0, st>>>(a); break;
-    case 5: exact_gradient_kernel<5><<<blocks, 256, 0, st>>>(a); break;
-    case 6: exact_gradient_kernel<6><<<blocks, 256, 0, st>>>(a); break;
-    case 7: exact_gradient_kernel<7><<<blocks, 256, 0, st>>>(a); break;
-    case 8: exact_gradient_kernel<8><<<blocks, 256, 0, st>>>(a); break;
-    case 9: exact_gradient_kernel<9><<<blocks, 256, 0, st>>>(a); break;
-    default: return fail(SBFWI_EUNSUPPORTED, "line order outside 1..8");
-  }
+int exact_gradient_launch(const ExactGradArgs& a, cudaStream_t st) {
+  if (a.pp < 2 || a.pp > 9) return fail(SBFWI_EUNSUPPORTED, "line order outside 1..8");
+  const size_t smem = sizeof(double) * (size_t)a.B * (5 * (size_t)a.nb + 3 * (size_t)a.L * a.pp);
+  if (smem > 48 * 1024)
+    SBFWI_CUDA(cudaFuncSetAttribute(exact_gradient_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  exact_gradient_kernel<<<(unsigned)(a.E * (a.n + 3)), 128, smem, st>>>(a);
   SBFWI_CUDA(cudaGetLastError());
   return SBFWI_OK;
 }
 
 int exact_finalize_launch(const ExactFinalArgs& a, const int64_t* inc_ptr, const int64_t* inc_list, int64_t N,
                           double* g_nodal_b, cudaStream_t st) {
+  const int64_t sums = a.E * (int64_t)(a.n + 1) * a.L * a.ng;
+  exact_collect_kernel<<<(unsigned)std::min<int64_t>((sums + 127) / 128, 152 * 32), 128, 0, st>>>(a);
   const int64_t tot = a.E * (int64_t)(a.n + 1) * a.nb;
   exact_finalize_kernel<<<(unsigned)std::min<int64_t>((tot + 255) / 256, 152 * 16), 256, 0, st>>>(a);
   exact_gather_nodes_kernel<<<(unsigned)std::min<int64_t>((N + 255) / 256, 152 * 8), 256, 0, st>>>(

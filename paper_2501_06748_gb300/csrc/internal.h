@@ -335,10 +335,7 @@ struct ExactBoundaryArgs {
 
 struct ExactGradArgs {
   int64_t E, N;
-  int nb, n, B, Bp, L, ng;
-  double h;
-  const double* xi;                        // [n+1]
-  const double* tab;                       // Gauss weights and Lagrange tables (double-double pairs)
+  int nb, n, B, L, pp;
   const int64_t* lptr;                     // [E+1]
   const int32_t* line_local;               // [lines][p+1]
   const int32_t* dofs;
@@ -347,7 +344,7 @@ struct ExactGradArgs {
   const double* fu_int; const double* fu_b;   // forward u after the step
   const double* fa_int; const double* fa_b;   // forward u'' after the step
   const double* ghost;                     // [E][2][nb][B]
-  double* gacc;                            // [E][n+1][4][L][ng]
+  double* prod;                            // [E][n+3][L][4][pp][pp] (exact_gradient_kernel)
 };
 
 struct ExactFinalArgs {
@@ -357,7 +354,10 @@ struct ExactFinalArgs {
   const int32_t* line_local;
   const double* tab;
   const double* kq;                        // [E][L][ng][4]
-  const double* gacc;
+  double h;
+  const double* xi;                        // [n+1]
+  const double* prod;                      // ExactGradArgs::prod
+  double* gacc;                            // [E][n+1][4][L][ng] (exact_collect_kernel)
   double* g_nodal;                         // interior part of the library's nodal layout
   double* g_bnd;                           // [E][nb] boundary station per element
 };
@@ -367,7 +367,7 @@ int exact_element_launch(const ExactElemArgs& a, cudaStream_t st);
 int exact_misfit_launch(double* ub, int B, int R, const int64_t* rec, const double* res, int64_t K, int64_t k, double dt,
                         cudaStream_t st);
 int exact_boundary_launch(const ExactBoundaryArgs& a, bool post, cudaStream_t st);
-int exact_gradient_launch(const ExactGradArgs& a, int p, cudaStream_t st);
+int exact_gradient_launch(const ExactGradArgs& a, cudaStream_t st);
 int exact_finalize_launch(const ExactFinalArgs& a, const int64_t* inc_ptr, const int64_t* inc_list, int64_t N,
                           double* g_nodal_b, cudaStream_t st);
 

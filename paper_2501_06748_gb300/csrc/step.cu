@@ -1396,7 +1396,7 @@ struct RunBuffers {
   DevBuf grad_int;                  // grad accumulators [n_nodal][B] (adjoint; boundary nodes alone if tg holds the rest)
   // exact adjoint: mu of rows -1..n, v_bar_n per element, ghosts of the forward solution,
   // Gauss-point products, boundary station of the gradient per element
-  DevBuf mu, vbn, ghost, gacc, gbnd;
+  DevBuf mu, vbn, ghost, gprod, gacc, gbnd;
 };
 
 // Forward: the forward solve; Adjoint: the paper's time-reversed adjoint with the velocity
@@ -1611,10 +1611,11 @@ int Stepper::init() {
     SBFWI_CUDA(rb.mu.alloc(sizeof(double) * E * (n + 2) * nb * B));
     SBFWI_CUDA(rb.vbn.alloc(sizeof(double) * E * nb * B));
     SBFWI_CUDA(rb.ghost.alloc(sizeof(double) * E * 2 * nb * B));
+    SBFWI_CUDA(rb.gprod.alloc(sizeof(double) * E * (n + 3) * 4 * m.L * (m.p + 1) * (m.p + 1)));
     SBFWI_CUDA(rb.gacc.alloc(sizeof(double) * E * (n + 1) * 4 * m.L * ng));
     SBFWI_CUDA(rb.gbnd.alloc(sizeof(double) * E * nb));
     SBFWI_CUDA(rb.grad_int.alloc(sizeof(double) * np));
-    for (DevBuf* b : {&rb.mu, &rb.vbn, &rb.ghost, &rb.gacc, &rb.gbnd, &rb.grad_int})
+    for (DevBuf* b : {&rb.mu, &rb.vbn, &rb.ghost, &rb.gprod, &rb.gacc, &rb.gbnd, &rb.grad_int})
       SBFWI_CUDA(cudaMemsetAsync(b->p, 0, b->bytes, st));
   }
   int rc = zero_state();
@@ -1765,15 +1766,11 @@ int Stepper::init() {
     xba.ub = rb.ub.as<double>(); xba.udb = rb.udb.as<double>(); xba.uddb = rb.uddb.as<double>();
     xba.ext = rb.ext.as<double>(); xba.vbn = rb.vbn.as<double>();
     xba.inc_ptr = md.dev().inc_ptr.as<int64_t>(); xba.inc_list = md.dev().inc_list.as<int64_t>();
-    int Bp = 1;
-    while (Bp < B) Bp <<= 1;
-    xga.E = E; xga.N = N; xga.nb = nb; xga.n = n; xga.B = B; xga.Bp = Bp; xga.L = m.L; xga.ng = (3 * m.p + 2) / 2;
-    xga.h = (1.0 - m.xi0) / n;
-    xga.xi = md.dev().xih.as<double>(); xga.tab = md.dev().tab.as<double>();
+    xga.E = E; xga.N = N; xga.nb = nb; xga.n = n; xga.B = B; xga.L = m.L; xga.pp = m.p + 1;
     xga.lptr = md.dev().lptr.as<int64_t>(); xga.line_local = md.dev().lloc.as<int32_t>();
     xga.dofs = md.dev().dofs.as<int32_t>();
     xga.mu = rb.mu.as<double>(); xga.fbar = rb.x.as<double>(); xga.ghost = rb.ghost.as<double>();
-    xga.gacc = rb.gacc.as<double>();
+    xga.prod = rb.gprod.as<double>();
   }
   return SBFWI_OK;
 }
@@ -2029,7 +2026,7 @@ int Stepper::run_exact(int64_t k0, int64_t k1) {
     if (rc) return rc;
     if ((rc = exact_boundary_launch(xba, true, st))) return rc;
     xga.fu_int = fu; xga.fu_b = fu + nint * B; xga.fa_int = fa_; xga.fa_b = fa_ + nint * B;
-    if ((rc = exact_gradient_launch(xga, md.mesh->p, st))) return rc;
+    if ((rc = exact_gradient_launch(xga, st))) return rc;
     prof.count(kPhaseOther, 2);
   }
   SBFWI_CUDA(cudaGetLastError());
@@ -2042,10 +2039,11 @@ int Stepper::finalize_exact() {
   f.E = E; f.nb = nb; f.n = n; f.pp = m.p + 1; f.ng = (3 * m.p + 2) / 2; f.L = m.L;
   f.lptr = md.dev().lptr.as<int64_t>(); f.line_local = md.dev().lloc.as<int32_t>(); f.tab = md.dev().tab.as<double>();
   f.kq = md.kq.as<double>(); f.gacc = rb.gacc.as<double>();
+  f.prod = rb.gprod.as<double>(); f.xi = md.dev().xih.as<double>(); f.h = (1.0 - md.mesh->xi0) / n;
   f.g_nodal = rb.grad_int.as<double>(); f.g_bnd = rb.gbnd.as<double>();
   int rc = exact_finalize_launch(f, md.dev().inc_ptr.as<int64_t>(), md.dev().inc_list.as<int64_t>(), N,
                                  rb.grad_int.as<double>() + nint, st);
-  profiler().count(kPhaseOther, 2);
+  profiler().count(kPhaseOther, 3);
   return rc;
 }
 
