@@ -300,7 +300,7 @@ int lfe_setup_device(Model& md, const double* Emat, double* S, double* M, cudaSt
 // exact discrete adjoint kernels (exact.cu)
 // ---------------------------------------------------------------------------
 struct ExactElemArgs {
-  int nb, n, B, epc;
+  int nb, n, B, epc, sms;
   int64_t E, N;
   double a0, a1, a2;                       // Newmark predictor coefficients
   double cu, cud, cudd, du, dud, dudd;     // u' and u'' of the Newmark update: c_u (u_new - u) + c_ud u' + c_udd u''

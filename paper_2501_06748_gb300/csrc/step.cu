@@ -1749,6 +1749,7 @@ int Stepper::init() {
     const double beta = md.beta, gamma = md.gamma, dt = md.dt;
     xa.nb = nb; xa.n = n; xa.B = B; xa.E = E; xa.N = N;
     xa.epc = std::max(1, 128 / (nb * B));
+    xa.sms = sms;
     xa.a0 = md.a0; xa.a1 = md.a1; xa.a2 = md.a2;
     xa.cu = gamma / (beta * dt); xa.cud = 1.0 - gamma / beta; xa.cudd = dt * (1.0 - gamma / (2.0 * beta));
     xa.du = 1.0 / (beta * dt * dt); xa.dud = -1.0 / (beta * dt); xa.dudd = 1.0 - 1.0 / (2.0 * beta);

@@ -38,3 +38,36 @@ def test_against_the_oracle(lib, nx, ny, p, n_r, shots):
     g = lib.adjoint_gradient(md, st, res, mode=lib.GRAD_EXACT)
     go = modex.misfit_and_gradient(mesh, n_r, 1.0, rho, dt, src, wav, rec, obs)[1]
     assert np.linalg.norm(g - go) <= GRAD_TOL * np.linalg.norm(go)
+
+
+@pytest.mark.parametrize("nx,ny,p,n_r,shots", [
+    (4, 3, 4, 4, 8),      # one element a block, operators copied ahead in 16-byte pieces
+    (4, 3, 1, 3, 2),      # sixteen elements a block, the last block short
+    (3, 2, 5, 3, 5),      # n_b 20
+    (2, 2, 4, 40, 8),     # too many radial points to stage
+    (40, 33, 4, 3, 3),    # more blocks of two elements than fit the SMs at once: direct
+])
+def test_operators_copied_ahead_or_not(lib, nx, ny, p, n_r, shots):
+    """The transposed sweeps against the derivative along one direction: <g, d> and the misfit's central
+    difference (truncation h^2, rounding 1e-13 / h of the misfit: 1e-5 at h = 1e-4)."""
+    mesh = structured_mesh(nx, ny, p)
+    rng = np.random.default_rng(nx)
+    M = lib.Mesh.from_inputs(mesh, n_r)
+    rho, d = 1.0 + 0.3 * rng.random(M.n_nodal), rng.standard_normal(M.n_nodal)
+    s = 1.0 / (max(nx, ny) * p)
+    K, dt = 25, 0.4 * s
+    src = rng.permutation(mesh.n_nodes)[:shots]
+    wav = np.stack([(1 + 0.2 * k) * ricker(1 / (6 * s), dt, K) for k in range(shots)])
+    obs = np.zeros((shots, shots, K))
+
+    def run(r, gradient):
+        md = lib.Model(M, 1.0, r, dt, rho_kind=lib.RHO_NODAL)
+        lib.set_gradient_mode(md, lib.GRAD_EXACT)
+        tr, st = lib.forward(md, src, wav, np.sort(src))
+        E, res = lib.misfit(tr, obs, dt)
+        return E, lib.adjoint_gradient(md, st, res, mode=lib.GRAD_EXACT) if gradient else None
+
+    h = 1e-4
+    g = run(rho, True)[1]
+    fd = (run(rho + h * d, False)[0] - run(rho - h * d, False)[0]) / (2 * h)
+    assert abs(g @ d - fd) <= 1e-5 * abs(fd)
