@@ -224,10 +224,10 @@ int sbfwi_set_model_lfe(sbfwi_model** out, const sbfwi_mesh* mesh, double c, con
  *            most 8 shots run); AUTO picks it for a padded n_b of 17..20 or beyond 32.
  *   solve    SBFWI_SOLVE_AUTO: the dataflow solve (SBFWI_SOLVE=barrier|levels in
  *            the environment selects the others); SBFWI_SOLVE_DATAFLOW: one
- *            cooperative launch, tasks ordered by dependencies; SBFWI_SOLVE_BARRIER:
+ *            launch, tasks ordered by dependencies; SBFWI_SOLVE_BARRIER:
  *            one cooperative launch, grid barriers between tree levels;
  *            SBFWI_SOLVE_LEVELS: one launch per tree level and direction.  The
- *            cooperative schedules need a device that launches cooperatively
+ *            first two need a device that launches cooperatively
  *            (SBFWI_EUNSUPPORTED at the time-loop call otherwise).
  *
  * A checkpointed forward state must be consumed by an adjoint with the same
@@ -439,7 +439,8 @@ void sbfwi_session_destroy(sbfwi_session* session);
  * for a stored field) is kept in a one-slot cache instead of being freed, and the
  * next sbfwi_forward on the same device whose store is at least as large and at
  * most a third larger reuses it (an evaluation loop then allocates it once).
- * sbfwi_release_cache() frees the cached store; a forward that needs a store that
+ * sbfwi_release_cache() frees the cached store, and the partial sums' buffers that
+ * sbfwi_misfit keeps between calls; a forward that needs a store that
  * the cached one does not fit frees the cached one first.  (A service of the
  * library; the paper has no counterpart.)
  */

@@ -1,7 +1,7 @@
 // sbfwi_misfit_noalloc: the misfit reduction without any device allocation.
 //
-// sbfwi_misfit stages its per-block partial sums in a buffer it allocates with
-// cudaMalloc on every call.  Some callers cannot let a library allocate device
+// sbfwi_misfit stages its per-block partial sums in a buffer from a small pool that it
+// fills with cudaMalloc.  Some callers cannot let a library allocate device
 // memory: a host framework that has reserved (nearly) all of HBM in its own
 // caching pool, a real-time loop that must not hit the driver's allocator or
 // its implicit synchronisation, or a process running under a fixed memory

@@ -16,19 +16,17 @@
 //  * each integer is written in six balanced base-512 digits (|digit| <= 257, exact
 //    in FP16): A_int = sum_k a_k 2^(9(6-k)), x_int = sum_l x_l 2^(9(6-l));
 //  * the digit products of one significance level L = k + l are summed by
-//    mma.sync.m16n8k16 (FP16 in, FP32 accumulate) into one accumulator per level;
-//    every partial sum is an integer below 2^24, so the accumulation is exact;
+//    mma.sync.m16n8k16 (FP16 in, FP32 accumulate), at most four products of 16 terms per
+//    accumulator: every partial sum is an integer of at most 2^22, so the accumulation is exact;
 //  * levels L = 2..8 are kept (the dropped ones weigh < 2^-57 of the scale), turned
 //    back into integers, summed in int64 with their weights 2^(9(8-L)), the two lowest
 //    levels rounded once to the nearest unit, and converted once to FP64:
 //    A x ~ 2^(e_r + f - 52) * T'.
 //
 // The splitting of the vectors and the recombination are integer work; what stays on
-// the FP64 pipe is the conversion of each result and the Newmark arithmetic.
-// Shapes: n_b <= 16 (padded to the 16 rows/columns of one m16n8k16 tile) and B <= 8
-// shots (padded to its 8 columns); one warp per element.  The joint product sums two
-// k-tiles into each level: at most 12 digit products of <= 257^2 times 16 terms,
-// 1.3e7 < 2^24, still exact in FP32.
+// the FP64 pipe is the Newmark arithmetic.
+// Shapes: n_b <= 16 (padded to 16) and 3 <= B <= 8 shots (padded to 8) here, n_b 21..32 in
+// tc2.cu, one or two shots in tc_small.cu; one warp per element.
 #include "tc_step.cuh"
 
 namespace sbfwi {
