@@ -31,27 +31,13 @@
 #include <cstdint>
 
 #include "internal.h"
+#include "sync.cuh"
 
 namespace sbfwi {
 
 // ---------------------------------------------------------------------------
 // element kernel: down sweep of step k fused with the up sweep of step k-1
 // ---------------------------------------------------------------------------
-// count doubles global -> shared by nthr threads, asynchronously; in pairs where wide (both addresses on 16 bytes)
-__device__ __forceinline__ void copy_async(double* dst, const double* src, int count, int tid, int nthr, bool wide) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  if (wide) {
-    for (int t = 2 * tid; t < count; t += 2 * nthr)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d + 8 * t), "l"(src + t) : "memory");
-  } else {
-    for (int t = tid; t < count; t += nthr)
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d + 8 * t), "l"(src + t) : "memory");
-  }
-}
-__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int kPending>
-__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(kPending) : "memory"); }
-
 // Bound by the FP64 pipe: four products per radial point and shot.  kStaged: the operators of the next
 // point (G, P, Q down; H up) are copied to shared memory while the current one's products run, in two buffers an
 // element; read straight from memory, their latency left the pipe 71 % busy: 0.42 -> 0.32 ms a step for 576
@@ -454,8 +440,6 @@ __global__ void exact_gather_nodes_kernel(const double* g_bnd, const int64_t* in
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
-constexpr size_t kStagedSmem = 56 * 1024;      // a quarter of an SM's shared memory
-
 int exact_element_launch(const ExactElemArgs& a, cudaStream_t st) {
   const int threads = a.epc * a.nb * a.B;
   const unsigned blocks = (unsigned)((a.E + a.epc - 1) / a.epc);
@@ -465,7 +449,7 @@ int exact_element_launch(const ExactElemArgs& a, cudaStream_t st) {
   // of a step, us: 24 x 24 elements, order 4, 8 shots 389 | 341, order 3, 5 shots 75 | 60; 64 x 64, order 4, 8 shots
   // 2212 | 2148, 3 shots (two elements a block) 1053 | 1072.
   const size_t staged = smem + sizeof(double) * (size_t)a.epc * 6 * a.nb * a.nb;
-  if (staged <= kStagedSmem && (a.epc == 1 || blocks <= 4u * (unsigned)a.sms)) {
+  if (stage_operators(staged, a.epc, blocks, a.sms)) {
     if (staged > 48 * 1024)
       SBFWI_CUDA(cudaFuncSetAttribute(exact_element_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged));
     exact_element_kernel<true><<<blocks, threads, staged, st>>>(a);

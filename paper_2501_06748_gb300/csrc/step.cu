@@ -59,8 +59,12 @@ struct ElemStepArgs {
   int64_t n_elems;
 };
 
+// Bound by the FP64 pipe: three products per radial point and shot.  kStaged: the operators of the next point
+// (H down; P, Q up) are copied to shared memory while the current one's products run, in two buffers an element.
+template <bool kStaged>
 __global__ void __launch_bounds__(512) element_step_kernel(ElemStepArgs a) {
-  extern __shared__ double sh[];
+  extern __shared__ double sh_all[];
+  double* sh = sh_all + (kStaged ? (size_t)a.epc * 4 * a.nb * a.nb : 0);
   const int nb = a.nb, n = a.n, B = a.B;
   const int per = nb * B;
   const int tid = threadIdx.x;
@@ -74,15 +78,35 @@ __global__ void __launch_bounds__(512) element_step_kernel(ElemStepArgs a) {
   const int64_t nn = (int64_t)nb * nb;
   const double* Me = a.mats + (act ? e : 0) * (int64_t)n * 3 * nn;
   const int64_t base = (act ? e : 0) * (int64_t)n * per;    // interior offset of this element
+  double* ops = kStaged ? sh_all + (size_t)le * 4 * nn : nullptr;   // [2][H] or [2][P Q] of this element
+  // point i's operators of either sweep to buffer i & 1
+  auto stage_down = [&](int i) {
+    if constexpr (kStaged) {
+      if (act && i >= 0) copy_async(ops + (i & 1) * 2 * nn, Me + ((int64_t)i * 3 + 2) * nn, (int)nn, rem, per, (nb & 1) == 0);
+      copy_commit();
+    }
+  };
+  auto stage_up = [&](int i) {
+    if constexpr (kStaged) {
+      if (act && i < n) copy_async(ops + (i & 1) * 2 * nn, Me + (int64_t)i * 3 * nn, (int)(2 * nn), rem, per, (nb & 1) == 0);
+      copy_commit();
+    }
+  };
 
   if (a.do_down) {
+    stage_down(n - 1);
     if (act) xb[r * B + s] = a.ub[(int64_t)a.dofs[e * nb + r] * B + s];
-    __syncthreads();
+    if (!kStaged) __syncthreads();
     for (int i = n - 1; i >= 0; --i) {
       double un = 0.0;
+      if constexpr (kStaged) {           // the buffer written was last read before the barrier of the last round
+        stage_down(i - 1);
+        copy_wait<1>();
+        __syncthreads();                 // every thread's copies, and xb
+      }
       if (act) {
         const int64_t o = base + (int64_t)i * per + r * B + s;
-        const double* H = Me + (int64_t)i * 3 * nn + 2 * nn + (int64_t)r * nb;
+        const double* H = (kStaged ? ops + (i & 1) * 2 * nn : Me + (int64_t)i * 3 * nn + 2 * nn) + (int64_t)r * nb;
         double acc = a.q[o];
         for (int c = 0; c < nb; ++c) acc = fma(-H[c], xb[c * B + s], acc);
         un = acc;
@@ -99,7 +123,7 @@ __global__ void __launch_bounds__(512) element_step_kernel(ElemStepArgs a) {
       }
       __syncthreads();
       if (act) xb[r * B + s] = un;
-      __syncthreads();
+      if (!kStaged) __syncthreads();
     }
   } else if (a.do_up && act) {
     for (int i = 0; i < n; ++i) {
@@ -108,6 +132,7 @@ __global__ void __launch_bounds__(512) element_step_kernel(ElemStepArgs a) {
     }
   }
   if (!a.do_up) return;
+  stage_up(0);                           // its buffer was last read before the barrier that ended the last round's products
   if (act) {
     const int64_t g = (int64_t)a.dofs[e * nb + r] * B + s;
     vn[r * B + s] = fma(a.a0, a.ub[g], fma(a.a1, a.udb[g], a.a2 * a.uddb[g]));
@@ -115,8 +140,13 @@ __global__ void __launch_bounds__(512) element_step_kernel(ElemStepArgs a) {
   __syncthreads();
   for (int i = 0; i < n; ++i) {
     double qv = 0.0;
+    if constexpr (kStaged) {
+      stage_up(i + 1);
+      copy_wait<1>();
+      __syncthreads();
+    }
     if (act) {
-      const double* P = Me + (int64_t)i * 3 * nn + (int64_t)r * nb;
+      const double* P = (kStaged ? ops + (i & 1) * 2 * nn : Me + (int64_t)i * 3 * nn) + (int64_t)r * nb;
       const double* v = vbuf + i * per;
       double acc = 0.0;
       for (int c = 0; c < nb; ++c) acc = fma(P[c], v[c * B + s], acc);
@@ -129,8 +159,9 @@ __global__ void __launch_bounds__(512) element_step_kernel(ElemStepArgs a) {
     }
     __syncthreads();
     if (act) xb[r * B + s] = qv;
-    __syncthreads();
+    if (!kStaged) __syncthreads();
   }
+  if (kStaged) __syncthreads();
   if (act) {
     const double* R = a.rt + e * 2 * nn + (int64_t)r * nb;
     const double* T = R + nn;
@@ -1492,6 +1523,7 @@ struct Stepper {
   const Task* ftasks = nullptr;
   const Task* btasks = nullptr;
   size_t s_smem = 0, e_smem = 0;
+  bool e_staged = false;             // the FP64 element kernel's operators are copied ahead
   int e_threads = 0, p_grid = 0;
   unsigned e_blocks = 0, b_blocks = 0;
   DevBuf bar, pstatus;
@@ -1656,11 +1688,17 @@ int Stepper::init() {
   e_blocks = (unsigned)std::max<int64_t>(1, (ea.n_elems + ea.epc - 1) / ea.epc);
   e_smem = sizeof(double) * (size_t)ea.epc * (n + 2) * nb * B;
   cudaFuncAttributes eattr;
-  SBFWI_CUDA(cudaFuncGetAttributes(&eattr, element_step_kernel));
+  SBFWI_CUDA(cudaFuncGetAttributes(&eattr, element_step_kernel<false>));
   if (!use_tc && !md.lfe && (e_threads > eattr.maxThreadsPerBlock || e_smem > 227 * 1024))
     return fail(SBFWI_EUNSUPPORTED, "n_b x shots x radial points too large for one element block: run fewer shots per pass");
+  // a launch direct | staged, us: 24 x 24 elements, order 4, 8 shots 356 | 327, order 3, 5 shots 53 | 49; 20 x 20,
+  // order 5, 7 shots 193 | 173; 64 x 64, order 4, 8 shots 2160 | 2065
+  const size_t staged = e_smem + sizeof(double) * (size_t)ea.epc * 4 * nb * nb;
+  e_staged = stage_operators(staged, ea.epc, e_blocks, sms);
+  if (e_staged) e_smem = staged;
   if (e_smem > 48 * 1024 && !md.lfe)
-    SBFWI_CUDA(cudaFuncSetAttribute(element_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e_smem));
+    SBFWI_CUDA(cudaFuncSetAttribute(e_staged ? element_step_kernel<true> : element_step_kernel<false>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e_smem));
 
   const MeshDevice& mdev = md.dev();
   sa.sep_nodes = md.solve_sep; sa.bnd_nodes = md.solve_bnd;
@@ -1886,7 +1924,8 @@ int Stepper::element_launch(int down, int up, int64_t done_step) {
     l.status = pstatus.as<int>();
     tc_element_launch(md, l, st);
   }
-  if (!use_tc && (!use_mixed || n_fp > 0)) element_step_kernel<<<e_blocks, e_threads, e_smem, st>>>(ea);
+  if (!use_tc && (!use_mixed || n_fp > 0))
+    (e_staged ? element_step_kernel<true> : element_step_kernel<false>)<<<e_blocks, e_threads, e_smem, st>>>(ea);
   prof.end(kPhaseElement, st);
   prof.count(kPhaseElement, use_mixed ? 2 : 1);
   if (grad_term) {

@@ -35,6 +35,27 @@ cudaError_t launch_next(void (*kernel)(Params...), unsigned grid, unsigned block
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// count doubles global -> shared by nthr threads, asynchronously; in pairs where wide (both addresses on 16 bytes)
+__device__ __forceinline__ void copy_async(double* dst, const double* src, int count, int tid, int nthr, bool wide) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  if (wide) {
+    for (int t = 2 * tid; t < count; t += 2 * nthr)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d + 8 * t), "l"(src + t) : "memory");
+  } else {
+    for (int t = tid; t < count; t += nthr)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d + 8 * t), "l"(src + t) : "memory");
+  }
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int kPending>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(kPending) : "memory"); }
+
+// FP64 element kernels: operators copied ahead where they leave room for four blocks on an SM and either all
+// blocks are on the SMs at once anyway or a block is one element (figures at the launches)
+inline bool stage_operators(size_t smem, int elements_per_block, unsigned blocks, int sms) {
+  return smem <= 56 * 1024 && (elements_per_block == 1 || blocks <= 4u * (unsigned)sms);
+}
+
 // Grid-wide barrier for a cooperative launch (all blocks co-resident).  The wait
 // is bounded: after `budget` clock cycles it records SBFWI_ETIMEOUT and gives up,
 // so a broken launch returns an error instead of hanging the device.
