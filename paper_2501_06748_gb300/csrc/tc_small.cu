@@ -18,8 +18,11 @@ namespace tc {
 
 constexpr int kSmallShots = 2;
 
-// digits of one operand [shot][5 zero rows, digits 0..5, zero row][4 lanes t: rows 2t, 2t+1, 2t+8, 2t+9]
-constexpr int kDigitRows = 12;
+// digits of one operand [shot][5 zero rows, digits 0..5, zero rows][4 lanes t: rows 2t, 2t+1, 2t+8, 2t+9]; level
+// row g of the fragment for operator digit k reads row kZeroRows + g - k, g 0..7 (level 7 is formed and not kept)
+constexpr int kZeroRows = kSlices - 1, kDigitRows = kZeroRows + kTile / 2;
+static_assert(kZeroRows + kSlices <= kDigitRows && kZeroRows >= kSlices - 1 && kZeroRows + 7 < kDigitRows,
+              "a row for every digit and for every level row that is read");
 struct SmallDigits {
   __half d[kSmallShots][kDigitRows][kTile];
 };
@@ -51,8 +54,8 @@ __device__ __forceinline__ void put_digits(SmallDigits& D, double x, int E, int 
   const unsigned h[3] = {unbias(w54, 0x65006500u), unbias(w32, 0x65006500u), unbias(w10, 0x66006500u)};
 #pragma unroll
   for (int p = 0; p < 3; ++p) {
-    D.d[s][5 + 5 - 2 * p][at] = __ushort_as_half((unsigned short)(h[p] & 0xFFFFu));
-    D.d[s][5 + 4 - 2 * p][at] = __ushort_as_half((unsigned short)(h[p] >> 16));
+    D.d[s][kZeroRows + 5 - 2 * p][at] = __ushort_as_half((unsigned short)(h[p] & 0xFFFFu));
+    D.d[s][kZeroRows + 4 - 2 * p][at] = __ushort_as_half((unsigned short)(h[p] >> 16));
   }
 }
 
@@ -78,8 +81,8 @@ __device__ __forceinline__ double small_product(const SmallDigits* D, int* lev, 
     const uint2* b = (op == 0 ? b0 : b1) + lane;
 #pragma unroll
     for (int k = 0; k < kSlices; ++k) {
-      const uint2 x0 = *reinterpret_cast<const uint2*>(&D[op].d[0][g + 5 - k][4 * t]);
-      const uint2 x1 = *reinterpret_cast<const uint2*>(&D[op].d[1][g + 5 - k][4 * t]);
+      const uint2 x0 = *reinterpret_cast<const uint2*>(&D[op].d[0][kZeroRows + g - k][4 * t]);
+      const uint2 x1 = *reinterpret_cast<const uint2*>(&D[op].d[1][kZeroRows + g - k][4 * t]);
       const uint4 x = make_uint4(x0.x, x1.x, x0.y, x1.y);
       const int pos = op * kSlices + k;
 #pragma unroll
