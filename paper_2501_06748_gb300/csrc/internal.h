@@ -381,6 +381,7 @@ int tc_prepare_one_tile(Model& md, cudaStream_t st);   // one-tile digits even w
 constexpr int kTileShots = 8;
 struct TcState {
   bool tiles = false;
+  int rows = 0;           // of one point: 16 or 32 (tiles), or n_b
   int doubles = 0;        // of one point
 };
 TcState tc_state(const Model& md, int B, int64_t n_elems, int sms);

@@ -1004,7 +1004,9 @@ __global__ void boundary_update_kernel(BoundaryArgs a) {
 __device__ __forceinline__ int tile_place(int row, int s) { return ((row >> 1) * kTileShots + s) * 2 + (row & 1); }
 
 // The per-shot gradient accumulators: rows [row][shot] from nodal point row0 on, and those of the
-// interior points of the tensor-core kernels' elements, in their state's layout
+// interior points of the tensor-core kernels' elements, in their state's layout.  On a mesh padded beyond
+// the class's tile (mixed kernels: 16 rows a tile, nb 17 and more) the rows past the tile are padding of
+// the class's elements and have no place in it: theirs is the one in acc, which holds every nodal point then.
 struct GradCells {
   double* acc;              // [n_nodal - row0][B]
   int64_t row0;
@@ -1019,7 +1021,7 @@ __device__ __forceinline__ double* grad_cell(const GradCells& g, int64_t q, int 
     const int64_t ei = q / g.nb, e = ei / g.n;
     const int64_t t = g.place ? (int64_t)g.place[e] : e;
     const int row = (int)(q - ei * g.nb);
-    if (t >= 0)
+    if (t >= 0 && row < g.state.rows)
       return g.tc + (t * g.n + (ei - e * g.n)) * g.state.doubles + (g.state.tiles ? tile_place(row, s) : row * g.B + s);
   }
   return g.acc + (q - g.row0) * g.B + s;

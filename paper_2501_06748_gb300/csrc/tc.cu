@@ -83,6 +83,7 @@ TcState tc_state(const Model& md, int B, int64_t n_elems, int sms) {
   const int rows = tc_tile_rows(md), nb = md.nb;
   const double most = n_elems <= kFewElements * (int64_t)sms ? 5.4 : rows > tc::kTile ? 2.0 : 1.1;
   t.tiles = rows * kTileShots <= most * nb * B && !(rows == tc::kTile && B <= kFewShots);
+  t.rows = t.tiles ? rows : nb;
   t.doubles = t.tiles ? rows * kTileShots : nb * B;
   return t;
 }
