@@ -440,6 +440,15 @@ __global__ void exact_gather_nodes_kernel(const double* g_bnd, const int64_t* in
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
+int exact_prepare_launches() {
+  for (const void* f : {(const void*)exact_element_kernel<false>, (const void*)exact_element_kernel<true>,
+                        (const void*)exact_gradient_kernel}) {
+    const int rc = allow_shared_memory(f);
+    if (rc) return rc;
+  }
+  return SBFWI_OK;
+}
+
 int exact_element_launch(const ExactElemArgs& a, cudaStream_t st) {
   const int threads = a.epc * a.nb * a.B;
   const unsigned blocks = (unsigned)((a.E + a.epc - 1) / a.epc);
@@ -450,12 +459,8 @@ int exact_element_launch(const ExactElemArgs& a, cudaStream_t st) {
   // 2212 | 2148, 3 shots (two elements a block) 1053 | 1072.
   const size_t staged = smem + sizeof(double) * (size_t)a.epc * 6 * a.nb * a.nb;
   if (stage_operators(staged, a.epc, blocks, a.sms)) {
-    if (staged > 48 * 1024)
-      SBFWI_CUDA(cudaFuncSetAttribute(exact_element_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged));
     exact_element_kernel<true><<<blocks, threads, staged, st>>>(a);
   } else {
-    if (smem > 48 * 1024)
-      SBFWI_CUDA(cudaFuncSetAttribute(exact_element_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     exact_element_kernel<false><<<blocks, threads, smem, st>>>(a);
   }
   SBFWI_CUDA(cudaGetLastError());
@@ -485,8 +490,6 @@ int exact_boundary_launch(const ExactBoundaryArgs& a, bool post, cudaStream_t st
 int exact_gradient_launch(const ExactGradArgs& a, cudaStream_t st) {
   if (a.pp < 2 || a.pp > 9) return fail(SBFWI_EUNSUPPORTED, "line order outside 1..8");
   const size_t smem = sizeof(double) * (size_t)a.B * (5 * (size_t)a.nb + 3 * (size_t)a.L * a.pp);
-  if (smem > 48 * 1024)
-    SBFWI_CUDA(cudaFuncSetAttribute(exact_gradient_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   exact_gradient_kernel<<<(unsigned)(a.E * (a.n + 3)), 128, smem, st>>>(a);
   SBFWI_CUDA(cudaGetLastError());
   return SBFWI_OK;

@@ -363,6 +363,7 @@ struct ExactFinalArgs {
 };
 
 size_t exact_element_smem(int nb, int n, int B, int epc);
+int exact_prepare_launches();   // before the launches of a time loop
 int exact_element_launch(const ExactElemArgs& a, cudaStream_t st);
 int exact_misfit_launch(double* ub, int B, int R, const int64_t* rec, const double* res, int64_t K, int64_t k, double dt,
                         cudaStream_t st);

@@ -1834,7 +1834,8 @@ static int launch_element_setup(Model& md, const Mesh& m, const double* rho_hi, 
   const bool in_smem = smem_all <= 160 * 1024;
   a.scratch = (int)(in_smem ? scratch_smem : temps);
   const size_t smem = in_smem ? smem_all : tables + sizeof(dd) * temps;
-  SBFWI_CUDA(cudaFuncSetAttribute(element_setup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int rc_s = allow_shared_memory((const void*)element_setup_kernel);
+  if (rc_s) return rc_s;
   cudaFuncAttributes fattr;
   SBFWI_CUDA(cudaFuncGetAttributes(&fattr, element_setup_kernel));
   int threads = (int)std::min<int64_t>((nn + 31) / 32 * 32, fattr.maxThreadsPerBlock / 32 * 32);

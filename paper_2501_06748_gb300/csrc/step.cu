@@ -1667,8 +1667,9 @@ int Stepper::init() {
   if (s_smem > 226 * 1024) return fail(SBFWI_EUNSUPPORTED, "solve staging area exceeds shared memory");
   for (const void* f : {(const void*)solve_forward_kernel, (const void*)solve_backward_kernel,
                         (const void*)solve_persistent_kernel, (const void*)solve_flow_kernel<false>,
-                        (const void*)solve_flow_kernel<true>})
-    if (s_smem > 48 * 1024) SBFWI_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_smem));
+                        (const void*)solve_flow_kernel<true>, (const void*)element_step_kernel<false>,
+                        (const void*)element_step_kernel<true>})
+    if ((rc = allow_shared_memory(f))) return rc;
 
   ea.nb = nb; ea.n = n; ea.B = B; ea.E = E;
   ea.epc = std::max(1, 128 / (nb * B));
@@ -1698,9 +1699,6 @@ int Stepper::init() {
   const size_t staged = e_smem + sizeof(double) * (size_t)ea.epc * 4 * nb * nb;
   e_staged = stage_operators(staged, ea.epc, e_blocks, sms);
   if (e_staged) e_smem = staged;
-  if (e_smem > 48 * 1024 && !md.lfe)
-    SBFWI_CUDA(cudaFuncSetAttribute(e_staged ? element_step_kernel<true> : element_step_kernel<false>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e_smem));
 
   const MeshDevice& mdev = md.dev();
   sa.sep_nodes = md.solve_sep; sa.bnd_nodes = md.solve_bnd;
@@ -1801,6 +1799,7 @@ int Stepper::init() {
     xa.fu_int = xa.fu_b = xa.fa_b = nullptr;
     if (xa.epc * nb * B > 512 || exact_element_smem(nb, n, B, xa.epc) > 227 * 1024)
       return fail(SBFWI_EUNSUPPORTED, "n_b x shots x radial points too large for one element block of the exact adjoint");
+    if ((rc = exact_prepare_launches())) return rc;
     xba.N = N; xba.B = B;
     xba.a0 = md.a0; xba.a1 = md.a1; xba.a2 = md.a2;
     xba.cu = xa.cu; xba.cud = xa.cud; xba.cudd = xa.cudd; xba.du = xa.du; xba.dud = xa.dud; xba.dudd = xa.dudd;

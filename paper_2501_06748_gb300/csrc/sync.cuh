@@ -50,6 +50,21 @@ __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_gr
 template <int kPending>
 __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(kPending) : "memory"); }
 
+// Lets a kernel be launched with as much dynamic shared memory as the device has.  The limit belongs to the kernel,
+// for all that use it in the process: were it set to what one caller needs, it would be lowered under the launches
+// of others (a session keeps its own; other threads).
+inline int allow_shared_memory(const void* kernel) {
+  int device = 0, most = 0;
+  SBFWI_CUDA(cudaGetDevice(&device));
+  SBFWI_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
+  cudaFuncAttributes at;
+  SBFWI_CUDA(cudaFuncGetAttributes(&at, kernel));
+  const int limit = most - (int)at.sharedSizeBytes;
+  if (at.maxDynamicSharedSizeBytes < limit)
+    SBFWI_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
+  return SBFWI_OK;
+}
+
 // FP64 element kernels: operators copied ahead where they leave room for four blocks on an SM and either all
 // blocks are on the SMs at once anyway or a block is one element (figures at the launches)
 inline bool stage_operators(size_t smem, int elements_per_block, unsigned blocks, int sms) {
