@@ -216,6 +216,19 @@ __device__ __forceinline__ int column_scale2(double (&v)[kV], double (&q)[kV], i
   return ex < kMinExp ? 1022 : ex;
 }
 
+// The exponent at which q's digits of the joint operand are taken, E - bal; where it is too small for that q is
+// scaled up first, exactly, which leaves its digits as they are (q is below 2^-958 then; units in which P is 2^-64
+// of Q and fields near the bottom of the range)
+template <int kV>
+__device__ __forceinline__ int joint_q_exp(double (&q)[kV], int e) {
+  if (e < kMinExp) {
+#pragma unroll
+    for (int j = 0; j < kV; ++j) q[j] *= 0x1p256;
+    e = max(e + kScaleBits, kMinExp);
+  }
+  return e;
+}
+
 // mma of a digit pair fragment and an operator digit, on top of c (kFirst: of the start value)
 template <bool kFirst>
 __device__ __forceinline__ void mma_pair(float (&c)[4], const uint4& a, const uint2& b, const float (&start)[4]) {

@@ -219,7 +219,9 @@ element_step_small_kernel(ElemTcArgs a) {
     int adj;
     const int E = small_scale2(v, x, bal, adj);
     put_digits(M.dig[0], v, E, s, row);
-    put_digits(M.dig[1], x, max(E - bal, kMinExp), s, row);
+    double xq[1] = {x};
+    const int Eq = joint_q_exp<1>(xq, E - bal);
+    put_digits(M.dig[1], xq[0], Eq, s, row);
     x = small_product<2, true>(M.dig, M.lev, ring.frags(s0), ring.frags(s1), er, E - 1022 - adj, lane,
                                [&] { ring.template release<2>(lane); });
     if (ok) a.l.q[p] = x;

@@ -331,8 +331,9 @@ element_step_tc_kernel(ElemTcArgs a) {
     XDigits d[2 * kRT];
 #pragma unroll
     for (int r = 0; r < kRT; ++r) split_rows(v + 4 * r, E, d[r]);
+    const int Eq = joint_q_exp<kV>(x, E - bal);
 #pragma unroll
-    for (int r = 0; r < kRT; ++r) split_rows(x + 4 * r, max(E - bal, kMinExp), d[kRT + r]);
+    for (int r = 0; r < kRT; ++r) split_rows(x + 4 * r, Eq, d[kRT + r]);
     product<kRT, 2, true>(
         ring.frags(s0), ring.frags(s1), ring.exps(s0), d, E - 1022 - adj, lane, start,
         [&] { ring.template release<2>(lane); },
