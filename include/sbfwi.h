@@ -144,7 +144,9 @@ int sbfwi_build_mesh3d(sbfwi_mesh** out, const double* node_xyz, int64_t n_nodes
 
 /* info[0..7] = n_elem, n_nodes, n_b (the largest), N_r, n_nodal (= n_int + n_nodes),
  * n_int (= (N_r - 1) x the sum of n_b(e)), levels of the global elimination tree,
- * nonzeros kept by the global factors. */
+ * entries (8 bytes each) of the global factors that every model on the mesh keeps.  The
+ * mesh's set-up workspaces (fronts, updates, and factors merged into those) stay with
+ * the mesh from its first model on and are not counted. */
 int sbfwi_mesh_info(const sbfwi_mesh* mesh, int64_t* info);
 void sbfwi_destroy_mesh(sbfwi_mesh* mesh);
 

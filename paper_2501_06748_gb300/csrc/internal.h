@@ -119,7 +119,7 @@ struct Tree {
   std::vector<int32_t> map0, map1;     // per front position: child0 / child1 bnd index, -1 if absent;
                                        // leaves: map0 = local dof of the element
   std::vector<std::vector<int32_t>> nodes_at_level;
-  int64_t X_total = 0, F_total = 0, U_total = 0;
+  int64_t F_total = 0, U_total = 0;
   int64_t W_total = 0;                 // set-up workspace for factors that are merged further
   // the tree of the solve: groups of the nodes above, children before parents
   std::vector<SolveNode> snodes;
@@ -132,7 +132,8 @@ struct Tree {
   std::vector<Src4> ssrc;
   std::vector<int32_t> smore;
   std::vector<std::vector<int32_t>> snodes_at_level;
-  int64_t sX_total = 0, sep_rows = 0, bnd_rows = 0;
+  int64_t sX_total = 0;                // factor entries of the solve's nodes, which a model keeps
+  int64_t sep_rows = 0, bnd_rows = 0;
   std::vector<int32_t> sep_owner;      // per global node: tree node that eliminates it
 };
 

@@ -308,7 +308,7 @@ int build_tree(Mesh& m) {
   // node records, maps and offsets
   t.nodes.resize(T);
   t.level_of.assign(T, 0);
-  int64_t sep_off = 0, bnd_off = 0, map_off = 0, X_off = 0, F_off = 0, U_off = 0;
+  int64_t sep_off = 0, bnd_off = 0, map_off = 0, F_off = 0, U_off = 0;
   for (int nd = 0; nd < T; ++nd) {
     TreeNodeDev& r = t.nodes[nd];
     r.s = (int32_t)sep[nd].size();
@@ -319,12 +319,10 @@ int build_tree(Mesh& m) {
     r.sep_off = sep_off;
     r.bnd_off = bnd_off;
     r.map_off = map_off;
-    r.X_off = X_off;
     r.F_off = F_off;
     r.U_off = U_off;
     const int64_t s = r.s, b = r.b, f = s + b;
     sep_off += s; bnd_off += b; map_off += f;
-    X_off += s * s + 2 * s * b;
     F_off += f * f;
     U_off += b * b;
     t.sep_nodes.insert(t.sep_nodes.end(), sep[nd].begin(), sep[nd].end());
@@ -354,7 +352,6 @@ int build_tree(Mesh& m) {
   t.levels = t.level_of[root] + 1;
   t.nodes_at_level.assign(t.levels, {});
   for (int nd = 0; nd < T; ++nd) t.nodes_at_level[t.level_of[nd]].push_back(nd);
-  t.X_total = X_off;
   t.F_total = F_off;
   t.U_total = U_off;
   if (sep_off != m.n_nodes) return fail(SBFWI_EINVAL, "internal: separators do not cover the nodes");
@@ -744,7 +741,7 @@ int sbfwi_mesh_info(const sbfwi_mesh* m, int64_t* info) {
   info[4] = m->n_nodal_api;
   info[5] = m->n_int_api;
   info[6] = m->tree.levels;
-  info[7] = m->tree.X_total;
+  info[7] = m->tree.sX_total;
   return SBFWI_OK;
 }
 
