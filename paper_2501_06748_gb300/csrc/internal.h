@@ -273,8 +273,10 @@ struct Model {
   // the same operators split into FP16 digits for the tensor-core element kernels: one block
   // (digits, row exponents; tc::OpBlock) per operator, [E][P_0 Q_0 H_0 .. H_{n-1} R T]
   DevBuf tc_ops;
-  bool tc_ready = false;
-  bool tc_one_tile = false;   // tc_ops holds one-tile digits although nb > 16 (mixed element kernels)
+  // the one-tile digits of the elements with n_b <= 16 where nb is beyond (mixed element kernels).  Both sets stay
+  // once made: a session's launches go on with theirs when a later call on the model takes the other kernels.
+  DevBuf tc_ops_one;
+  bool tc_ready = false, tc_one_ready = false;
   DevBuf rho_lo;           // [n_nodal] low part of the set-up's double-double density (re-runs of the set-up)
   // exact discrete adjoint (sbfwi_set_gradient_mode(EXACT)): operators the set-up emits on request
   int grad_mode = SBFWI_GRAD_KERNEL;
@@ -377,7 +379,7 @@ int exact_finalize_launch(const ExactFinalArgs& a, const int64_t* inc_ptr, const
 bool tc_supported(int nb, int B);   // the tensor-core kernel is the default for these shapes
 bool tc_available(int nb, int B);   // a tensor-core kernel exists for these shapes
 int tc_prepare(Model& md, cudaStream_t st);
-int tc_prepare_one_tile(Model& md, cudaStream_t st);   // one-tile digits even when n_b is padded beyond 16
+int tc_prepare_one_tile(Model& md, cudaStream_t st);   // one-tile digits of a mesh padded beyond 16 (tc_ops_one)
 // The interior state of the tensor-core element kernels, per element and radial point: whole tiles
 // [16 or 32 rows / 2][8 shots][2], zero beyond n_b(e) and the shots of the pass, or [n_b][B]
 constexpr int kTileShots = 8;
@@ -386,10 +388,11 @@ struct TcState {
   int rows = 0;           // of one point: 16 or 32 (tiles), or n_b
   int doubles = 0;        // of one point
 };
-TcState tc_state(const Model& md, int B, int64_t n_elems, int sms);
+TcState tc_state(const Model& md, int B, int64_t n_elems, int sms, bool one_tile);
 struct TcLaunch {
   int B, do_down, do_up;
   bool tiles;             // the layout of the state (TcState)
+  bool one_tile;          // the operators are Model::tc_ops_one
   double* v; double* z;   // the predictor v and z = u' + dt (1 - gamma) u'' (u, u'' are not kept)
   double* q;
   double* grad;           // adjoint: gradient accumulators, in the state's layout (nullable)

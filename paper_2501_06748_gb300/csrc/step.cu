@@ -1590,12 +1590,12 @@ int Stepper::init() {
   if (md.elem_pref == SBFWI_ELEMENT_AUTO && mixed_ok && !tc_supported(nb, B) &&
       !(elem_env && std::strcmp(elem_env, "fp64") == 0))
     use_mixed = true;                // padded n_b 17..20 or beyond 32
-  if (use_tc && (!md.tc_ready || md.tc_one_tile)) {
+  if (use_tc && !md.tc_ready) {
     const int rc_tc = tc_prepare(md, st);
     if (rc_tc) return rc_tc;
   }
   if (use_mixed) {
-    if (!md.tc_ready || !md.tc_one_tile) {
+    if (!md.tc_one_ready) {
       const int rc_tc = tc_prepare_one_tile(md, st);
       if (rc_tc) return rc_tc;
     }
@@ -1618,7 +1618,7 @@ int Stepper::init() {
   for (DevBuf* b : {&rb.u, &rb.ud, &rb.udd, &rb.q}) SBFWI_CUDA(b->alloc(sizeof(double) * si_state));
   const int64_t n_state = use_tc ? E : use_mixed ? n_tc : 0;
   if (n_state > 0) {
-    tcs = tc_state(md, B, n_state, sms);
+    tcs = tc_state(md, B, n_state, sms, use_mixed);
     const size_t bytes = sizeof(double) * (size_t)n_state * n * tcs.doubles;
     for (DevBuf* b : {&rb.tv, &rb.tz, &rb.tq}) SBFWI_CUDA(b->alloc(bytes));
     if (mode == Mode::Adjoint) {
@@ -1914,7 +1914,7 @@ int Stepper::element_launch(int down, int up, int64_t done_step) {
   prof.begin(kPhaseElement, st);
   if (use_tc || use_mixed) {
     TcLaunch l;
-    l.B = B; l.do_down = down; l.do_up = up; l.tiles = tcs.tiles;
+    l.B = B; l.do_down = down; l.do_up = up; l.tiles = tcs.tiles; l.one_tile = use_mixed;
     l.v = rb.tv.as<double>(); l.z = rb.tz.as<double>(); l.q = rb.tq.as<double>();
     l.grad = ea.fwd_int ? rb.tg.as<double>() : nullptr;
     l.ub = ea.ub; l.udb = ea.udb; l.uddb = ea.uddb; l.fhat = ea.fhat;

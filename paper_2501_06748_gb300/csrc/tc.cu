@@ -50,37 +50,38 @@ bool tc_supported(int nb, int B) {
 }
 bool tc_available(int nb, int B) { return nb <= 2 * tc::kTile && B <= tc::kCols; }
 
+static int prepare_one_tile(Model& md, DevBuf& ops, cudaStream_t st) {
+  const int rc = tc_prepare_tiles<1>(md, ops, st);
+  return rc ? rc : tc_small_prepare();
+}
+
 int tc_prepare(Model& md, cudaStream_t st) {
-  if (md.nb <= tc::kTile) return tc_prepare_one_tile(md, st);
-  const int rc = tc2_prepare(md, st);
-  if (rc) return rc;
-  md.tc_ready = true;
-  md.tc_one_tile = false;
-  return SBFWI_OK;
+  const int rc = md.nb <= tc::kTile ? prepare_one_tile(md, md.tc_ops, st) : tc2_prepare(md, st);
+  md.tc_ready = rc == SBFWI_OK;
+  return rc;
 }
 
 // One-tile digits of every element's operators (their top-left 16 x 16 block; for a mesh
 // padded beyond 16 this is the whole operator of its elements with n_b <= 16, whose padded
 // rows and columns are zero)
 int tc_prepare_one_tile(Model& md, cudaStream_t st) {
-  int rc = tc_prepare_tiles<1>(md, st);
-  if (rc == SBFWI_OK) rc = tc_small_prepare();
-  if (rc) return rc;
-  md.tc_ready = true;
-  md.tc_one_tile = md.nb > tc::kTile;
-  return SBFWI_OK;
+  const int rc = prepare_one_tile(md, md.tc_ops_one, st);
+  md.tc_one_ready = rc == SBFWI_OK;
+  return rc;
 }
 
-int tc_tile_rows(const Model& md) { return md.nb > tc::kTile && !md.tc_one_tile ? 2 * tc::kTile : tc::kTile; }
+static int tc_tile_rows(const Model& md, bool one_tile) {
+  return md.nb > tc::kTile && !one_tile ? 2 * tc::kTile : tc::kTile;
+}
 
 // Whole tiles save the bounds checks, rows save the traffic of the padding.  Fused launches, tiles | rows, ms:
 // 24 x 24 elements, N_r 16: n_b 16, 8 shots 0.055 | 0.060, n_b 8, 3 shots (5.3 times the values) 0.053 | 0.054,
 // n_b 4, 3 shots (10.7 times) 0.053 | 0.053, n_b 4, 1 shot 0.053 | 0.051; 64 x 64 elements: n_b 16, 8 shots
 // 0.217 | 0.219, 5 shots (1.6 times) 0.212 | 0.203, n_b 8, 8 shots (twice) 0.211 | 0.198.  Two tiles, 32 x 32
 // elements: n_b 24, 8 shots 0.243 | 0.254, n_b 32, 4 shots (twice) 0.243 | 0.249.
-TcState tc_state(const Model& md, int B, int64_t n_elems, int sms) {
+TcState tc_state(const Model& md, int B, int64_t n_elems, int sms, bool one_tile) {
   TcState t;
-  const int rows = tc_tile_rows(md), nb = md.nb;
+  const int rows = tc_tile_rows(md, one_tile), nb = md.nb;
   const double most = n_elems <= kFewElements * (int64_t)sms ? 5.4 : rows > tc::kTile ? 2.0 : 1.1;
   t.tiles = rows * kTileShots <= most * nb * B && !(rows == tc::kTile && B <= kFewShots);
   t.rows = t.tiles ? rows : nb;
@@ -93,7 +94,7 @@ int tc_element_launch(const Model& md, const TcLaunch& l, cudaStream_t st) {
   a.l = l;
   a.nb = md.nb; a.n = md.n; a.E = md.E;
   a.a0 = md.a0; a.a1 = md.a1; a.a2 = md.a2; a.c1 = md.c1; a.c2 = md.c2; a.dt = md.dt;
-  a.ops = md.tc_ops.as<unsigned char>();
+  a.ops = (l.one_tile ? md.tc_ops_one : md.tc_ops).as<unsigned char>();
   a.dofs = md.dev().dofs.as<int32_t>();
   if (!l.elems) a.l.n_elems = md.E;
   if (a.l.n_elems == 0) return SBFWI_OK;
@@ -101,7 +102,7 @@ int tc_element_launch(const Model& md, const TcLaunch& l, cudaStream_t st) {
   const bool avg = md.a2 == 1.0 && md.c1 == md.c2;
   // one 16-row tile: n_b <= 16, or the elements of n_b <= 16 of a mesh padded beyond (the
   // one-tile digits of its operators, prepared by tc_prepare_one_tile)
-  if (tc_tile_rows(md) > tc::kTile) tc2_element_launch(a, avg, st);
+  if (tc_tile_rows(md, l.one_tile) > tc::kTile) tc2_element_launch(a, avg, st);
   else if (l.B <= kFewShots) tc_small_launch(a, avg, st);
   else tc_launch_tiles<1>(a, avg, st);
   return SBFWI_OK;

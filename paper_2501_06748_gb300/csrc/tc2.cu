@@ -7,7 +7,7 @@
 
 namespace sbfwi {
 
-int tc2_prepare(Model& md, cudaStream_t st) { return tc_prepare_tiles<2>(md, st); }
+int tc2_prepare(Model& md, cudaStream_t st) { return tc_prepare_tiles<2>(md, md.tc_ops, st); }
 
 void tc2_element_launch(const ElemTcArgs& a, bool avg_accel, cudaStream_t st) {
   tc_launch_tiles<2>(a, avg_accel, st);

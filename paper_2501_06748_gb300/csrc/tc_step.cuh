@@ -384,14 +384,14 @@ constexpr int tc_block_smem() {
 }
 
 template <int kRT>
-int tc_prepare_tiles(Model& md, cudaStream_t st) {
+int tc_prepare_tiles(Model& md, DevBuf& ops, cudaStream_t st) {
   using namespace tc;
   const int64_t warps = md.E * (3 * (int64_t)md.n + 2);
-  SBFWI_CUDA(md.tc_ops.alloc((size_t)warps * OpBlock<kRT>::kBytes));
+  SBFWI_CUDA(ops.alloc((size_t)warps * OpBlock<kRT>::kBytes));
   SliceArgs a;
   a.nb = md.nb; a.n = md.n; a.E = md.E;
   a.mats = md.mats.as<double>(); a.rt = md.rt.as<double>();
-  a.ops = md.tc_ops.as<unsigned char>();
+  a.ops = ops.as<unsigned char>();
   slice_operators_kernel<kRT><<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(a);
   profiler().count(kPhaseSetup);
   SBFWI_CUDA(cudaGetLastError());

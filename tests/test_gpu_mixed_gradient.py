@@ -75,3 +75,24 @@ def test_adjoint_session(lib, n_b):
         tr, st = lib.forward(md, src[k:k + 1], wav[k:k + 1], rec)
         solo = lib.adjoint_gradient(md, st, -tr)
         assert np.abs(adj.collect(k).cpu().numpy() - solo).max() <= 1e-12 * np.abs(solo).max()
+
+
+@pytest.mark.parametrize("first,then", [("MIXED", "TENSOR"), ("TENSOR", "MIXED")])
+def test_session_goes_on_with_its_kernels(lib, first, then):
+    """A session's operator digits outlive a later call on the model that takes the other kernels' digits."""
+    m = _mesh(24)
+    rho, dt, src, wav, rec = _problem(m, 4)
+    md = lib.Model(lib.Mesh.from_inputs(m, 5), 1.0, rho, dt)
+    lib.set_schedule(md, getattr(lib, "ELEMENT_" + first))
+    solo = lib.forward(md, src, wav, rec, keep=False)[0]
+    ses = lib.Session(md, lib.SESSION_FORWARD, 4, rec, window=8)
+    lib.set_schedule(md, getattr(lib, "ELEMENT_" + then))
+    for k in range(4):
+        ses.admit(k, wav[k], int(src[k]))
+    done = []
+    while len(done) < 4:
+        other = lib.forward(md, src, wav, rec, keep=False)[0]
+        assert np.linalg.norm(other - solo) <= 1e-12 * np.linalg.norm(solo)       # the kernels' agreement
+        done = ses.step()
+    for k in range(4):
+        assert np.abs(ses.collect(k).cpu().numpy() - solo[k]).max() <= 1e-13 * np.abs(solo).max()
