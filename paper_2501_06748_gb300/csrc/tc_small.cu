@@ -127,15 +127,9 @@ __device__ __forceinline__ int small_scale(double& x, int& adj) {
   }
   return ex < kMinExp ? 1022 : ex;
 }
-__device__ __forceinline__ int small_scale2(double& v, double& q, int bal, int& adj) {
-  auto ex_of = [&] { return half_max(max(exp_of_key(mag_key(v)), exp_of_key(mag_key(q)) + bal)); };
-  int ex = ex_of();
-  adj = 0;
-  if (__any_sync(0xffffffffu, scale_small(ex))) {
-    if (scale_small(ex)) { adj = kScaleBits; v *= 0x1p256; q *= 0x1p256; }
-    ex = ex_of();
-  }
-  return ex < kMinExp ? 1022 : ex;
+__device__ __forceinline__ int small_scale2(double (&v)[1], double (&q)[1], int bal, int& adj, int& eq) {
+  return joint_scale<1>(v, q, bal, adj, eq,
+                        [&] { return half_max(max(exp_of_key(mag_key(v[0])), exp_of_key(mag_key(q[0])) + bal)); });
 }
 
 }  // namespace tc
@@ -216,12 +210,11 @@ element_step_small_kernel(ElemTcArgs a) {
     ring.wait(s0, a.l.status);
     ring.wait(s1, a.l.status);
     const int bal = *ring.exps(s1), er = ring.exps(s0)[row];
-    int adj;
-    const int E = small_scale2(v, x, bal, adj);
-    put_digits(M.dig[0], v, E, s, row);
-    double xq[1] = {x};
-    const int Eq = joint_q_exp<1>(xq, E - bal);
-    put_digits(M.dig[1], xq[0], Eq, s, row);
+    int adj, Eq;
+    double vs[1] = {v}, qs[1] = {x};
+    const int E = small_scale2(vs, qs, bal, adj, Eq);
+    put_digits(M.dig[0], vs[0], E, s, row);
+    put_digits(M.dig[1], qs[0], Eq, s, row);
     x = small_product<2, true>(M.dig, M.lev, ring.frags(s0), ring.frags(s1), er, E - 1022 - adj, lane,
                                [&] { ring.template release<2>(lane); });
     if (ok) a.l.q[p] = x;

@@ -326,12 +326,11 @@ element_step_tc_kernel(ElemTcArgs a) {
     ring.wait(s0, a.l.status);
     ring.wait(s1, a.l.status);
     const int bal = *ring.exps(s1);
-    int adj;
-    const int E = column_scale2<kV>(v, x, bal, adj);
+    int adj, Eq;
+    const int E = column_scale2<kV>(v, x, bal, adj, Eq);
     XDigits d[2 * kRT];
 #pragma unroll
     for (int r = 0; r < kRT; ++r) split_rows(v + 4 * r, E, d[r]);
-    const int Eq = joint_q_exp<kV>(x, E - bal);
 #pragma unroll
     for (int r = 0; r < kRT; ++r) split_rows(x + 4 * r, Eq, d[kRT + r]);
     product<kRT, 2, true>(
