@@ -349,18 +349,9 @@ struct DDOps {
   static __device__ __forceinline__ dd fma(dd acc, dd x, dd y) { return dd_fma(acc, x, y); }
   static __device__ __forceinline__ dd div(dd x, dd y) { return dd_div(x, y); }
   static __device__ __forceinline__ dd neg(dd x) { return dd_neg(x); }
-  // Terms of a sum: the high parts by TwoSum, all errors in the low part (the compensated dot product of
-  // Ogita, Rump and Oishi with the low parts' products): 12 operations, against 28 of fma, for an error of
-  // n^2 2^-106 sum |x y|.  norm makes the sum a dd.
-  static __device__ __forceinline__ dd mac(dd acc, dd x, dd y) {
-    const double p = __dmul_rn(x.hi, y.hi);
-    const double e = ::fma(x.lo, y.hi, ::fma(x.hi, y.lo, ::fma(x.hi, y.hi, -p)));
-    const dd s = two_sum(acc.hi, p);
-    return dd{s.hi, acc.lo + (s.lo + e)};
-  }
-  static __device__ __forceinline__ dd norm(dd x) { return fast_two_sum(x.hi, x.lo); }
-  // a - x y
-  static __device__ __forceinline__ dd fms(dd a, dd x, dd y) { return norm(mac(a, neg(x), y)); }
+  // terms of a sum, and a - x y
+  static __device__ __forceinline__ dd mac(dd acc, dd x, dd y) { return dd_mac(acc, x, y); }
+  static __device__ __forceinline__ dd fms(dd a, dd x, dd y) { return dd_mac(a, neg(x), y); }
 };
 struct F64Ops {
   static __device__ __forceinline__ dd make(double a) { return dd{a, 0.0}; }
@@ -372,7 +363,6 @@ struct F64Ops {
   static __device__ __forceinline__ dd div(dd x, dd y) { return dd{x.hi / y.hi, 0.0}; }
   static __device__ __forceinline__ dd neg(dd x) { return dd{-x.hi, 0.0}; }
   static __device__ __forceinline__ dd mac(dd acc, dd x, dd y) { return fma(acc, x, y); }
-  static __device__ __forceinline__ dd norm(dd x) { return x; }
   static __device__ __forceinline__ dd fms(dd a, dd x, dd y) { return dd{::fma(-x.hi, y.hi, a.hi), 0.0}; }
 };
 constexpr int kSetupMats = 15;       // working matrices of the element set-up
@@ -405,7 +395,6 @@ __device__ void coefficient_matrices(const ElemArgs& a, const ElemSmem& sm, int6
       const int64_t idx = (i < a.n) ? e * (int64_t)a.n * nbs + (int64_t)i * nbs + j : a.n_int + a.dofs[e * nbs + j];
       r = Op::mac(r, sm.phi[g * pp + q], ldd(a.rho_hi, a.rho_lo, idx));
     }
-    r = Op::norm(r);
     for (int k = 0; k < nk; ++k) sm.KR[(l * ng + g) * nk + k] = Op::mul(sm.K[(l * ng + g) * nk + k], r);
   }
   __syncthreads();
@@ -437,7 +426,7 @@ __device__ void coefficient_matrices(const ElemArgs& a, const ElemSmem& sm, int6
         }
       }
     }
-    sm.Eline[lab * 4 + k] = Op::norm(s);
+    sm.Eline[lab * 4 + k] = s;
   }
   __syncthreads();
   // assemble the element matrices from the lines (faces)
@@ -535,7 +524,7 @@ __device__ void mm(int nb, const dd* A, const dd* B, dd* C) {
     const int r = t / nb, c = t - r * nb;
     dd s = Op::make(0.0);
     for (int k = 0; k < nb; ++k) s = Op::mac(s, A[r * nb + k], B[k * nb + c]);
-    C[t] = Op::norm(s);
+    C[t] = s;
   }
   __syncthreads();
 }
@@ -756,7 +745,7 @@ __global__ void __launch_bounds__(768) element_setup_kernel(ElemArgs a) {
             for (int k = 0; k < nb; ++k) g = Op::mac(g, G[r * nb + k], E1w[s_cur][cc * nb + k]);
             const int64_t to = (int64_t)r * nbs + cc;
             X[to] = Hp[t].hi;
-            X[2 * nns + to] = -Op::norm(g).hi;
+            X[2 * nns + to] = -g.hi;
           }
           __syncthreads();
         }
@@ -769,8 +758,8 @@ __global__ void __launch_bounds__(768) element_setup_kernel(ElemArgs a) {
             s1 = Op::mac(s1, rk, E1w[s_cur][cc * nb + k]);               // phi_{-1}[k][c] = E1[c][k]
             s2 = Op::mac(s2, rk, E0w[s_cur][k * nb + cc]);               // psi_{-1} = E0 xi / (2h)
           }
-          ph[t] = Op::sub(ph[t], Op::norm(s1));
-          ps[t] = Op::fms(ps[t], Op::norm(s2), Op::mul(xi, inv_2h));
+          ph[t] = Op::sub(ph[t], s1);
+          ps[t] = Op::fms(ps[t], s2, Op::mul(xi, inv_2h));
         }
         __syncthreads();
       } else {
@@ -784,7 +773,7 @@ __global__ void __launch_bounds__(768) element_setup_kernel(ElemArgs a) {
           const int r = t / nb, cc = t - r * nb;
           dd s = Op::make(0.0);
           for (int k = 0; k < nb; ++k) s = Op::mac(s, th[r * nb + k], Hp[k * nb + cc]);
-          ph[t] = Op::sub(ph[t], Op::norm(s));
+          ph[t] = Op::sub(ph[t], s);
         }
         __syncthreads();
       }
@@ -804,9 +793,7 @@ __global__ void __launch_bounds__(768) element_setup_kernel(ElemArgs a) {
             sq = Op::mac(sq, gk, th[k * nb + cc]);
             sh = Op::mac(sh, gk, ps[k * nb + cc]);
           }
-          sp = Op::mul(Op::norm(sp), x2);
-          sq = Op::norm(sq);
-          sh = Op::norm(sh);
+          sp = Op::mul(sp, x2);
           const int64_t to = (int64_t)r * nbs + cc;
           Pi[to] = sp.hi;
           Pi[nns + to] = (i == 0) ? 0.0 : sq.hi;
@@ -824,7 +811,7 @@ __global__ void __launch_bounds__(768) element_setup_kernel(ElemArgs a) {
           dd s = Op::make(0.0);
           for (int k = 0; k < nb; ++k)
             s = Op::mac(s, Op::mul(Op::mul(xi, E0w[s_cur][r * nb + k]), inv_2h), Gm[k * nb + cc]);
-          T1[t] = Op::norm(s);
+          T1[t] = s;
         }
         __syncthreads();
         if (a.xel) {
@@ -842,7 +829,6 @@ __global__ void __launch_bounds__(768) element_setup_kernel(ElemArgs a) {
               yp = Op::mac(yp, gk, Op::add(E0w[s_next][k * nb + cc], Op::mul(a.mass, mk)));
               ym = Op::mac(ym, gk, mk);
             }
-            yt = Op::norm(yt); yp = Op::norm(yp); ym = Op::norm(ym);
             const int64_t to = (int64_t)r * nbs + cc;
             X[nns + to] = T1[t].hi;
             X[3 * nns + to] = yt.hi;
@@ -857,7 +843,7 @@ __global__ void __launch_bounds__(768) element_setup_kernel(ElemArgs a) {
           dd s = E1w[s_cur][cc * nb + r];
           for (int k = 0; k < nb; ++k)
             s = Op::mac(s, Op::mul(Op::mul(xi, E0w[s_cur][r * nb + k]), inv_2h), Hp[k * nb + cc]);
-          Gm[t] = Op::norm(s);
+          Gm[t] = s;
         }
         __syncthreads();
         double* Se = a.S + e * nns;
@@ -871,7 +857,6 @@ __global__ void __launch_bounds__(768) element_setup_kernel(ElemArgs a) {
             rr = Op::mac(rr, wk, th[k * nb + cc]);
             tt = Op::mac(tt, wk, M0w[w_cur][k * nb + cc]);
           }
-          s = Op::norm(s); rr = Op::norm(rr); tt = Op::norm(tt);
           const int64_t to = (int64_t)r * nbs + cc;
           Se[to] = s.hi;
           Re[to] = rr.hi;
