@@ -96,9 +96,19 @@ struct Builder {
 // 1000 polygons, 2 shots 108 | 50; 64 x 64, 1 shot 152 | 101, 8 shots 222 | 184; 128 x 128, 8 shots (mostly
 // products) 624 | 647; 16^3 cube, 8 shots 922 | 872.  With 9 us and 2e-5 us the small meshes keep a level
 // more (24 x 24: 73, 4 x 4: 23); with 16 us the cube merges a pair of levels too many (930).
+// The rule is one for all passes of a mesh, of 1 to 16 shots; an entry costs more of them.  Whole steps, levels apart |
+// grouped, us, at 12 and 16 shots: 24 x 24 order 4 273 | 196, 334 | 245; 32 x 32 order 4 275 | 243, 362 | 307; 64 x 64
+// order 4 1151 | 1131, 1448 | 1407; 96 x 96 order 4 1250 | 1236, 1598 | 1590; 128 x 128 order 1 467 | 394, 537 | 442;
+// 48 x 48 order 8, where the upper levels' staging leaves one block per SM, 1004 | 1013, 1274 | 1303.
+// Precision: the factors of a group are products of its members' and not an elimination with pivots over the group.
+// Over 64 indefinite matrices (order-5 quadtrees, densities of 0.05 to 2 at random), whose elimination without
+// exchanges between fronts amplifies rounding, the traces' errors are 0.90 times those of the binary levels in the
+// geometric mean (0.19 to 6.3 times for one matrix, as two orders of elimination differ; at most 9e-11, binary 4e-10).
 constexpr double kHopUs = 12.0, kEntryUs = 2.4e-5;
 constexpr int kMaxMerged = 5;
-// the staging of a merged front (separator + boundary) fits the solve kernel at four blocks per SM
+// largest merged front (separator + boundary): at 8 shots its block tasks of one row stage about what still runs at
+// four blocks per SM (9 (s + b) + b / 2 doubles backward, 11 s + 10 forward, of the 7152 of kQuarterSm in step.cu).
+// More rows a task or more shots take it beyond: the level then runs in the launch of the large fronts.
 constexpr int kMaxMergedFront = 777;
 
 // the group of every level

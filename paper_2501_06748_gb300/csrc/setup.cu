@@ -529,11 +529,11 @@ __device__ void mm(int nb, const dd* A, const dd* B, dd* C) {
   __syncthreads();
 }
 
-// Bound by the FP64 pipe (2 operations per clock and SM): 77 % of it busy, 21 ms for 4096 elements of
-// 16 boundary nodes and 32 radial points (54 ms before), three quarters of the operations in the
+// Bound by the FP64 pipe (2 operations per clock and SM): 79 % of it busy, 25 ms for 4096 elements of
+// 16 boundary nodes and 32 radial points (54 ms before), two thirds of the operations in the
 // eliminations and products of the binary64 points.  So operations are what is saved: eliminations in
-// place (1 instead of 4 per entry and step), extended sums by compensated dot products (12 instead of
-// 28 a term), the shape functions' products formed once.  The 15 working matrices leave room for three
+// place (1 instead of 4 per entry and step), extended sums by dd_mac (21 instead of 28 a term; 21 ms
+// with its less accurate form of 12), the shape functions' products formed once.  The 15 working matrices leave room for three
 // blocks per SM at 80 registers (with 96, two blocks: 24 ms); one block barrier per elimination step is
 // for warp 0, which finds the next pivot.
 __global__ void __launch_bounds__(768) element_setup_kernel(ElemArgs a) {

@@ -259,8 +259,8 @@ __device__ __forceinline__ void stage_copy(double* dst, const double* src, int n
 // constant part wrote, so the two are separated by a block (or warp) barrier.
 //
 // Forward task (rows r0..r1 of the node's boundary):
-//   [front values: c_sep (s B), then c_bnd of the task's rows (rows B) | the task's rows
-//    of C (rows x s) | sources of those s + rows positions (int4 each)]
+//   [sources of the s + rows positions (int4 each) | front values: c_sep (s B), then c_bnd of
+//    the task's rows (rows B) | the task's rows of C (rows x s)]
 // c = ext + f_hat parts + ybnd parts, in this order for every schedule.
 struct FwdStage {
   double* vals;
@@ -1711,8 +1711,9 @@ int Stepper::init() {
   sa.warp_doubles = (int)solve_warp_doubles(B);
   sa.bdiv = B >= 2 ? (unsigned)((1ULL << 32) / (unsigned long long)B + 1ULL) : 0u;
 
-  // one cooperative persistent launch per time step for the whole tree, unless the
-  // device cannot launch cooperatively or SBFWI_SOLVE=levels asks for one launch per level
+  // one launch per time step for the whole tree, unless the device cannot launch cooperatively (which the barrier
+  // schedule needs; the dataflow does not, and is offered on the same devices) or SBFWI_SOLVE=levels asks for one
+  // launch per level
   SBFWI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solve_persistent_kernel, 256, s_smem));
   // SBFWI_SOLVE=levels: one launch per tree level; =barrier: one launch with grid
   // barriers between levels; default: one dataflow launch

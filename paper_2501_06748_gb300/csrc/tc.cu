@@ -13,11 +13,11 @@
 //    [v ; q 2^a] with a per-point balancing power a (a shared exponent without it
 //    loses ~1e-12 relative near the scaling centre, where |P| << |Q|), H u, R q and
 //    T v are scaled on their own;
-//  * each integer is written in six balanced base-512 digits (|digit| <= 257, exact
-//    in FP16): A_int = sum_k a_k 2^(9(6-k)), x_int = sum_l x_l 2^(9(6-l));
+//  * each integer is written in six balanced base-512 digits (-256..255, the first one up
+//    to 256 = 2^53 / 2^45, exact in FP16): A_int = sum_k a_k 2^(9(6-k)), x_int = sum_l x_l 2^(9(6-l));
 //  * the digit products of one significance level L = k + l are summed by
 //    mma.sync.m16n8k16 (FP16 in, FP32 accumulate), at most four products of 16 terms per
-//    accumulator: every partial sum is an integer of at most 2^22, so the accumulation is exact;
+//    accumulator: every partial sum is an integer of at most 4 x 16 x 256^2 = 2^22, so the accumulation is exact;
 //  * levels L = 2..8 are kept (the dropped ones weigh < 2^-57 of the scale), turned
 //    back into integers, summed in int64 with their weights 2^(9(8-L)), the two lowest
 //    levels rounded once to the nearest unit, and converted once to FP64:

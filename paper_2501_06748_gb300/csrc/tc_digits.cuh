@@ -1,7 +1,7 @@
 // FP16 digit splitting of FP64 operands for the tensor-core element kernels (shared by
 // the one- and two-row-tile kernels): binary64 fields to fixed point, balanced base-512
 // digits, m16n8k16 products per significance level, exact integer recombination, and
-// the cp.async helpers of the operator pipeline.  The method is described in tc.cu.
+// the bulk copies and mbarriers of the operator ring.  The method is described in tc.cu.
 #pragma once
 #include <cstdint>
 #include <cuda_fp16.h>
