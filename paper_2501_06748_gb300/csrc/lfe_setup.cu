@@ -114,6 +114,7 @@ __device__ bool ginv(int n, double* A, double* Inv, double* col, double* red, do
     __syncthreads();
   }
   if (logdet) *logdet = lsum;
+  __syncthreads();                      // every thread has read lsum before the next call resets it
   (void)red;
   return true;
 }
